@@ -318,7 +318,7 @@ int band_kernels_apply(const BandArgs &a, const double *x, double *y, cudaStream
 }  // namespace
 
 void mg_band_free(mg_ctx *ctx) {
-    mg_free(ctx->d_Jeffb); mg_free(ctx->d_Mb); mg_free(ctx->d_bcells); mg_free(ctx->d_bw); mg_free(ctx->d_blu);
+    mg_free(ctx->d_Jeffb); mg_free(ctx->d_Mb); mg_free(ctx->d_Mpart); ctx->band_part_cap = 0; mg_free(ctx->d_bcells); mg_free(ctx->d_bw); mg_free(ctx->d_blu);
     mg_free(ctx->d_bpiv); mg_free(ctx->d_bs); mg_free(ctx->d_bz); mg_free(ctx->d_bx); mg_free(ctx->d_bw2);
     mg_free(ctx->d_bV); mg_free(ctx->d_bpart); mg_free(ctx->d_bh);
     ctx->band_cap_n = 0;

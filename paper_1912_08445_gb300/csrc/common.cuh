@@ -30,6 +30,7 @@ struct LineConst {
     double Bul;     // A c^2 / (2 h nu^3)
     double Blu;     // (g_u/g_l) B_ul
     double pre;     // h nu / (4 pi)
+    double pnorm;   // c / (nu sqrt(pi)), the profile normalisation times the width
     int32_t up, lo;
 };
 
@@ -163,6 +164,8 @@ struct mg_ctx {
     int band_cap_lev = 0, band_cap_L = 0, band_cap_R = 0;
     int64_t band_gmres_iters = 0;
     double *d_Jeffb = nullptr, *d_Mb = nullptr;
+    double *d_Mpart = nullptr;     // coupling terms per chunk of bins, before their sum
+    int64_t band_part_cap = 0;
     int2 *d_bcells = nullptr;
     double *d_bw = nullptr, *d_blu = nullptr, *d_bs = nullptr, *d_bz = nullptr, *d_bx = nullptr, *d_bw2 = nullptr;
     double *d_bV = nullptr, *d_bpart = nullptr, *d_bh = nullptr;

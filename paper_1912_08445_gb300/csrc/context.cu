@@ -355,6 +355,7 @@ extern "C" int mg_set_species(mg_ctx *ctx, int32_t n_lev, const double *E, const
         c.Bul = A[l] * kC * kC / (2.0 * kH * c.nu * c.nu * c.nu);
         c.Blu = g[up[l]] / g[lo[l]] * c.Bul;
         c.pre = kH * c.nu / (4.0 * kPi);
+        c.pnorm = kC / (c.nu * kSqrtPi);
     }
     std::vector<float> lconst(2 * n_lines);
     for (int l = 0; l < n_lines; l++) {

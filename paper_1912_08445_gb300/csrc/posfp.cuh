@@ -1,0 +1,143 @@
+// Arithmetic on non-negative numbers with 64-bit significands on the integer pipe.
+//
+// GB300 issues one warp-wide FP64 instruction per SM sub-partition about every 80 cycles
+// (measured: 0.50 T DFMA/s on 152 SMs), so a double-precision operation costs as much as
+// 80 integer or FP32 instructions. The transfer sweep works on non-negative quantities
+// only: without signs and cancellation a multiplication is one 64-bit high product and a
+// normalisation by at most two bits (about 15 instructions). Significands keep 64
+// bits, 11 more than a double, and results are rounded once when they are packed.
+//
+// - 2^(-t) is table driven (Tang 1989: a table of 2^(-i/256) and a short polynomial), in
+//   fixed point: the error is below 2^-58 of the result, against 2^-53 of a rounded
+//   double.
+// - The reciprocal is Newton's iteration y <- y + y (1 - D y) from a single-precision
+//   reciprocal (24 -> 46 -> 62 bits).
+#pragma once
+#include <cstdint>
+
+namespace mg {
+
+// A number m 2^e >= 0: m has its top bit set, or is 0.
+struct PosFp {
+    uint64_t m;
+    int e;
+};
+
+// From a non-negative double (subnormals count as zero).
+__device__ __forceinline__ PosFp pos_from(double x) {
+    const uint64_t b = (uint64_t)__double_as_longlong(x);
+    const int ex = (int)(b >> 52) & 0x7ff;
+    if (ex == 0) return PosFp{0, 0};
+    return PosFp{((b << 11) | 0x8000000000000000ull), ex - 1086};   // 1086 = 1023 + 63
+}
+
+// m 2^e rounded to a double; m may have up to two leading zero bits. Below the smallest
+// normal double the result is 0, beyond the largest it is infinity.
+__device__ __forceinline__ double pos_pack(uint64_t m, int e) {
+    const int z = (m >> 63) ? 0 : ((m >> 62) & 1 ? 1 : 2);
+    m <<= z;
+    const int E = e - z + 1086;
+    // the rounded significand carries its leading bit (and a carry) into the exponent
+    const uint64_t r = (m >> 11) + ((m >> 10) & 1);
+    uint64_t b = ((uint64_t)(uint32_t)(E - 1) << 52) + r;
+    if (E >= 0x7ff) b = 0x7ff0000000000000ull;
+    if (E < 1 || !(m >> 63)) b = 0;
+    return __longlong_as_double((long long)b);
+}
+__device__ __forceinline__ double pos_pack(const PosFp &a) { return pos_pack(a.m, a.e); }
+
+__device__ __forceinline__ PosFp pos_mul(const PosFp &a, const PosFp &b) {
+    uint64_t h = __umul64hi(a.m, b.m);
+    int e = a.e + b.e + 64;
+    if (!(h >> 63)) {
+        h <<= 1;
+        e--;
+    }
+    return PosFp{h, e};
+}
+
+// 1/a, a > 0.
+__device__ __forceinline__ PosFp pos_rcp(const PosFp &a) {
+    const float d = (float)(uint32_t)(a.m >> 40);            // D 2^24, exact; D = m/2^64 in [1/2, 1)
+    float r;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(d));
+    // y = 1/D in units of 2^-62, in (1, 2]: 1/D = r 2^24, so y 2^62 = r 2^86
+    const uint32_t rb = __float_as_uint(r);
+    uint64_t y = (uint64_t)((rb & 0x7fffffu) | 0x800000u) << ((int)(rb >> 23) - 127 - 23 + 86);
+#pragma unroll
+    for (int it = 0; it < 2; it++) {
+        const int64_t err = (int64_t)((1ull << 62) - __umul64hi(a.m, y));   // (1 - D y) 2^62
+        y += (uint64_t)__mul64hi((int64_t)(y >> 1), err << 3);
+    }
+    // 1/a = (1/D) 2^(-64 - e) = y 2^(-62 - 64 - e)
+    PosFp q{y, -126 - a.e};
+    if (!(q.m >> 63)) {
+        q.m <<= 1;
+        q.e--;
+    }
+    return q;
+}
+
+// ---------------------------------------------------------------- 2^(-t)
+// 2^(-2^-k), k = 1 .. 8, in units of 2^-64.
+constexpr uint64_t kExp2Half[8] = {
+    0xb504f333f9de6484ull,
+    0xd744fccad69d6af4ull,
+    0xeac0c6e7dd24392eull,
+    0xf5257d152486cc2cull,
+    0xfa83b2db722a033aull,
+    0xfd3e0c0cf486c174ull,
+    0xfe9e115c7b8f884bull,
+    0xff4ecb59511ec8a5ull};
+
+struct Exp2Table {
+    uint64_t t[256];   // 2^(-i/256) in units of 2^-63
+};
+constexpr uint64_t mulhi_u64(uint64_t a, uint64_t b) { return (uint64_t)(((unsigned __int128)a * b) >> 64); }
+constexpr Exp2Table make_exp2_table() {
+    Exp2Table T{};
+    T.t[0] = 1ull << 63;
+    for (int i = 1; i < 256; i++) {
+        uint64_t p = 0;
+        for (int k = 0; k < 8; k++)
+            if (i & (128 >> k)) p = p ? mulhi_u64(p, kExp2Half[k]) : kExp2Half[k];
+        T.t[i] = p >> 1;
+    }
+    return T;
+}
+__device__ constexpr Exp2Table kExp2Table = make_exp2_table();
+
+// c_k = ln(2)^k / k!: c1, c2 in units of 2^-64, c3 .. c5 in units of 2^-32
+constexpr uint64_t kExpC1 = 0xb17217f7d1cf79abull;
+constexpr uint64_t kExpC2 = 0x3d7f7bff058b1d50ull;
+constexpr uint32_t kExpC3 = 0x0e35846bu;
+constexpr uint32_t kExpC4 = 0x0276556du;
+constexpr uint32_t kExpC5 = 0x005761ffu;
+
+// Significand (in units of 2^-63, in [2^62, 2^63]) and integer exponent n of
+// 2^(-x^2) = sig 2^(-n), for |x| < 64 (t: the table in shared memory).
+__device__ __forceinline__ uint64_t exp2_neg_sq(double x, const uint64_t *t, int &n) {
+    // U = |x| 2^57
+    const uint64_t b = (uint64_t)__double_as_longlong(x) & 0x7fffffffffffffffull;
+    const int sh = (int)(b >> 52) - 1023 + 5;                 // exponent + 57 - 52
+    const uint64_t mant = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
+    const uint64_t U = sh >= 0 ? mant << sh : (sh > -64 ? mant >> -sh : 0);
+    // U^2 = x^2 2^114: integer part, fraction of 64 bits
+    const uint64_t hi = __umul64hi(U, U), lo = U * U;
+    n = (int)(hi >> 50);
+    const uint64_t f = (hi << 14) | (lo >> 50);
+    const uint64_t T = t[f >> 56];
+    const uint64_t r = f << 8;                                // remainder / 2^-8, in units of 2^-64
+    const uint32_t r32 = (uint32_t)(r >> 32);
+    // 2^(-r') = 1 - r' (c1 - r' (c2 - r' (c3 - r' (c4 - r' c5)))), c_k = ln(2)^k / k!,
+    // r' = r 2^-8; the inner terms need 32 bits only
+    const uint32_t a4 = kExpC4 - (__umulhi(kExpC5, r32) >> 8);
+    const uint32_t a3 = kExpC3 - (__umulhi(a4, r32) >> 8);
+    const uint64_t a2 = kExpC2 - (((uint64_t)a3 * (uint32_t)(r >> 32) + (((uint64_t)a3 * (uint32_t)r) >> 32)) >> 8);
+    const uint64_t a1 = kExpC1 - (__umul64hi(a2, r) >> 8);
+    const uint64_t d = __umul64hi(a1, r) >> 8;                // 1 - 2^(-r'), in units of 2^-64
+    const uint64_t s = T - __umul64hi(T, d);
+    return s < (1ull << 62) ? (1ull << 62) : s;               // (one unit below 1/2 by truncation)
+}
+
+}  // namespace mg

@@ -1,6 +1,7 @@
 // K2 (line data) and K3 (Feautrier formal solve with the diagonal ALO), Sec. 3.3-3.4.
 #include <cmath>
 #include "common.cuh"
+#include "posfp.cuh"
 
 using namespace mg;
 
@@ -400,6 +401,12 @@ __global__ void k_feautrier64(SolveArgs a) {
         }
 }
 
+}  // namespace
+
+#include "feautrier64.cuh"
+
+namespace {
+
 // ---------------------------------------------------------------- images
 // Image along direction n (Sec. 3.5): each origin point o gives the intensity leaving the
 // model along n on its ray pair, carried from the far end of the -n half to the far end
@@ -766,6 +773,71 @@ static int launch_fp64(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount,
     size_t smem = smem_for(1);
     if (smem > 227 * 1024)
         return mg_fail(ctx, MG_ERR_CAPACITY, "FP64 formal solve: longest ray pair does not fit in shared memory");
+    const bool sca = !olist && ctx->sca_on;
+    if (sca) {
+        a.chi_sca = ctx->d_chisca;
+        a.Jsca = ctx->d_Jsca;
+        a.Jnu = ctx->d_Jsca_new;
+    }
+    if (!olist) MG_CUDA(cudaMemsetAsync(ctx->d_err, 0, 4, ctx->stream));
+    const char *name = olist ? "feautrier_fp64_promoted" : "feautrier_fp64";
+    bool overlap = false;
+    for (int l = 0; l < a.L; l++) overlap |= (ctx->h_ovl_off[l + 1] - ctx->h_ovl_off[l]) > 1;
+    if (!overlap) {
+        // no line overlaps another: the warp-autonomous kernel
+        Sweep64 A{};
+        A.nc = (F + 31) / 32;
+        A.nl = std::min(a.L, (31 + a.Q - 1) / a.Q + 1);
+        A.kl = (a.Q + 30) / 32 + 1;
+        A.dmin = a.dtau_min / kSqrt2_64;
+        A.inv_chi_min = 1.0 / a.chi_min;
+        A.skip = ctx->opt.chi_min * ctx->extent < 1e-14;
+        // up to 8 warps per origin (16 when there are few origins, for 4 warps per SM
+        // sub-partition): every chunk of bins, and several groups of ray pairs when the
+        // chunks are few, balanced over the rounds each warp makes
+        const int wmax = (int64_t)grid * 8 < 4 * 4 * 152 ? 16 : 8;
+        int warps;
+        if (A.nc >= wmax) {
+            const int rounds = (A.nc + wmax - 1) / wmax;
+            warps = (A.nc + rounds - 1) / rounds;
+            a.groups = 1;
+        } else {
+            const int gmax = std::min(a.P, wmax / A.nc), rounds = (a.P + gmax - 1) / gmax;
+            a.groups = (a.P + rounds - 1) / rounds;
+            warps = A.nc * a.groups;
+        }
+        auto bytes = [&]() {
+            return 2048 + sizeof(double) * ((sca ? a.Q : 0) + (size_t)a.groups * F * (4 + B)) + 16 +
+                   warps * warp64_bytes(A.nl, B, sca);
+        };
+        while (a.groups > 1 && bytes() > 227 * 1024) warps = A.nc * --a.groups;
+        while (a.groups == 1 && warps > 1 && bytes() > 227 * 1024) warps--;
+        smem = bytes();
+        if (smem <= 227 * 1024) {
+            if (B > 0) {
+                if (ctx->band_part_cap < (int64_t)A.kl * a.n * a.L * a.R * B) {
+                    const int64_t need = (int64_t)A.kl * a.n * a.L * a.R * B;
+                    int rc = mg_alloc(ctx, &ctx->d_Mpart, need);
+                    ctx->band_part_cap = rc ? 0 : need;
+                    if (rc) return rc;
+                }
+                A.Mpart = ctx->d_Mpart;
+            }
+            A.s = a;
+            void (*kern)(Sweep64) = sca ? (B == 0 ? k_feautrier64w<0, true> : (B == 1 ? k_feautrier64w<1, true> : k_feautrier64w<2, true>))
+                                        : (B == 0 ? k_feautrier64w<0, false> : (B == 1 ? k_feautrier64w<1, false> : k_feautrier64w<2, false>));
+            MG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            MgTimed t(ctx, name);
+            kern<<<grid, 32 * warps, smem, ctx->stream>>>(A);
+            if (B > 0) {
+                const int64_t m = a.n * a.L * a.R * B;
+                k_band_terms64<<<(unsigned)((m + 255) / 256), 256, 0, ctx->stream>>>(a.n, a.L, a.R, B, a.Q, 1.0 / a.P,
+                                                                                   A.Mpart, a.line, a.Mb);
+            }
+            MG_CUDA(cudaGetLastError());
+            return MG_OK;
+        }
+    }
     // up to 8 warps per point solve different ray pairs when one warp covers all bins,
     // as many as two CTAs per SM leave room for, balanced over the pairs
     a.groups = 1;
@@ -776,20 +848,13 @@ static int launch_fp64(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount,
         a.groups = (a.P + rounds - 1) / rounds;
     }
     smem = smem_for(a.groups);
-    const bool sca = !olist && ctx->sca_on;
     void (*kern)(SolveArgs) = sca ? (B == 0 ? k_feautrier64<0, true> : (B == 1 ? k_feautrier64<1, true> : k_feautrier64<2, true>))
                                   : (B == 0 ? k_feautrier64<0, false> : (B == 1 ? k_feautrier64<1, false> : k_feautrier64<2, false>));
-    if (sca) {
-        a.chi_sca = ctx->d_chisca;
-        a.Jsca = ctx->d_Jsca;
-        a.Jnu = ctx->d_Jsca_new;
-    }
     MG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
     int threads = a.groups > 1 ? 32 * a.groups : ((F + 31) / 32) * 32;
     if (threads > 256) threads = 256;
-    if (!olist) MG_CUDA(cudaMemsetAsync(ctx->d_err, 0, 4, ctx->stream));
     {
-        MgTimed t(ctx, olist ? "feautrier_fp64_promoted" : "feautrier_fp64");
+        MgTimed t(ctx, name);
         kern<<<grid, threads, smem, ctx->stream>>>(a);
     }
     MG_CUDA(cudaGetLastError());
