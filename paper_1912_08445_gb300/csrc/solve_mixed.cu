@@ -1006,6 +1006,11 @@ const WarpVariant kWarpVariants[] = {
     // below 48 KB
     MG_VARIANT_W(4, 8, 3, false, 3), MG_VARIANT_W(4, 8, 4, false, 3), MG_VARIANT_W(4, 8, 3, true, 3),
     MG_VARIANT_W(4, 8, 4, true, 3),
+    // shapes for few and for odd numbers of bins: up to 16 (two or four lines per warp), 17-24
+    // and 33-48 bins per line
+    MG_VARIANT(2, 1, 8, true), MG_VARIANT(2, 1, 8, false), MG_VARIANT(4, 2, 5, true), MG_VARIANT(4, 2, 5, false),
+    MG_VARIANT(4, 3, 4, true), MG_VARIANT(4, 3, 4, false), MG_VARIANT_W(4, 6, 4, true, 3),
+    MG_VARIANT_W(4, 6, 4, false, 3),
 };
 #undef MG_VARIANT
 #undef MG_VARIANT_W
@@ -1035,7 +1040,10 @@ bool variant_valid(int v, int L, int Q) {
     if (v < 0 || v >= kNumWarpVariants) return false;
     const WarpVariant &w = kWarpVariants[v];
     if (w.G > L) return false;
-    return Q <= w.NB * (32 / w.G) && Q > (w.NB == 1 ? 0 : (w.NB / 2) * (32 / w.G));
+    // the smallest number of bins per lane that holds the line among 1, 2, 4, 8 (and 3, 6
+    // between them)
+    const int less = w.NB == 1 ? 0 : (w.NB == 3 ? 2 : (w.NB == 6 ? 4 : w.NB / 2));
+    return Q <= w.NB * (32 / w.G) && Q > less * (32 / w.G);
 }
 
 }  // namespace
@@ -1113,14 +1121,27 @@ static int launch_mixed(mg_ctx *ctx, int variant) {
     return MG_OK;
 }
 
-// Default launch variant for a model: two lines per warp with two bins per lane when the
-// lines have <= 32 bins, otherwise one line per warp with as many bins per lane as needed.
+// Default launch variant for a model. A warp's time grows with its bins per lane and has a
+// share that does not (staging, windows, pair ends): measured per line group on a disc of 31
+// bins 1.13 ms at 1 line x 1 bin, 1.06 ms at 2 x 2 and 0.83 ms at 4 x 4 per line, and with 63
+// bins 13.8 ms, 10.6 ms and 9.9 ms per line at 1 x 2, 2 x 4 and 4 x 8: proportional to NB +
+// 1.6 per group in all six. The default takes the shape with the smallest ceil(L/G) (NB +
+// 1.6): 4 lines x 4 bins (8 for 33-64 bins) for most numbers of lines, two lines per warp
+// where four would leave half of the last warp idle (5, 6 lines). Among equal shapes the
+// first of the list, the fastest number of blocks per SM.
 static int default_variant(int L, int Q) {
-    const int order[] = {4, 3, 2, 0, 1, 6, 5, 8, 7, 12, 11, 10, 9, 17, 16, 15, 13, 14, 19, 18, 21, 20, 25, 24, 23, 22,
-                         26, 27, 28, 29, 30, 31};
-    for (int v : order)
-        if (variant_valid(v, L, Q)) return v;
-    return -1;
+    const int order[] = {12, 31, 34, 36, 38, 3, 10, 32, 0, 6, 8};
+    int best = -1;
+    float cost = 1e30f;
+    for (int v : order) {
+        if (!variant_valid(v, L, Q)) continue;
+        const float c = (float)((L + kWarpVariants[v].G - 1) / kWarpVariants[v].G) * (kWarpVariants[v].NB + 1.6f);
+        if (c < cost) {
+            cost = c;
+            best = v;
+        }
+    }
+    return best;
 }
 
 int mg_launch_feautrier_mixed(mg_ctx *ctx) {
