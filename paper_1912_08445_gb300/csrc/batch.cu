@@ -236,12 +236,9 @@ extern "C" int mg_batch_destroy(mg_batch *b) {
 extern "C" const char *mg_batch_last_error(const mg_batch *b) { return b ? b->err.c_str() : "null batch"; }
 
 // Line data of every model, then one persistent formal-solve launch for all of them.
-static int enqueue_formal_solve(mg_batch *b) {
-    for (auto *c : b->models) {
-        cudaMemsetAsync(c->d_scal + 4, 0, sizeof(unsigned long long), b->stream);
-        int rc = mg_launch_line_data(c);
-        if (rc) return bfail(b, rc, "batch: line data launch failed");
-    }
+static int enqueue_formal_solve(mg_batch *b, bool update = false) {
+    int rc = mg_launch_line_data_batch(b->models.data(), b->n_models, update, b->stream);
+    if (rc) return bfail(b, rc, "batch: line data launch failed");
     return launch_solve(b);
 }
 
@@ -257,13 +254,16 @@ extern "C" int mg_batch_formal_solve(mg_batch *b) {
 }
 
 // One ALI iteration for all active models: line data, persistent formal solve,
-// statistical equilibrium into pops_new, copy back, gather of the convergence words.
+// statistical equilibrium (in place, all models in one launch where that suits them), gather
+// of the convergence words.
 static int enqueue_iteration(mg_batch *b) {
-    int rc = enqueue_formal_solve(b);
+    int rc = enqueue_formal_solve(b, true);
     if (rc) return rc;
-    for (int m = 0; m < b->n_models; m++) {
+    rc = mg_launch_stateq_batch(b->models.data(), b->n_models, b->d_active, b->stream);
+    if (rc < 0) return bfail(b, rc, "batch: stateq");
+    for (int m = 0; rc == 1 && m < b->n_models; m++) {   // a launch per model
         mg_ctx *c = b->models[m];
-        cudaMemsetAsync(c->d_scal, 0, 3 * sizeof(unsigned long long), b->stream);
+        int rc;
         if ((rc = mg_launch_stateq_into(c, c->d_pops, c->d_pops_new, b->d_active + m))) return bfail(b, rc, "batch: stateq");
         const int64_t mm = c->n * c->n_lev;
         k_copy_if_active<<<(unsigned)std::min<int64_t>(1024, (mm + 255) / 256), 256, 0, b->stream>>>(
@@ -305,6 +305,8 @@ extern "C" int mg_batch_iterate(mg_batch *b, mg_ali_report *reps) {
         B_CUDA(cudaGraphLaunch(b->exec, b->stream));
         B_CUDA(cudaStreamSynchronize(b->stream));
         bool changed = false;
+        std::vector<mg_ctx *> push, step;   // models that keep iterating; those that take an Ng step
+        std::vector<int> step_m;
         for (int m = 0; m < b->n_models; m++) {
             if (!b->h_active[m]) continue;
             mg_ctx *c = b->models[m];
@@ -321,18 +323,30 @@ extern "C" int mg_batch_iterate(mg_batch *b, mg_ali_report *reps) {
                 changed = true;
                 continue;
             }
-            // Ng acceleration of this model, as in mg_iterate (outside the graph: the
-            // history ring rotates and the step's acceptance is read on the host)
             if (c->opt.ng_period > 0) {
-                int rc = mg_launch_push_history(c);
-                if (rc) return bfail(b, rc, "batch: Ng history");
+                push.push_back(c);
                 if (nh[m] < 4) nh[m]++;
                 if (nh[m] == 4 && (it + 1) % c->opt.ng_period == 0) {
-                    int acc = 0;
-                    if ((rc = mg_launch_ng(c, &acc))) return bfail(b, rc, "batch: Ng step");
-                    r[m].ng_steps += acc;
+                    step.push_back(c);
+                    step_m.push_back(m);
                     nh[m] = 0;
                 }
+            }
+        }
+        // Ng acceleration, as in mg_iterate (outside the graph: the history rings rotate and
+        // a step's acceptance is read on the host), all models in one launch per kernel
+        if (!push.empty() && mg_launch_push_history_batch(push.data(), (int)push.size(), b->stream))
+            return bfail(b, MG_ERR_CUDA, "batch: Ng history");
+        if (!step.empty()) {
+            if (mg_launch_ng_batch(step.data(), (int)step.size(), b->stream)) return bfail(b, MG_ERR_CUDA, "batch: Ng step");
+            for (size_t i = 0; i < step.size(); i++)
+                B_CUDA(cudaMemcpyAsync(b->h_scal_all + i, step[i]->d_scal + 3, 8, cudaMemcpyDeviceToHost, b->stream));
+            B_CUDA(cudaStreamSynchronize(b->stream));
+            for (size_t i = 0; i < step.size(); i++) {
+                if (b->h_scal_all[i]) continue;
+                r[step_m[i]].ng_steps++;
+                B_CUDA(cudaMemcpyAsync(step[i]->d_pops, step[i]->d_ng_tmp, 8 * step[i]->n * step[i]->n_lev,
+                                       cudaMemcpyDeviceToDevice, b->stream));
             }
         }
         if (changed)

@@ -17,6 +17,10 @@ constexpr double kPi = 3.14159265358979323846;
 
 constexpr int kMaxLev = 64;
 
+// Dynamic shared memory a kernel may use: set once per kernel to the same value whatever the
+// launch needs, so that threads that launch it with other sizes do not change each other's.
+constexpr int kMaxDynSmem = 227 * 1024;
+
 // Scales of the FP32 formal solve: intensities in units of kI0 (W m^-2 Hz^-1 sr^-1);
 // float line data hold chi_int * kChiScale and eta_int * kEtaScale = chi scale / kI0.
 constexpr float kI0 = 1e-20f;
@@ -86,6 +90,7 @@ struct mg_ctx {
     double mass = 0.0;
     std::vector<double> h_E, h_g, h_Tgrid, h_Kdown;
     std::vector<mg::LineConst> h_lines;
+    bool dup_lines = false;        // two lines share a pair of levels
     mg::LineConst *d_lines = nullptr;
     float *d_lconst = nullptr;    // [2L]: c/(nu_l sqrt(pi))/kChiScale, nu_l in GHz (FP32 solve)
     double *d_E = nullptr, *d_g = nullptr, *d_Tgrid = nullptr, *d_Kdown = nullptr;
@@ -241,6 +246,10 @@ int mg_launch_stateq(mg_ctx *ctx);
 int mg_launch_ng(mg_ctx *ctx, int *accepted);
 int mg_launch_push_history(mg_ctx *ctx);
 int mg_launch_stateq_into(mg_ctx *ctx, const double *pops_old, double *pops_new, const int32_t *active);
+int mg_launch_stateq_batch(mg_ctx *const *models, int count, const int32_t *active, cudaStream_t stream);
+int mg_launch_push_history_batch(mg_ctx *const *models, int count, cudaStream_t stream);
+int mg_launch_ng_batch(mg_ctx *const *models, int count, cudaStream_t stream);
+int mg_launch_line_data_batch(mg_ctx *const *models, int count, bool reset_update, cudaStream_t stream);
 int mg_ensure_solve_state(mg_ctx *ctx);   // state buffers, overlaps and collision rates ready
 void mg_noalloc_prepare(mg_ctx *ctx);     // set-up of mg_update_populations_noalloc
 int mg_band_alloc(mg_ctx *ctx);

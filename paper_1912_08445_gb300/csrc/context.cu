@@ -357,6 +357,10 @@ extern "C" int mg_set_species(mg_ctx *ctx, int32_t n_lev, const double *E, const
         c.pre = kH * c.nu / (4.0 * kPi);
         c.pnorm = kC / (c.nu * kSqrtPi);
     }
+    ctx->dup_lines = false;
+    for (int l = 0; l < n_lines; l++)
+        for (int k = 0; k < l; k++)
+            ctx->dup_lines |= up[k] == up[l] && lo[k] == lo[l];
     std::vector<float> lconst(2 * n_lines);
     for (int l = 0; l < n_lines; l++) {
         lconst[l] = (float)(kC / (ctx->h_lines[l].nu * kSqrtPi) / kChiScale);

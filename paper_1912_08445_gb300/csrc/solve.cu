@@ -826,7 +826,7 @@ static int launch_fp64(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount,
             A.s = a;
             void (*kern)(Sweep64) = sca ? (B == 0 ? k_feautrier64w<0, true> : (B == 1 ? k_feautrier64w<1, true> : k_feautrier64w<2, true>))
                                         : (B == 0 ? k_feautrier64w<0, false> : (B == 1 ? k_feautrier64w<1, false> : k_feautrier64w<2, false>));
-            MG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+            MG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem));
             MgTimed t(ctx, name);
             kern<<<grid, 32 * warps, smem, ctx->stream>>>(A);
             if (B > 0) {

@@ -19,6 +19,7 @@
 // kernel:
 //   dtau = max((chi_prev + chi) ds/2, dtau_min),  t = (dtau_prev + dtau)/2,
 //   Phi = t + Phi iota,  iota = 1/(1 + dtau Phi),  psi = (t S + psi) iota.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <type_traits>
@@ -44,25 +45,51 @@ __device__ __forceinline__ float rcpf(float x) {
     return y;
 }
 
-__global__ void k_line_data_f32(int64_t n, int L, int nlev, const double *__restrict__ pops,
-                                const LineConst *__restrict__ lc, double *__restrict__ line,
-                                float *__restrict__ linef, unsigned long long *neg) {
+// Line data of one or several models (blockIdx.y), arguments by value.
+struct LineArgs {
+    int64_t n;
+    int L, nlev;
+    const double *pops;
+    const LineConst *lc;
+    double *line;
+    float *linef;
+    unsigned long long *scal;   // [4]: negative line opacities
+};
+constexpr int kLineBatch = 48;
+struct LineBatch {
+    LineArgs m[kLineBatch];
+};
+static_assert(sizeof(LineBatch) <= 4096, "kernel parameter size");
+
+__global__ void k_line_data_f32(const __grid_constant__ LineBatch b) {
+    const LineArgs &a = b.m[blockIdx.y];
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n * L) return;
-    const int64_t c = t / L;
-    const int l = (int)(t - c * L);
-    const LineConst k = lc[l];
-    const double nu_ = pops[c * nlev + k.up], nl_ = pops[c * nlev + k.lo];
+    if (t >= a.n * a.L) return;
+    const int64_t c = t / a.L;
+    const int l = (int)(t - c * a.L);
+    const LineConst k = a.lc[l];
+    const double nu_ = a.pops[c * a.nlev + k.up], nl_ = a.pops[c * a.nlev + k.lo];
     const double eta = k.pre * nu_ * k.A;
     const double chi = k.pre * (nl_ * k.Blu - nu_ * k.Bul);
-    line[2 * t] = eta;
-    line[2 * t + 1] = chi;
-    if (chi < 0.0) atomicAdd(neg, 1ull);
+    a.line[2 * t] = eta;
+    a.line[2 * t + 1] = chi;
+    if (chi < 0.0) atomicAdd(a.scal + 4, 1ull);
     // (eta, chi) times the profile normalisation c / (nu_l sqrt(pi)): the line opacity of a
     // bin is then chi' 2^(-x'^2) / b, and S = eta'/chi' keeps the scale kEtaScale/kChiScale
     const double kl = kC / (k.nu * kSqrtPi);
-    linef[2 * t] = (float)(eta * (kEtaScale / kChiScale) * kl);
-    linef[2 * t + 1] = (float)(chi * kl);
+    a.linef[2 * t] = (float)(eta * (kEtaScale / kChiScale) * kl);
+    a.linef[2 * t + 1] = (float)(chi * kl);
+}
+
+// Clears the words that a batch's line data ([4]) and population update ([0..2]) count in.
+struct ScalBatch {
+    unsigned long long *scal[256];
+};
+__global__ void k_clear_words(const __grid_constant__ ScalBatch b, int count, int update) {
+    const int m = threadIdx.x;
+    if (m >= count) return;
+    b.scal[m][4] = 0;
+    if (update) b.scal[m][0] = b.scal[m][1] = b.scal[m][2] = 0;
 }
 
 struct MixArgs {
@@ -1048,14 +1075,41 @@ bool variant_valid(int v, int L, int Q) {
 
 }  // namespace
 
+static LineArgs line_args(const mg_ctx *c) {
+    return LineArgs{c->n, c->n_lines, c->n_lev, c->d_pops, c->d_lines, c->d_line, c->d_linef, c->d_scal};
+}
+
 int mg_launch_line_data_mixed(mg_ctx *ctx) {
     const int64_t m = ctx->n * ctx->n_lines;
     MgTimed t(ctx, "line_data");
-    k_line_data_f32<<<(unsigned)((m + 255) / 256), 256, 0, ctx->stream>>>(ctx->n, ctx->n_lines, ctx->n_lev,
-                                                                          ctx->d_pops, ctx->d_lines, ctx->d_line,
-                                                                          ctx->d_linef, ctx->d_scal + 4);
+    LineBatch b{};
+    b.m[0] = line_args(ctx);
+    k_line_data_f32<<<(unsigned)((m + 255) / 256), 256, 0, ctx->stream>>>(b);
     MG_CUDA(cudaGetLastError());
     return MG_OK;
+}
+
+// Line data of every model of a batch: one launch per 48 models (a launch each left 5 us of
+// mostly empty GPU per model and iteration). The counters are cleared first, those of the
+// population update too when one follows.
+int mg_launch_line_data_batch(mg_ctx *const *models, int count, bool reset_update, cudaStream_t stream) {
+    for (int i0 = 0; i0 < count; i0 += 256) {
+        ScalBatch b{};
+        const int k = std::min(256, count - i0);
+        for (int i = 0; i < k; i++) b.scal[i] = models[i0 + i]->d_scal;
+        k_clear_words<<<1, 256, 0, stream>>>(b, k, reset_update ? 1 : 0);
+    }
+    for (int i0 = 0; i0 < count; i0 += kLineBatch) {
+        LineBatch b{};
+        const int k = std::min(kLineBatch, count - i0);
+        int64_t mmax = 0;
+        for (int i = 0; i < k; i++) {
+            b.m[i] = line_args(models[i0 + i]);
+            mmax = std::max(mmax, b.m[i].n * b.m[i].L);
+        }
+        k_line_data_f32<<<dim3((unsigned)((mmax + 255) / 256), k), 256, 0, stream>>>(b);
+    }
+    return cudaGetLastError() == cudaSuccess ? MG_OK : MG_ERR_CUDA;
 }
 
 
