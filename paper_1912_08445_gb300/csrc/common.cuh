@@ -181,6 +181,8 @@ struct mg_ctx {
     bool sca_on = false;
     double *d_chisca = nullptr, *d_Jsca = nullptr, *d_Jsca_new = nullptr;
     unsigned long long *d_scaw = nullptr;
+    double *d_part64 = nullptr;    // FP64 solve: sums of the CTAs that share an origin (grow-only)
+    int64_t part64_cap = 0;
     double sca_tol = 1e-8, sca_change = 0.0;
     int32_t sca_max_iter = 100, sca_iters = 0;
 

@@ -111,7 +111,7 @@ static void drop_state(mg_ctx *ctx) {
     mg_band_free(ctx);
     ctx->band_solved = 0;
     // scattering buffers are sized by the point, line and bin counts: set them again
-    mg_free(ctx->d_chisca); mg_free(ctx->d_Jsca); mg_free(ctx->d_Jsca_new); mg_free(ctx->d_scaw);
+    mg_free(ctx->d_chisca); mg_free(ctx->d_Jsca); mg_free(ctx->d_part64); ctx->part64_cap = 0; mg_free(ctx->d_Jsca_new); mg_free(ctx->d_scaw);
     ctx->sca_on = false;
 }
 
@@ -133,7 +133,7 @@ extern "C" int mg_destroy(mg_ctx *ctx) {
     mg_free(ctx->d_err);
     mg_free(ctx->d_uch); mg_free(ctx->d_img); mg_free(ctx->d_imgxy); mg_free(ctx->d_imgov); mg_free(ctx->d_imglf);
     mg_band_free(ctx);
-    mg_free(ctx->d_chisca); mg_free(ctx->d_Jsca); mg_free(ctx->d_Jsca_new); mg_free(ctx->d_scaw);
+    mg_free(ctx->d_chisca); mg_free(ctx->d_Jsca); mg_free(ctx->d_part64); mg_free(ctx->d_Jsca_new); mg_free(ctx->d_scaw);
     if (ctx->h_scal) cudaFreeHost(ctx->h_scal);
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);
     if (ctx->ev1) cudaEventDestroy(ctx->ev1);

@@ -17,17 +17,24 @@
 
 namespace mg {
 
+// High 64 bits of a product, short of it by at most two units (the low halves' product is
+// left out: three 32-bit multiplications instead of four and no carries).
+__device__ __forceinline__ uint64_t mulhi_near(uint64_t a, uint64_t b) {
+    const uint32_t ah = (uint32_t)(a >> 32), al = (uint32_t)a, bh = (uint32_t)(b >> 32), bl = (uint32_t)b;
+    return (uint64_t)ah * bh + __umulhi(ah, bl) + __umulhi(al, bh);
+}
+
 // A number m 2^e >= 0: m has its top bit set, or is 0.
 struct PosFp {
     uint64_t m;
     int e;
 };
 
-// From a non-negative double (subnormals count as zero).
+// From a non-negative double (subnormals count as zero, whose exponent is below every other).
 __device__ __forceinline__ PosFp pos_from(double x) {
     const uint64_t b = (uint64_t)__double_as_longlong(x);
     const int ex = (int)(b >> 52) & 0x7ff;
-    if (ex == 0) return PosFp{0, 0};
+    if (ex == 0) return PosFp{0, -(1 << 20)};
     return PosFp{((b << 11) | 0x8000000000000000ull), ex - 1086};   // 1086 = 1023 + 63
 }
 
@@ -47,13 +54,30 @@ __device__ __forceinline__ double pos_pack(uint64_t m, int e) {
 __device__ __forceinline__ double pos_pack(const PosFp &a) { return pos_pack(a.m, a.e); }
 
 __device__ __forceinline__ PosFp pos_mul(const PosFp &a, const PosFp &b) {
-    uint64_t h = __umul64hi(a.m, b.m);
+    uint64_t h = mulhi_near(a.m, b.m);
     int e = a.e + b.e + 64;
     if (!(h >> 63)) {
         h <<= 1;
         e--;
     }
     return PosFp{h, e};
+}
+
+// a + b. Both normalised; a zero has m = 0 and an exponent below every other.
+__device__ __forceinline__ PosFp pos_add(const PosFp &a, const PosFp &b) {
+    const bool sw = a.e < b.e;
+    const uint64_t hm = sw ? b.m : a.m, lm = sw ? a.m : b.m;
+    const int he = sw ? b.e : a.e, d = sw ? b.e - a.e : a.e - b.e;
+    uint64_t m = hm + (d < 64 ? lm >> d : 0);
+    const bool carry = m < hm;
+    m = carry ? (m >> 1) | 0x8000000000000000ull : m;
+    return PosFp{m, he + (carry ? 1 : 0)};
+}
+
+// Normalised from a significand with up to two leading zero bits.
+__device__ __forceinline__ PosFp pos_norm(uint64_t m, int e) {
+    const int z = (m >> 63) ? 0 : ((m >> 62) & 1 ? 1 : 2);
+    return PosFp{m << z, e - z};
 }
 
 // 1/a, a > 0.
@@ -66,7 +90,7 @@ __device__ __forceinline__ PosFp pos_rcp(const PosFp &a) {
     uint64_t y = (uint64_t)((rb & 0x7fffffu) | 0x800000u) << ((int)(rb >> 23) - 127 - 23 + 86);
 #pragma unroll
     for (int it = 0; it < 2; it++) {
-        const int64_t err = (int64_t)((1ull << 62) - __umul64hi(a.m, y));   // (1 - D y) 2^62
+        const int64_t err = (int64_t)((1ull << 62) - mulhi_near(a.m, y));   // (1 - D y) 2^62
         y += (uint64_t)__mul64hi((int64_t)(y >> 1), err << 3);
     }
     // 1/a = (1/D) 2^(-64 - e) = y 2^(-62 - 64 - e)
@@ -114,18 +138,25 @@ constexpr uint32_t kExpC3 = 0x0e35846bu;
 constexpr uint32_t kExpC4 = 0x0276556du;
 constexpr uint32_t kExpC5 = 0x005761ffu;
 
+// sqrt(log2 e) in units of 2^-63
+constexpr uint64_t kSqrtLog2eFix = 0x99be610c1d827eefull;
+
 // Significand (in units of 2^-63, in [2^62, 2^63]) and integer exponent n of
-// 2^(-x^2) = sig 2^(-n), for |x| < 64 (t: the table in shared memory).
-__device__ __forceinline__ uint64_t exp2_neg_sq(double x, const uint64_t *t, int &n) {
-    // U = |x| 2^57
+// exp(-x^2) = sig 2^(-n), for |x| < 53 (t: the table in shared memory). The factor
+// sqrt(log2 e) is applied in fixed point: folded into a double-precision x it would carry a
+// rounding that is the same at every point.
+__device__ __forceinline__ uint64_t exp_neg_sq(double x, const uint64_t *t, int &n) {
+    // U = sqrt(log2 e) |x| 2^57
     const uint64_t b = (uint64_t)__double_as_longlong(x) & 0x7fffffffffffffffull;
     const int sh = (int)(b >> 52) - 1023 + 5;                 // exponent + 57 - 52
     const uint64_t mant = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
-    const uint64_t U = sh >= 0 ? mant << sh : (sh > -64 ? mant >> -sh : 0);
-    // U^2 = x^2 2^114: integer part, fraction of 64 bits
-    const uint64_t hi = __umul64hi(U, U), lo = U * U;
+    const uint64_t U = mulhi_near(sh >= 0 ? mant << sh : (sh > -64 ? mant >> -sh : 0), kSqrtLog2eFix) << 1;
+    // U^2 = log2(e) x^2 2^114: integer part, fraction of 64 bits
+    const uint32_t ua = (uint32_t)(U >> 32), ub = (uint32_t)U;
+    const uint64_t mid = 2 * ((uint64_t)ua * ub) + __umulhi(ub, ub);   // (below 2^64: U < 2^63)
+    const uint64_t hi = (uint64_t)ua * ua + (mid >> 32);
     n = (int)(hi >> 50);
-    const uint64_t f = (hi << 14) | (lo >> 50);
+    const uint64_t f = (hi << 14) | ((uint32_t)mid >> 18);
     const uint64_t T = t[f >> 56];
     const uint64_t r = f << 8;                                // remainder / 2^-8, in units of 2^-64
     const uint32_t r32 = (uint32_t)(r >> 32);
@@ -134,9 +165,9 @@ __device__ __forceinline__ uint64_t exp2_neg_sq(double x, const uint64_t *t, int
     const uint32_t a4 = kExpC4 - (__umulhi(kExpC5, r32) >> 8);
     const uint32_t a3 = kExpC3 - (__umulhi(a4, r32) >> 8);
     const uint64_t a2 = kExpC2 - (((uint64_t)a3 * (uint32_t)(r >> 32) + (((uint64_t)a3 * (uint32_t)r) >> 32)) >> 8);
-    const uint64_t a1 = kExpC1 - (__umul64hi(a2, r) >> 8);
-    const uint64_t d = __umul64hi(a1, r) >> 8;                // 1 - 2^(-r'), in units of 2^-64
-    const uint64_t s = T - __umul64hi(T, d);
+    const uint64_t a1 = kExpC1 - (mulhi_near(a2, r) >> 8);
+    const uint64_t d = mulhi_near(a1, r) >> 8;                // 1 - 2^(-r'), in units of 2^-64
+    const uint64_t s = T - mulhi_near(T, d);
     return s < (1ull << 62) ? (1ull << 62) : s;               // (one unit below 1/2 by truncation)
 }
 

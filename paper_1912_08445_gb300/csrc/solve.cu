@@ -789,29 +789,47 @@ static int launch_fp64(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount,
         A.nc = (F + 31) / 32;
         A.nl = std::min(a.L, (31 + a.Q - 1) / a.Q + 1);
         A.kl = (a.Q + 30) / 32 + 1;
-        A.dmin = a.dtau_min / kSqrt2_64;
+        A.dmin = a.dtau_min;
         A.inv_chi_min = 1.0 / a.chi_min;
+        auto host_pos = [](double x) {   // (a normal double)
+            int e;
+            const uint64_t m = (uint64_t)std::ldexp(std::frexp(x, &e), 53) << 11;
+            return PosFp{m, e - 64};
+        };
+        A.cmin = host_pos(a.chi_min);
+        A.half_dmin = host_pos(0.5 * a.dtau_min);
         A.skip = ctx->opt.chi_min * ctx->extent < 1e-14;
-        // up to 8 warps per origin (16 when there are few origins, for 4 warps per SM
-        // sub-partition): every chunk of bins, and several groups of ray pairs when the
-        // chunks are few, balanced over the rounds each warp makes
-        const int wmax = (int64_t)grid * 8 < 4 * 4 * 152 ? 16 : 8;
-        int warps;
-        if (A.nc >= wmax) {
-            const int rounds = (A.nc + wmax - 1) / wmax;
-            warps = (A.nc + rounds - 1) / rounds;
+        // A unit is a warp with a chunk of bins and a share of the ray pairs. A CTA has up to
+        // 8 units: every chunk, and several groups of pairs when the chunks are few, balanced
+        // over the rounds each unit makes. Fewer origins than four waves of two CTAs per SM
+        // share their pairs among several CTAs, so that no SM waits for a last one; and
+        // where even a unit per pair would leave an SM sub-partition 2 warps, the two halves
+        // of a pair go to two warps (the sweep of a half is one dependent chain). 200 shells, 6
+        // pairs, one CTA per origin: 453 us; two warps per pair: 358 us; six CTAs of two
+        // warps per origin: 349 us.
+        const int umax = 8;
+        A.split = olist ? 1 : (int)std::min<int64_t>(a.P, (4 * 2 * 152 + grid - 1) / grid);
+        const int pairs = (a.P + A.split - 1) / A.split;
+        int units;
+        if (A.nc >= umax) {
+            const int rounds = (A.nc + umax - 1) / umax;
+            units = (A.nc + rounds - 1) / rounds;
             a.groups = 1;
         } else {
-            const int gmax = std::min(a.P, wmax / A.nc), rounds = (a.P + gmax - 1) / gmax;
-            a.groups = (a.P + rounds - 1) / rounds;
-            warps = A.nc * a.groups;
+            const int gmax = std::min(pairs, umax / A.nc), rounds = (pairs + gmax - 1) / gmax;
+            a.groups = (pairs + rounds - 1) / rounds;
+            units = A.nc * a.groups;
         }
+        A.duo = !olist && (int64_t)grid * A.split * units <= 8 * 152;
         auto bytes = [&]() {
+            const size_t warps = (size_t)units << A.duo;
             return 2048 + sizeof(double) * ((sca ? a.Q : 0) + (size_t)a.groups * F * (4 + B)) + 16 +
-                   warps * warp64_bytes(A.nl, B, sca);
+                   warps * warp64_bytes(A.nl, B, sca) + (A.duo ? sizeof(double) * 32 * units * (B ? 12 : 4) : 0);
         };
-        while (a.groups > 1 && bytes() > 227 * 1024) warps = A.nc * --a.groups;
-        while (a.groups == 1 && warps > 1 && bytes() > 227 * 1024) warps--;
+        if (bytes() > 227 * 1024) A.duo = 0;
+        while (a.groups > 1 && bytes() > 227 * 1024) units = A.nc * --a.groups;
+        while (a.groups == 1 && units > 1 && bytes() > 227 * 1024) units--;
+        const int warps = units << A.duo;
         smem = bytes();
         if (smem <= 227 * 1024) {
             if (B > 0) {
@@ -823,12 +841,25 @@ static int launch_fp64(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount,
                 }
                 A.Mpart = ctx->d_Mpart;
             }
+            if (A.split > 1) {
+                const int64_t need = a.n * A.split * F * (4 + B);
+                if (ctx->part64_cap < need) {
+                    int rc = mg_alloc(ctx, &ctx->d_part64, need);
+                    ctx->part64_cap = rc ? 0 : need;
+                    if (rc) return rc;
+                }
+                A.part = ctx->d_part64;
+            }
             A.s = a;
             void (*kern)(Sweep64) = sca ? (B == 0 ? k_feautrier64w<0, true> : (B == 1 ? k_feautrier64w<1, true> : k_feautrier64w<2, true>))
                                         : (B == 0 ? k_feautrier64w<0, false> : (B == 1 ? k_feautrier64w<1, false> : k_feautrier64w<2, false>));
             MG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem));
             MgTimed t(ctx, name);
-            kern<<<grid, 32 * warps, smem, ctx->stream>>>(A);
+            kern<<<grid * A.split, 32 * warps, smem, ctx->stream>>>(A);
+            if (A.split > 1) {
+                void (*sums)(SolveArgs, int, const double *) = B == 0 ? k_sums64<4> : (B == 1 ? k_sums64<5> : k_sums64<6>);
+                sums<<<(unsigned)((a.n * a.L + 3) / 4), 128, 0, ctx->stream>>>(a, A.split, A.part);
+            }
             if (B > 0) {
                 const int64_t m = a.n * a.L * a.R * B;
                 k_band_terms64<<<(unsigned)((m + 255) / 256), 256, 0, ctx->stream>>>(a.n, a.L, a.R, B, a.Q, 1.0 / a.P,
