@@ -236,7 +236,7 @@ int mg_launch_line_data(mg_ctx *ctx);
 int mg_launch_line_data_mixed(mg_ctx *ctx);
 int mg_launch_line_data64(mg_ctx *ctx, float *linef, unsigned long long *neg);
 int mg_launch_image(mg_ctx *ctx, int ray, int line, int n_ch, const double *d_u, const mg::Overlap *d_ov,
-                    int n_ov, double *d_I, double *d_xy);
+                    const mg::Overlap *h_ov, int n_ov, double *d_I, double *d_xy);
 int mg_launch_feautrier(mg_ctx *ctx);
 int mg_launch_max_rel_change(mg_ctx *ctx, int64_t m, const double *a_new, const double *a_old,
                              unsigned long long *word);

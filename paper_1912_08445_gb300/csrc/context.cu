@@ -896,7 +896,7 @@ static int image_common(mg_ctx *ctx, int32_t ray, int32_t line, int32_t n_ch, co
     double *d_I = dev ? I : ctx->d_img;
     double *d_xy = dev ? xy : ctx->d_imgxy;
     if (!d_xy) d_xy = ctx->d_imgxy;
-    if ((rc = mg_launch_image(ctx, ray, line, n_ch, ctx->d_uch, ctx->d_imgov, (int)ov.size(), d_I, d_xy))) return rc;
+    if ((rc = mg_launch_image(ctx, ray, line, n_ch, ctx->d_uch, ctx->d_imgov, ov.data(), (int)ov.size(), d_I, d_xy))) return rc;
     if (!dev) {
         MG_CUDA(cudaMemcpyAsync(I, d_I, 8 * (size_t)need, cudaMemcpyDeviceToHost, ctx->stream));
         if (xy) MG_CUDA(cudaMemcpyAsync(xy, d_xy, 16 * (size_t)ctx->n, cudaMemcpyDeviceToHost, ctx->stream));

@@ -296,14 +296,15 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
         const int i = own.x, x = own.y - (c0 + lane);
         bool far = false;
         double hin = 0.0, gz = 0.0, gy = 0.0, ibk = 0.0, w = 0.0;
-        float xerr = 0.0f;
+        float xerr = 0.0f, shrink = 1.0f;
         int eb = 0;
         if (lane < cnt) {
             const int j = x - own.z + 1;
             w = j == own.w ? 1.0 : (double)j * W.rn[i];
             const double w0 = 1.0 - w;
             const double v = w0 * W.v[i + 1] + w * W.v[i];
-            ibk = pos_pack(pos_rcp(pos_from(w0 * W.b[i + 1] + w * W.b[i])));
+            const double bp = w0 * W.b[i + 1] + w * W.b[i];
+            ibk = pos_pack(pos_rcp(pos_from(bp)));
             hin = j < own.w ? W.ds[i] : (i > 0 ? W.ds[i - 1] : hc);
             gy = v * ibk;
             gz = ibk - gy * (1.0 / kC);
@@ -315,7 +316,10 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
                 const float ylo = aq_lo * gzf, yhi = aq_hi * gzf;
                 xerr = 1e-6f * (fabsf(ylo) + fabsf(yhi) + fabsf(gyf));
                 const float xlo = ylo - gyf, xhi = yhi - gyf;
-                const float xm = fmaxf((xlo > 0.0f ? xlo : (xhi < 0.0f ? -xhi : 0.0f)) - xerr, 0.0f);
+                // (with the larger width of the element's ends, so that the next point, up to the
+                // inner cell itself, is at the floor too: its opacity is in the line's bound)
+                shrink = 0.999999f * (float)bp / fmaxf((float)W.b[i], (float)W.b[i + 1]);
+                const float xm = fmaxf((xlo > 0.0f ? xlo : (xhi < 0.0f ? -xhi : 0.0f)) - xerr, 0.0f) * shrink;
                 far = 0.999f * kLog2e64 * xm * xm > bound;
                 if (B > 0) far = far && x >= 3;
                 if constexpr (SCAT) far = far && a.chi_sca[W.cell[i]] == 0.0 && a.chi_sca[W.cell[i + 1]] == 0.0;
@@ -339,7 +343,7 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
             W.h[j] = hin;
             for (int k = 0; k < nl; k++) {
                 W.tt[32 * k + j] = make_float4(
-                    (float)gz, -(float)gy, A.skip ? sqrtf(1.001f / kLog2e64 * fmaxf(line_bound64(W, k, i, eb, chi_min_e), 0.0f)) + xerr : INFINITY,
+                    (float)gz, -(float)gy, A.skip ? sqrtf(1.001f / kLog2e64 * fmaxf(line_bound64(W, k, i, eb, chi_min_e), 0.0f)) / shrink + xerr : INFINITY,
                     0.0f);
                 const double2 p0 = W.ln[32 * k + i + 1], p1 = W.ln[32 * k + i];
                 const double et = (1.0 - w) * p0.x + w * p1.x, ch = (1.0 - w) * p0.y + w * p1.y;

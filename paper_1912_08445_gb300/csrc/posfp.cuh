@@ -138,25 +138,11 @@ constexpr uint32_t kExpC3 = 0x0e35846bu;
 constexpr uint32_t kExpC4 = 0x0276556du;
 constexpr uint32_t kExpC5 = 0x005761ffu;
 
-// sqrt(log2 e) in units of 2^-63
-constexpr uint64_t kSqrtLog2eFix = 0x99be610c1d827eefull;
+// sqrt(log2 e) and log2 e in units of 2^-63
+constexpr uint64_t kSqrtLog2eFix = 0x99be610c1d827eefull, kLog2eFix = 0xb8aa3b295c17f0bbull;
 
-// Significand (in units of 2^-63, in [2^62, 2^63]) and integer exponent n of
-// exp(-x^2) = sig 2^(-n), for |x| < 53 (t: the table in shared memory). The factor
-// sqrt(log2 e) is applied in fixed point: folded into a double-precision x it would carry a
-// rounding that is the same at every point.
-__device__ __forceinline__ uint64_t exp_neg_sq(double x, const uint64_t *t, int &n) {
-    // U = sqrt(log2 e) |x| 2^57
-    const uint64_t b = (uint64_t)__double_as_longlong(x) & 0x7fffffffffffffffull;
-    const int sh = (int)(b >> 52) - 1023 + 5;                 // exponent + 57 - 52
-    const uint64_t mant = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
-    const uint64_t U = mulhi_near(sh >= 0 ? mant << sh : (sh > -64 ? mant >> -sh : 0), kSqrtLog2eFix) << 1;
-    // U^2 = log2(e) x^2 2^114: integer part, fraction of 64 bits
-    const uint32_t ua = (uint32_t)(U >> 32), ub = (uint32_t)U;
-    const uint64_t mid = 2 * ((uint64_t)ua * ub) + __umulhi(ub, ub);   // (below 2^64: U < 2^63)
-    const uint64_t hi = (uint64_t)ua * ua + (mid >> 32);
-    n = (int)(hi >> 50);
-    const uint64_t f = (hi << 14) | ((uint32_t)mid >> 18);
+// 2^(-f 2^-64) in units of 2^-63, in [2^62, 2^63] (t: the table in shared memory).
+__device__ __forceinline__ uint64_t exp2_neg_frac(uint64_t f, const uint64_t *t) {
     const uint64_t T = t[f >> 56];
     const uint64_t r = f << 8;                                // remainder / 2^-8, in units of 2^-64
     const uint32_t r32 = (uint32_t)(r >> 32);
@@ -169,6 +155,33 @@ __device__ __forceinline__ uint64_t exp_neg_sq(double x, const uint64_t *t, int 
     const uint64_t d = mulhi_near(a1, r) >> 8;                // 1 - 2^(-r'), in units of 2^-64
     const uint64_t s = T - mulhi_near(T, d);
     return s < (1ull << 62) ? (1ull << 62) : s;               // (one unit below 1/2 by truncation)
+}
+
+// Significand (in units of 2^-63, in [2^62, 2^63]) and integer exponent n of
+// exp(-x^2) = sig 2^(-n), for |x| < 53. The factor sqrt(log2 e) is applied in fixed point:
+// folded into a double-precision x it would carry a rounding that is the same at every point.
+__device__ __forceinline__ uint64_t exp_neg_sq(double x, const uint64_t *t, int &n) {
+    // U = sqrt(log2 e) |x| 2^57
+    const uint64_t b = (uint64_t)__double_as_longlong(x) & 0x7fffffffffffffffull;
+    const int sh = (int)(b >> 52) - 1023 + 5;                 // exponent + 57 - 52
+    const uint64_t mant = (b & 0x000fffffffffffffull) | 0x0010000000000000ull;
+    const uint64_t U = mulhi_near(sh >= 0 ? mant << sh : (sh > -64 ? mant >> -sh : 0), kSqrtLog2eFix) << 1;
+    // U^2 = log2(e) x^2 2^114: integer part, fraction of 64 bits
+    const uint32_t ua = (uint32_t)(U >> 32), ub = (uint32_t)U;
+    const uint64_t mid = 2 * ((uint64_t)ua * ub) + __umulhi(ub, ub);   // (below 2^64: U < 2^63)
+    const uint64_t hi = (uint64_t)ua * ua + (mid >> 32);
+    n = (int)(hi >> 50);
+    return exp2_neg_frac((hi << 14) | ((uint32_t)mid >> 18), t);
+}
+
+// The same for exp(-d), 0 <= d < 2^12, d as significand and exponent.
+__device__ __forceinline__ uint64_t exp_neg(const PosFp &d, const uint64_t *t, int &n) {
+    // log2(e) d = m 2^(e + 1): m in units of 2^(e + 1) = 2^-k
+    const uint64_t m = mulhi_near(d.m, kLog2eFix);
+    const int k = -(d.e + 1);                                 // 52 .. (d < 2^12)
+    n = k >= 64 ? 0 : (int)(m >> k);
+    const uint64_t f = k >= 64 ? (k - 64 < 64 ? m >> (k - 64) : 0) : m << (64 - k);
+    return exp2_neg_frac(f, t);
 }
 
 }  // namespace mg

@@ -1,4 +1,5 @@
 // K2 (line data) and K3 (Feautrier formal solve with the diagonal ALO), Sec. 3.3-3.4.
+#include <algorithm>
 #include <cmath>
 #include "common.cuh"
 #include "posfp.cuh"
@@ -434,6 +435,12 @@ struct ImageArgs {
     double *I;                // [n][n_ch]
     double *xy;               // [n][2]
     const float *dsf, *vparf, *bf, *linef;   // FP32 copies for the FP32 kernel
+    float nf[3], inv_chi_min;
+    struct {                  // the first lines within reach, for the line kernels (image.cuh)
+        int32_t l2;
+        float rat, dnl, nrm;  // nrm = c/(nu sqrt pi)
+        int32_t cm, ic;       // exponents of chi_min nu/2^28 and of the boundary intensity, rounded down
+    } lf[4];
 };
 
 __device__ __forceinline__ double ls_step(double I, double d, double Sa, double Sb) {
@@ -523,73 +530,7 @@ __global__ void k_image64(ImageArgs a) {
     }
 }
 
-// FP32 image of a mixed-precision context. The pair is staged once per point in shared
-// memory in FP32 (from the FP32 ray store, widths and line data): path length,
-// rest-frame line-of-sight velocity w, reciprocal width, and the interpolated (eta, chi)
-// of the NOV lines within reach; then each thread carries one channel through the pair.
-// The linear-source weights use their Taylor series below dtau = 0.05 (4 terms: relative
-// error below 2e-8 there), where 1 - alpha would cancel in FP32; divisions are the fast
-// approximate ones (2 ulp).
-constexpr int kImgLines = 4;
-
-struct ImgSmem32 {
-    float *ds, *w, *ib, *lin;   // lin: [K][NOV][2] (eta, chi)
-};
-
-template <int NOV>
-__device__ void stage_half_img32(const ImageArgs &a, int64_t o, int r, int base, int dir, float nvo, float sgn,
-                                 const ImgSmem32 &S) {
-    const SolveArgs &sa = a.s;
-    const int64_t off = sa.ray_off[o * sa.R + r];
-    const int len = (int)(sa.ray_off[o * sa.R + r + 1] - off);
-    int l2[NOV];
-#pragma unroll
-    for (int i = 0; i < NOV; i++) l2[i] = a.ov[i].l2;
-    for (int e = threadIdx.x; e < len; e += blockDim.x) {
-        const int32_t c = sa.cells[off + e];
-        const int32_t prev = e ? sa.cells[off + e - 1] : (int32_t)o;
-        const int x0 = e ? sa.xcum[off + e - 1] : 0;
-        const int ns = sa.xcum[off + e] - x0 - 1;
-        const float pv = e ? a.vparf[off + e - 1] : 0.0f;
-        const float ve = a.vparf[off + e];
-        const float inv = 1.0f / (float)(ns + 1);
-        const float dse = a.dsf[off + e] * inv;
-        const float bp = a.bf[prev], bc = a.bf[c];
-        const float *pa = a.linef + (int64_t)prev * 2 * sa.L, *pb = a.linef + (int64_t)c * 2 * sa.L;
-        float la[NOV][2], lb[NOV][2];
-#pragma unroll
-        for (int i = 0; i < NOV; i++) {
-            la[i][0] = pa[2 * l2[i]]; la[i][1] = pa[2 * l2[i] + 1];
-            lb[i][0] = pb[2 * l2[i]]; lb[i][1] = pb[2 * l2[i] + 1];
-        }
-        for (int j = 1; j <= ns + 1; j++) {
-            const float wt = (float)j * inv;
-            const int idx = base + dir * (x0 + j - 1);
-            S.ds[dir < 0 ? idx : idx - 1] = dse;
-            S.w[idx] = nvo + sgn * ((1.0f - wt) * pv + wt * ve);
-            S.ib[idx] = 1.0f / ((1.0f - wt) * bp + wt * bc);
-#pragma unroll
-            for (int i = 0; i < NOV; i++) {
-                S.lin[(idx * NOV + i) * 2] = (1.0f - wt) * la[i][0] + wt * lb[i][0];
-                S.lin[(idx * NOV + i) * 2 + 1] = (1.0f - wt) * la[i][1] + wt * lb[i][1];
-            }
-        }
-    }
-}
-
-__device__ __forceinline__ float ls_step32(float I, float d, float Sa, float Sb) {
-    const float e = __expf(-d);
-    float wa, wb;
-    if (d < 0.05f) {
-        wb = d * (0.5f - d * (1.0f / 6.0f - d * (1.0f / 24.0f - d * (1.0f / 120.0f))));
-        wa = d * (0.5f - d * (1.0f / 3.0f - d * (1.0f / 8.0f - d * (1.0f / 30.0f))));
-    } else {
-        const float alpha = __fdividef(1.0f - e, d);
-        wb = 1.0f - alpha;
-        wa = alpha - e;
-    }
-    return e * I + wa * Sa + wb * Sb;
-}
+constexpr int kImgLines = 4;   // lines in reach that the line kernels (image.cuh) take
 
 // B_nu(T) in FP32, ordered so that no intermediate leaves the FP32 range.
 __device__ __forceinline__ float planck_f(float nu, float T) {
@@ -598,87 +539,9 @@ __device__ __forceinline__ float planck_f(float nu, float T) {
     return k2h * nc * nc * nu / expm1f(khk * nu / T);
 }
 
-template <int NOV>
-__global__ void k_image32(ImageArgs a) {
-    extern __shared__ float smf[];
-    const SolveArgs &sa = a.s;
-    const int kmax = sa.kmax;
-    ImgSmem32 S;
-    S.ds = smf;
-    S.w = S.ds + kmax;
-    S.ib = S.w + kmax;
-    S.lin = S.ib + kmax;
-    const int64_t o = blockIdx.x;
-    const double *xo = a.pos + 3 * o, *vo = a.vel + 3 * o;
-    if (threadIdx.x == 0) {
-        a.xy[2 * o] = xo[0] * a.e1[0] + xo[1] * a.e1[1] + xo[2] * a.e1[2];
-        a.xy[2 * o + 1] = xo[0] * a.e2[0] + xo[1] * a.e2[1] + xo[2] * a.e2[2];
-    }
-    const float nvo = (float)a.n0 * (float)vo[0] + (float)a.n1 * (float)vo[1] + (float)a.n2 * (float)vo[2];
-    const int64_t ofb = sa.ray_off[o * sa.R + a.rb], ofl = sa.ray_off[o * sa.R + a.rf];
-    const int lb = (int)(sa.ray_off[o * sa.R + a.rb + 1] - ofb);
-    const int lf = (int)(sa.ray_off[o * sa.R + a.rf + 1] - ofl);
-    const int Kb = lb ? sa.xcum[ofb + lb - 1] : 0;
-    const int Kf = lf ? sa.xcum[ofl + lf - 1] : 0;
-    const int K = Kb + 1 + Kf;
-    if (K > kmax) {
-        if (threadIdx.x == 0) atomicOr(sa.err, 2);
-        return;
-    }
-    stage_half_img32<NOV>(a, o, a.rb, Kb - 1, -1, nvo, -1.0f, S);
-    stage_half_img32<NOV>(a, o, a.rf, Kb + 1, +1, nvo, +1.0f, S);
-    if (threadIdx.x == 0) {
-        S.w[Kb] = nvo;
-        S.ib[Kb] = 1.0f / a.bf[o];
-        const float *pl = a.linef + o * 2 * sa.L;
-#pragma unroll
-        for (int i = 0; i < NOV; i++) {
-            S.lin[(Kb * NOV + i) * 2] = pl[2 * a.ov[i].l2];
-            S.lin[(Kb * NOV + i) * 2 + 1] = pl[2 * a.ov[i].l2 + 1];
-        }
-    }
-    __syncthreads();
-    constexpr float kCspf = (float)(kC / kSqrtPi);
-    float dnl[NOV], rat[NOV], nrm[NOV];
-#pragma unroll
-    for (int i = 0; i < NOV; i++) {
-        dnl[i] = (float)a.ov[i].dnl;
-        rat[i] = (float)a.ov[i].rat;
-        nrm[i] = (float)a.ov[i].inv_nu2 * kCspf;
-    }
-    const float chi_min = (float)sa.chi_min, dtau_min = (float)sa.dtau_min, T_cmb = (float)sa.T_cmb;
-    const float nu_l = (float)a.nu_l, kic = (float)(1.0 / kC);
-    for (int c = threadIdx.x; c < a.n_ch; c += blockDim.x) {
-        const float u = (float)a.u[c];
-        const float k1 = 1.0f + u * kic;
-        float I = 0.0f, chi_prev = 0.0f, S_prev = 0.0f;
-        for (int k = 0; k < K; k++) {
-            const float w = S.w[k], ibk = S.ib[k];
-            const float base = u - w * k1;
-            float eta = 0.0f, chi = 0.0f;
-#pragma unroll
-            for (int i = 0; i < NOV; i++) {
-                const float x = (dnl[i] + rat[i] * base) * ibk;
-                const float phi = __expf(-x * x) * (nrm[i] * ibk);
-                eta += S.lin[(k * NOV + i) * 2] * phi;
-                chi += S.lin[(k * NOV + i) * 2 + 1] * phi;
-            }
-            chi = fmaxf(chi, chi_min);
-            const float Sk = __fdividef(eta, chi);
-            if (k == 0) {
-                I = planck_f(nu_l * k1 * (1.0f - w * kic), T_cmb);
-            } else {
-                const float dt = fmaxf(0.5f * (chi_prev + chi) * S.ds[k - 1], dtau_min);
-                I = ls_step32(I, dt, S_prev, Sk);
-            }
-            chi_prev = chi;
-            S_prev = Sk;
-        }
-        a.I[o * a.n_ch + c] = (double)I;
-    }
-}
-
 }  // namespace
+
+#include "image.cuh"
 
 namespace {
 // Largest |a_new - a_old| / a_new over m values into *word (as the bits of a double, which
@@ -902,7 +765,7 @@ int mg_launch_line_data64(mg_ctx *ctx, float *linef, unsigned long long *neg) {
     return MG_OK;
 }
 
-int mg_launch_image(mg_ctx *ctx, int ray, int line, int n_ch, const double *d_u, const Overlap *d_ov, int n_ov,
+int mg_launch_image(mg_ctx *ctx, int ray, int line, int n_ch, const double *d_u, const Overlap *d_ov, const Overlap *h_ov, int n_ov,
                     double *d_I, double *d_xy) {
     ImageArgs a{};
     SolveArgs &s = a.s;
@@ -941,16 +804,44 @@ int mg_launch_image(mg_ctx *ctx, int ray, int line, int n_ch, const double *d_u,
     // FP32 in a mixed-precision context when the lines within reach fit the staging
     a.dsf = ctx->d_dsf; a.vparf = ctx->d_vparf; a.bf = ctx->d_bf; a.linef = ctx->d_imglf;
     const size_t smem32 = sizeof(float) * (size_t)s.kmax * (3 + 2 * (size_t)n_ov);
+    for (int i = 0; i < 3; i++) a.nf[i] = (float)n[i];
+    a.inv_chi_min = (float)(1.0 / s.chi_min);
+    for (int i = 0; i < std::min(n_ov, kImgLines); i++) {
+        const Overlap &v = h_ov[i];
+        const double nu = 1.0 / v.inv_nu2;
+        a.lf[i].l2 = v.l2;
+        a.lf[i].rat = (float)v.rat;
+        a.lf[i].dnl = (float)v.dnl;
+        a.lf[i].nrm = (float)v.inv_nu2 * (float)(kC / kSqrtPi);
+        a.lf[i].cm = std::ilogb(s.chi_min) + std::ilogb(nu) - 28 - 1;
+        a.lf[i].ic = std::ilogb(2.0 * kH * nu * nu * nu / (kC * kC) / std::expm1(kH * nu / (kKB * s.T_cmb)));
+    }
+    const size_t smem = sizeof(double) * (size_t)s.kmax * 4 + sizeof(int32_t) * 2 * (size_t)s.kmax;
+    const int skip = ctx->opt.chi_min * ctx->extent < 1e-14;
+    // points staged at a time: a quarter more than the mean pair (more would cost occupancy)
+    const double mean = 2.0 * (double)ctx->n_expanded / ((double)ctx->n * ctx->R) + 1.0;
+    const int cap = std::min({kImgCap, ((int)(1.25 * mean) + 63) / 32 * 32, (s.kmax + 31) / 32 * 32});
+    constexpr int kMaxImgSmem = 200 * 1024;   // (512 points of four lines with 256 threads need 152 KB)
     if (ctx->opt.precision == MG_MIXED && n_ov <= kImgLines && smem32 <= 227 * 1024 && a.linef) {
-        void (*kern)(ImageArgs) = n_ov == 1 ? k_image32<1> : n_ov == 2 ? k_image32<2> : n_ov == 3 ? k_image32<3>
-                                                                                                  : k_image32<4>;
-        MG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem32));
+        void (*kern)(ImageArgs) = n_ov == 1 ? k_image32_lines<1> : n_ov == 2 ? k_image32_lines<2>
+                                : n_ov == 3 ? k_image32_lines<3> : k_image32_lines<4>;
         MgTimed t(ctx, "image_fp32");
-        kern<<<(unsigned)ctx->n, threads, smem32, ctx->stream>>>(a);
+        kern<<<(unsigned)ctx->n, threads, 0, ctx->stream>>>(a);
+        k_image_xy<<<(unsigned)((ctx->n + 127) / 128), 128, 0, ctx->stream>>>(a);
+    } else if (smem > 227 * 1024) {
+        return mg_fail(ctx, MG_ERR_CAPACITY, "mg_image: longest ray pair does not fit in shared memory");
+    } else if (n_ov <= kImgLines) {
+        void (*kern)(ImageArgs, int, int) = n_ov == 1 ? k_image64_lines<1> : n_ov == 2 ? k_image64_lines<2>
+                                          : n_ov == 3 ? k_image64_lines<3> : k_image64_lines<4>;
+        auto bytes = [&](int cap) {
+            return n_ov == 1 ? ImgStage64<1>::bytes(cap, threads) : n_ov == 2 ? ImgStage64<2>::bytes(cap, threads)
+                 : n_ov == 3 ? ImgStage64<3>::bytes(cap, threads) : ImgStage64<4>::bytes(cap, threads);
+        };
+        MG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxImgSmem));
+        MgTimed t(ctx, "image_fp64");
+        kern<<<(unsigned)ctx->n, threads, bytes(cap), ctx->stream>>>(a, skip, cap);
+        k_image_xy<<<(unsigned)((ctx->n + 127) / 128), 128, 0, ctx->stream>>>(a);
     } else {
-        const size_t smem = sizeof(double) * (size_t)s.kmax * 4 + sizeof(int32_t) * 2 * (size_t)s.kmax;
-        if (smem > 227 * 1024)
-            return mg_fail(ctx, MG_ERR_CAPACITY, "mg_image: longest ray pair does not fit in shared memory");
         MG_CUDA(cudaFuncSetAttribute(k_image64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
         MgTimed t(ctx, "image_fp64");
         k_image64<<<(unsigned)ctx->n, threads, smem, ctx->stream>>>(a);

@@ -3,7 +3,7 @@ of its splits, against the oracle within 1e-10: bins that leave lanes idle, stra
 or need several chunks per line; one to sixteen warps per origin; few and many ray pairs;
 the band terms of a line spread over chunks; rescaling of very thick columns; inverted
 populations (the opacity floor keeps the line's emission); a floor too large for far
-points to be left out."""
+points to be left out; density jumps of ten decades between neighbours."""
 import numpy as np
 import pytest
 
@@ -70,3 +70,11 @@ def test_inverted_populations():
 
 def test_large_floor():
     _check(syn.model_clumpy_3d(n=150, seed=4, n_lev=3, nside=1), chi_min=1e-18)
+
+
+def test_density_and_temperature_jumps():
+    m = syn.model_clumpy_3d(n=200, seed=8, nside=1, n_lev=3)
+    dense = np.random.default_rng(1).random(m.n) < 0.2
+    m.n_spec = np.where(dense, m.n_spec, 1e-10 * m.n_spec)
+    m.T = np.where(dense, 10.0, 160.0)
+    _check(m)
