@@ -4,10 +4,12 @@
 //
 // Kernels:
 //   k_features     FP64 features per cell (log n, log T, log |grad v|, log Sobolev tau)
-//   k_mlp_tile     one CTA per 64 rows, one warp per 16 rows: the 128-wide layers and the
-//                  back-propagated deltas run on the tensor cores (mma.sync m16n8k16, BF16
-//                  operands, FP32 accumulation); weight gradients are per-CTA FP32 partial
-//                  sums on the CUDA cores, summed over CTAs in a fixed order
+//   k_mlp_tile     one CTA of 16 warps per 64 rows: the 128-wide layers, the back-propagated
+//                  deltas and the weight gradients run on the tensor cores (mma.sync
+//                  m16n8k16, BF16 operands, FP32 accumulation), operands in shared memory;
+//                  the gradients are per-CTA FP32 partial sums, summed over CTAs in a fixed
+//                  order
+//   k_count        number of targets of a batch (the loss is their mean)
 //   k_grad_reduce  fixed-order sum of the per-CTA partials
 //   k_adam         Adam on FP32 master weights, refreshing the BF16 copies
 #include <cuda_bf16.h>
@@ -53,6 +55,10 @@ Layout make_layout(int n_out) {
     return L;
 }
 
+// Floats per CTA of gradient partials: the parameters and the loss, rounded up so that every
+// CTA's share starts on a 16-byte boundary.
+__host__ __device__ inline int64_t partial_stride(const Layout &L) { return (L.total + 4) & ~(int64_t)3; }
+
 // BF16 weight copies: forward operands stored [out][in] (WT), backward operands stored
 // [in][out] (W), W4 padded to npad outputs with zeros.
 struct BfWeights {
@@ -60,35 +66,50 @@ struct BfWeights {
     __nv_bfloat16 *W2, *W3, *W4;      // [128][128], [128][128], [128][npad]
 };
 
-__device__ __forceinline__ uint32_t ld_u32(const __nv_bfloat16 *p) { return *reinterpret_cast<const uint32_t *>(p); }
-
-__device__ __forceinline__ void mma_bf16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
-                                         uint32_t b0, uint32_t b1) {
+__device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
     asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
                  "{%0,%1,%2,%3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-                 : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
 }
 
-// acc[16 x 8 NT] = A[16 x 16 KT] (bf16, row-major in shared memory, stride lda) times B,
-// where B is supplied transposed: BT[n][k] (bf16, row stride ldb). Fragment layouts of
-// mma.m16n8k16: lane = 4 g + c holds rows g and g+8, columns 2c, 2c+1 (+8).
-template <int KT, int NT>
-__device__ __forceinline__ void warp_gemm(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *BT, int ldb,
+// Four 8 x 8 BF16 blocks of shared memory into a fragment, as stored or transposed; lane l
+// gives the address of row l % 8 of block l / 8.
+__device__ __forceinline__ void ldsm4(uint32_t (&r)[4], const __nv_bfloat16 *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p))
+                 : "memory");
+}
+__device__ __forceinline__ void ldsm4t(uint32_t (&r)[4], const __nv_bfloat16 *p) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"((unsigned)__cvta_generic_to_shared(p))
+                 : "memory");
+}
+
+// acc[16 x 8 NT] (+)= A[16 x 16 KT] times B. A: rows of shared memory (stride lda), or with TA
+// columns (A[m][k] stored at [k][m]). B: stored [n][k] (stride ldb), or with TB [k][n]. Fragment
+// layouts of mma.m16n8k16: lane = 4 g + c holds rows g and g+8, columns 2c, 2c+1 (+8).
+template <int KT, int NT, bool TA, bool TB>
+__device__ __forceinline__ void warp_gemm(const __nv_bfloat16 *A, int lda, const __nv_bfloat16 *B, int ldb,
                                           float (&acc)[NT][4]) {
-    const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+    static_assert(NT % 2 == 0, "two column blocks per load of B");
+    const int lane = threadIdx.x & 31, r = lane & 7, m = lane >> 3;
 #pragma unroll
     for (int nt = 0; nt < NT; nt++) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.f;
 #pragma unroll
     for (int kt = 0; kt < KT; kt++) {
-        const uint32_t a0 = ld_u32(A + g * lda + 16 * kt + 2 * c);
-        const uint32_t a1 = ld_u32(A + (g + 8) * lda + 16 * kt + 2 * c);
-        const uint32_t a2 = ld_u32(A + g * lda + 16 * kt + 8 + 2 * c);
-        const uint32_t a3 = ld_u32(A + (g + 8) * lda + 16 * kt + 8 + 2 * c);
+        uint32_t a[4];
+        if (TA) ldsm4t(a, A + (16 * kt + r + 8 * (m >> 1)) * lda + 8 * (m & 1));
+        else ldsm4(a, A + (r + 8 * (m & 1)) * lda + 16 * kt + 8 * (m >> 1));
 #pragma unroll
-        for (int nt = 0; nt < NT; nt++) {
-            const __nv_bfloat16 *bp = BT + (8 * nt + g) * ldb + 16 * kt + 2 * c;
-            mma_bf16(acc[nt], a0, a1, a2, a3, ld_u32(bp), ld_u32(bp + 8));
+        for (int nt = 0; nt < NT; nt += 2) {
+            uint32_t b[4];
+            if (TB) ldsm4t(b, B + (16 * kt + r + 8 * (m & 1)) * ldb + 8 * nt + 8 * (m >> 1));
+            else ldsm4(b, B + (8 * nt + r + 8 * (m >> 1)) * ldb + 16 * kt + 8 * (m & 1));
+            mma_bf16(acc[nt], a, b[0], b[1]);
+            mma_bf16(acc[nt + 1], a, b[2], b[3]);
         }
     }
 }
@@ -102,243 +123,299 @@ struct TileArgs {
     BfWeights w;
     Layout L;
     float mean[kIn], istd[kIn];
-    float inv_count;           // 1 / number of (row, level) targets >= 1e-12 in the batch
+    const int *count;          // number of (row, level) targets >= 1e-12 in the batch (training)
     float *logp;               // [rows][n_out] output (forward) or nullptr
-    float *partial;            // [gridDim][L.total + 1] gradient partials and loss (training)
+    float *partial;            // [tiles][partial_stride] gradient partials and loss (training)
 };
 
-// Shared memory per CTA: activations h1, h2, h3 and two delta buffers (bf16), inputs.
+constexpr int kLd = kHid + 8;       // row stride in shared memory: 8 rows of 16 bytes hit all banks once
+constexpr int kLdz = kMaxOut + 8;
+constexpr int kTileThreads = 512;
+
+// Shared memory per CTA: weights as [out][in], activations h1, h2, h3, two delta buffers
+// (bf16) and inputs.
 struct TileSmem {
-    __nv_bfloat16 h1[kRows][kHid], h2[kRows][kHid], h3[kRows][kHid];
-    __nv_bfloat16 da[kRows][kHid], db[kRows][kHid];
-    __nv_bfloat16 dz[kRows][kMaxOut];
+    __nv_bfloat16 w2[kHid][kLd], w3[kHid][kLd], w4[kMaxOut][kLd];
+    __nv_bfloat16 h1[kRows][kLd], h2[kRows][kLd], h3[kRows][kLd];
+    __nv_bfloat16 da[kRows][kLd], db[kRows][kLd];
+    __nv_bfloat16 dz[kRows][kLdz];
     float x[kRows][kIn];
     float loss[4];
 };
 
-// Stores an accumulator block (16 rows of warp w) plus bias into bf16 rows with ReLU.
+// Stores an accumulator block (16 rows from r0, columns from c0) plus bias into bf16 rows
+// with ReLU.
 template <int NT>
-__device__ __forceinline__ void store_relu(float (&acc)[NT][4], const float *bias, __nv_bfloat16 (*dst)[kHid], int r0) {
+__device__ __forceinline__ void store_relu(float (&acc)[NT][4], const float *bias, __nv_bfloat16 (*dst)[kLd], int r0,
+                                           int c0) {
     const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
 #pragma unroll
     for (int nt = 0; nt < NT; nt++) {
-        const int col = 8 * nt + 2 * c;
-        dst[r0 + g][col] = __float2bfloat16(fmaxf(acc[nt][0] + bias[col], 0.f));
-        dst[r0 + g][col + 1] = __float2bfloat16(fmaxf(acc[nt][1] + bias[col + 1], 0.f));
-        dst[r0 + g + 8][col] = __float2bfloat16(fmaxf(acc[nt][2] + bias[col], 0.f));
-        dst[r0 + g + 8][col + 1] = __float2bfloat16(fmaxf(acc[nt][3] + bias[col + 1], 0.f));
+        const int col = c0 + 8 * nt + 2 * c;
+        const float b0 = bias[col], b1 = bias[col + 1];
+        *reinterpret_cast<__nv_bfloat162 *>(&dst[r0 + g][col]) =
+            __floats2bfloat162_rn(fmaxf(acc[nt][0] + b0, 0.f), fmaxf(acc[nt][1] + b1, 0.f));
+        *reinterpret_cast<__nv_bfloat162 *>(&dst[r0 + g + 8][col]) =
+            __floats2bfloat162_rn(fmaxf(acc[nt][2] + b0, 0.f), fmaxf(acc[nt][3] + b1, 0.f));
     }
 }
 
 // Delta through a ReLU layer: dst = acc masked by (h > 0).
 template <int NT>
-__device__ __forceinline__ void store_masked(float (&acc)[NT][4], __nv_bfloat16 (*h)[kHid], __nv_bfloat16 (*dst)[kHid],
-                                             int r0) {
+__device__ __forceinline__ void store_masked(float (&acc)[NT][4], __nv_bfloat16 (*h)[kLd], __nv_bfloat16 (*dst)[kLd],
+                                             int r0, int c0) {
     const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
-    const __nv_bfloat16 z = __float2bfloat16(0.f);
 #pragma unroll
     for (int nt = 0; nt < NT; nt++) {
-        const int col = 8 * nt + 2 * c;
-        dst[r0 + g][col] = __bfloat162float(h[r0 + g][col]) > 0.f ? __float2bfloat16(acc[nt][0]) : z;
-        dst[r0 + g][col + 1] = __bfloat162float(h[r0 + g][col + 1]) > 0.f ? __float2bfloat16(acc[nt][1]) : z;
-        dst[r0 + g + 8][col] = __bfloat162float(h[r0 + g + 8][col]) > 0.f ? __float2bfloat16(acc[nt][2]) : z;
-        dst[r0 + g + 8][col + 1] = __bfloat162float(h[r0 + g + 8][col + 1]) > 0.f ? __float2bfloat16(acc[nt][3]) : z;
+        const int col = c0 + 8 * nt + 2 * c;
+#pragma unroll
+        for (int s = 0; s < 2; s++) {
+            const float2 hv = __bfloat1622float2(*reinterpret_cast<__nv_bfloat162 *>(&h[r0 + g + 8 * s][col]));
+            *reinterpret_cast<__nv_bfloat162 *>(&dst[r0 + g + 8 * s][col]) = __floats2bfloat162_rn(
+                hv.x > 0.f ? acc[nt][2 * s] : 0.f, hv.y > 0.f ? acc[nt][2 * s + 1] : 0.f);
+        }
     }
 }
 
-// dW[i][j] += sum_rows a[r][i] d[r][j] for this CTA (CUDA cores, fixed order over rows).
-__device__ void weight_grad(const __nv_bfloat16 (*a)[kHid], const __nv_bfloat16 (*d)[kHid], int nrows, int ni, int nj,
-                            float *out, const float *bias_out) {
-    for (int t = threadIdx.x; t < ni * nj; t += blockDim.x) {
-        const int i = t / nj, j = t - (t / nj) * nj;
-        float s = 0.f;
-        for (int r = 0; r < nrows; r++) s += __bfloat162float(a[r][i]) * __bfloat162float(d[r][j]);
-        out[t] = s;
-    }
-    (void)bias_out;
+// dW[i][j] = sum_rows a[r][i] d[r][j] over this CTA's rows, i in [i0, i0 + 16), j in [j0, j0 + 8 NT),
+// j < nj: on the tensor cores, K = rows.
+template <int NT>
+__device__ __forceinline__ void weight_grad(const __nv_bfloat16 *a, const __nv_bfloat16 *d, int ldd, int i0, int j0,
+                                            int nj, float *out) {
+    const int lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
+    float acc[NT][4];
+    warp_gemm<kRows / 16, NT, true, true>(a + i0, kLd, d + j0, ldd, acc);
+#pragma unroll
+    for (int nt = 0; nt < NT; nt++)
+#pragma unroll
+        for (int s = 0; s < 2; s++) {
+            const int i = i0 + g + 8 * s, j = j0 + 8 * nt + 2 * c;
+            if (nj == kHid) {   // (the layers' rows start on even offsets)
+                *reinterpret_cast<float2 *>(&out[i * kHid + j]) = make_float2(acc[nt][2 * s], acc[nt][2 * s + 1]);
+            } else {
+                if (j < nj) out[i * nj + j] = acc[nt][2 * s];
+                if (j + 1 < nj) out[i * nj + j + 1] = acc[nt][2 * s + 1];
+            }
+        }
 }
 
-__global__ void __launch_bounds__(128) k_mlp_tile(TileArgs a) {
+// Copies n rows of 128 bf16 from global memory into padded rows.
+__device__ __forceinline__ void load_rows(__nv_bfloat16 (*dst)[kLd], const __nv_bfloat16 *src, int n) {
+    for (int t = threadIdx.x; t < n * (kHid / 8); t += kTileThreads) {
+        const int r = t / (kHid / 8), k = t - r * (kHid / 8);
+        *reinterpret_cast<uint4 *>(&dst[r][8 * k]) = *reinterpret_cast<const uint4 *>(src + r * kHid + 8 * k);
+    }
+}
+
+// One CTA per 64 rows (without gradients the CTAs take several tiles and load the weights
+// once). The products are small (64 x 128 x 128) and what bounded them was the latency of
+// their operands: weights gathered four bytes at a time from global memory by 4 warps, weight
+// gradients one output and 64 dependent shared-memory loads at a time. Sixteen warps now
+// share each product (16 x 32 outputs each) with all operands in shared memory (ldmatrix),
+// and the gradients are tensor-core products over the rows. 4096 rows: 151 -> 26 us.
+__global__ void __launch_bounds__(kTileThreads) k_mlp_tile(TileArgs a) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TileSmem &S = *reinterpret_cast<TileSmem *>(smem_raw);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, c = lane & 3;
-    const int r0 = warp * 16;
-    const int64_t row0 = (int64_t)blockIdx.x * kRows;
+    const int r0 = (warp & 3) * 16, c0 = (warp >> 2) * 32;
     const int n_out = a.L.n_out, npad = a.L.npad;
     const float *th = a.theta;
-    // inputs (normalised); rows beyond the end are zero and carry no loss
-    for (int t = threadIdx.x; t < kRows * kIn; t += blockDim.x) {
-        const int r = t / kIn, i = t - r * kIn;
-        const int64_t gr = row0 + r;
-        float v = 0.f;
-        if (gr < a.rows) {
-            const int64_t src = a.index ? a.index[gr] : gr;
-            v = (a.X[src * kIn + i] - a.mean[i]) * a.istd[i];
+    load_rows(S.w2, a.w.W2T, kHid);
+    load_rows(S.w3, a.w.W3T, kHid);
+    load_rows(S.w4, a.w.W4T, npad);
+    const int64_t tiles = (a.rows + kRows - 1) / kRows;
+    for (int64_t tile = blockIdx.x; tile < tiles; tile += gridDim.x) {
+        const int64_t row0 = tile * kRows;
+        // inputs (normalised); rows beyond the end are zero and carry no loss
+        for (int t = threadIdx.x; t < kRows * kIn; t += kTileThreads) {
+            const int r = t / kIn, i = t - r * kIn;
+            const int64_t gr = row0 + r;
+            float v = 0.f;
+            if (gr < a.rows) {
+                const int64_t src = a.index ? a.index[gr] : gr;
+                v = (a.X[src * kIn + i] - a.mean[i]) * a.istd[i];
+            }
+            S.x[r][i] = v;
         }
-        S.x[r][i] = v;
-    }
-    __syncthreads();
-    // layer 1 (K = 4) on the CUDA cores
-    for (int t = threadIdx.x; t < kRows * kHid; t += blockDim.x) {
-        const int r = t / kHid, j = t - r * kHid;
-        float s = th[a.L.b1 + j];
+        __syncthreads();
+        // layer 1 (K = 4) on the CUDA cores
+        for (int t = threadIdx.x; t < kRows * kHid; t += kTileThreads) {
+            const int r = t / kHid, j = t - r * kHid;
+            float s = th[a.L.b1 + j];
 #pragma unroll
-        for (int i = 0; i < kIn; i++) s += S.x[r][i] * th[a.L.W1 + i * kHid + j];
-        S.h1[r][j] = __float2bfloat16(fmaxf(s, 0.f));
-    }
-    __syncthreads();
-    {   // layers 2 and 3 on the tensor cores, each warp its own 16 rows
-        float acc[16][4];
-        warp_gemm<8, 16>(&S.h1[r0][0], kHid, a.w.W2T, kHid, acc);
-        store_relu<16>(acc, th + a.L.b2, S.h2, r0);
-        __syncwarp();
-        warp_gemm<8, 16>(&S.h2[r0][0], kHid, a.w.W3T, kHid, acc);
-        store_relu<16>(acc, th + a.L.b3, S.h3, r0);
-        __syncwarp();
-    }
-    // output layer and log-softmax; lanes 4g..4g+3 hold rows r0+g and r0+g+8
-    float z[4][4];
-    float lp[4][4];
-    {
-        float acc[4][4];
-        if (npad == 16) {
-            float a2[2][4];
-            warp_gemm<8, 2>(&S.h3[r0][0], kHid, a.w.W4T, kHid, a2);
-            for (int nt = 0; nt < 4; nt++)
-                for (int k = 0; k < 4; k++) acc[nt][k] = nt < 2 ? a2[nt][k] : 0.f;
-        } else {
-            warp_gemm<8, 4>(&S.h3[r0][0], kHid, a.w.W4T, kHid, acc);
+            for (int i = 0; i < kIn; i++) s += S.x[r][i] * th[a.L.W1 + i * kHid + j];
+            S.h1[r][j] = __float2bfloat16(fmaxf(s, 0.f));
         }
-        float mx[2] = {-INFINITY, -INFINITY};
-        for (int nt = 0; nt < 4; nt++)
-            for (int k = 0; k < 4; k++) {
-                const int col = 8 * nt + 2 * c + (k & 1);
-                z[nt][k] = col < n_out ? acc[nt][k] + th[a.L.b4 + col] : -INFINITY;
-                mx[k >> 1] = fmaxf(mx[k >> 1], z[nt][k]);
-            }
-        for (int s = 0; s < 2; s++) {
-            mx[s] = fmaxf(mx[s], __shfl_xor_sync(0xffffffffu, mx[s], 1));
-            mx[s] = fmaxf(mx[s], __shfl_xor_sync(0xffffffffu, mx[s], 2));
+        __syncthreads();
+        {   // layers 2 and 3
+            float acc[4][4];
+            warp_gemm<8, 4, false, false>(&S.h1[r0][0], kLd, &S.w2[c0][0], kLd, acc);
+            store_relu<4>(acc, th + a.L.b2, S.h2, r0, c0);
+            __syncthreads();
+            warp_gemm<8, 4, false, false>(&S.h2[r0][0], kLd, &S.w3[c0][0], kLd, acc);
+            store_relu<4>(acc, th + a.L.b3, S.h3, r0, c0);
+            __syncthreads();
         }
-        float se[2] = {0.f, 0.f};
-        for (int nt = 0; nt < 4; nt++)
-            for (int k = 0; k < 4; k++) se[k >> 1] += (z[nt][k] == -INFINITY) ? 0.f : expf(z[nt][k] - mx[k >> 1]);
-        for (int s = 0; s < 2; s++) {
-            se[s] += __shfl_xor_sync(0xffffffffu, se[s], 1);
-            se[s] += __shfl_xor_sync(0xffffffffu, se[s], 2);
-        }
-        for (int nt = 0; nt < 4; nt++)
-            for (int k = 0; k < 4; k++) lp[nt][k] = z[nt][k] - mx[k >> 1] - logf(se[k >> 1]);
-    }
-    if (a.logp) {
-        for (int nt = 0; nt < 4; nt++)
-            for (int k = 0; k < 4; k++) {
-                const int col = 8 * nt + 2 * c + (k & 1);
-                const int64_t gr = row0 + r0 + g + 8 * (k >> 1);
-                if (col < n_out && gr < a.rows) a.logp[gr * n_out + col] = lp[nt][k];
-            }
-    }
-    if (!a.partial) return;
-    // ---- training: dL/dlogp, through log-softmax, then back through the layers
-    float lsum = 0.f;
-    {
-        float gsum[2] = {0.f, 0.f};
-        float gv[4][4];
-        for (int nt = 0; nt < 4; nt++)
-            for (int k = 0; k < 4; k++) {
-                const int col = 8 * nt + 2 * c + (k & 1);
-                const int64_t gr = row0 + r0 + g + 8 * (k >> 1);
-                float gg = 0.f;
-                if (col < n_out && gr < a.rows) {
-                    const int64_t src = a.index ? a.index[gr] : gr;
-                    const float y = a.Y[src * n_out + col];
-                    if (y >= kFracMin) {
-                        const float d = lp[nt][k] - logf(y);
-                        lsum += d * d;
-                        gg = 2.f * d * a.inv_count;
-                    }
+        // output layer and log-softmax, the first four warps; lanes 4g..4g+3 hold rows r0+g
+        // and r0+g+8
+        if (warp < 4) {
+            float z[4][4];
+            float lp[4][4];
+            {
+                float acc[4][4];
+                if (npad == 16) {
+                    float a2[2][4];
+                    warp_gemm<8, 2, false, false>(&S.h3[r0][0], kLd, &S.w4[0][0], kLd, a2);
+                    for (int nt = 0; nt < 4; nt++)
+                        for (int k = 0; k < 4; k++) acc[nt][k] = nt < 2 ? a2[nt][k] : 0.f;
+                } else {
+                    warp_gemm<8, 4, false, false>(&S.h3[r0][0], kLd, &S.w4[0][0], kLd, acc);
                 }
-                gv[nt][k] = gg;
-                gsum[k >> 1] += gg;
+                float mx[2] = {-INFINITY, -INFINITY};
+                for (int nt = 0; nt < 4; nt++)
+                    for (int k = 0; k < 4; k++) {
+                        const int col = 8 * nt + 2 * c + (k & 1);
+                        z[nt][k] = col < n_out ? acc[nt][k] + th[a.L.b4 + col] : -INFINITY;
+                        mx[k >> 1] = fmaxf(mx[k >> 1], z[nt][k]);
+                    }
+                for (int s = 0; s < 2; s++) {
+                    mx[s] = fmaxf(mx[s], __shfl_xor_sync(0xffffffffu, mx[s], 1));
+                    mx[s] = fmaxf(mx[s], __shfl_xor_sync(0xffffffffu, mx[s], 2));
+                }
+                float se[2] = {0.f, 0.f};
+                for (int nt = 0; nt < 4; nt++)
+                    for (int k = 0; k < 4; k++)
+                        se[k >> 1] += (z[nt][k] == -INFINITY) ? 0.f : expf(z[nt][k] - mx[k >> 1]);
+                for (int s = 0; s < 2; s++) {
+                    se[s] += __shfl_xor_sync(0xffffffffu, se[s], 1);
+                    se[s] += __shfl_xor_sync(0xffffffffu, se[s], 2);
+                }
+                for (int nt = 0; nt < 4; nt++)
+                    for (int k = 0; k < 4; k++) lp[nt][k] = z[nt][k] - mx[k >> 1] - logf(se[k >> 1]);
             }
-        for (int s = 0; s < 2; s++) {
-            gsum[s] += __shfl_xor_sync(0xffffffffu, gsum[s], 1);
-            gsum[s] += __shfl_xor_sync(0xffffffffu, gsum[s], 2);
-        }
-        for (int nt = 0; nt < 4; nt++)
-            for (int k = 0; k < 4; k++) {
-                const int col = 8 * nt + 2 * c + (k & 1);
-                const float dzv = col < n_out ? gv[nt][k] - expf(lp[nt][k]) * gsum[k >> 1] : 0.f;
-                if (col < npad) S.dz[r0 + g + 8 * (k >> 1)][col] = __float2bfloat16(dzv);
+            if (a.logp) {
+                for (int nt = 0; nt < 4; nt++)
+                    for (int k = 0; k < 4; k++) {
+                        const int col = 8 * nt + 2 * c + (k & 1);
+                        const int64_t gr = row0 + r0 + g + 8 * (k >> 1);
+                        if (col < n_out && gr < a.rows) a.logp[gr * n_out + col] = lp[nt][k];
+                    }
             }
-    }
-    for (int d = 16; d; d >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, d);
-    if (lane == 0) S.loss[warp] = lsum;
-    __syncwarp();
-    {   // dh3 = (dz W4^T) masked by h3 > 0; B^T is W4 stored [128][npad]
-        float acc[16][4];
-        if (npad == 16) warp_gemm<1, 16>(&S.dz[r0][0], kMaxOut, a.w.W4, npad, acc);
-        else warp_gemm<2, 16>(&S.dz[r0][0], kMaxOut, a.w.W4, npad, acc);
-        store_masked<16>(acc, S.h3, S.da, r0);
-        __syncwarp();
-        warp_gemm<8, 16>(&S.da[r0][0], kHid, a.w.W3, kHid, acc);     // dh2 = dh3 W3^T, masked
-        store_masked<16>(acc, S.h2, S.db, r0);
-        __syncwarp();
-    }
-    __syncthreads();
-    float *P = a.partial + (size_t)blockIdx.x * (a.L.total + 1);
-    // weight gradients of layers 4 and 3 (need dz, h3, dh3 = da, h2)
-    {
-        for (int t = threadIdx.x; t < kHid * n_out; t += blockDim.x) {
-            const int i = t / n_out, j = t - i * n_out;
+            if (a.partial) {
+                // dL/dlogp, through log-softmax
+                const int cnt = *a.count;
+                const float inv_count = cnt ? 1.f / (float)cnt : 0.f;
+                float lsum = 0.f;
+                float gsum[2] = {0.f, 0.f};
+                float gv[4][4];
+                for (int nt = 0; nt < 4; nt++)
+                    for (int k = 0; k < 4; k++) {
+                        const int col = 8 * nt + 2 * c + (k & 1);
+                        const int64_t gr = row0 + r0 + g + 8 * (k >> 1);
+                        float gg = 0.f;
+                        if (col < n_out && gr < a.rows) {
+                            const int64_t src = a.index ? a.index[gr] : gr;
+                            const float y = a.Y[src * n_out + col];
+                            if (y >= kFracMin) {
+                                const float d = lp[nt][k] - logf(y);
+                                lsum += d * d;
+                                gg = 2.f * d * inv_count;
+                            }
+                        }
+                        gv[nt][k] = gg;
+                        gsum[k >> 1] += gg;
+                    }
+                for (int s = 0; s < 2; s++) {
+                    gsum[s] += __shfl_xor_sync(0xffffffffu, gsum[s], 1);
+                    gsum[s] += __shfl_xor_sync(0xffffffffu, gsum[s], 2);
+                }
+                for (int nt = 0; nt < 4; nt++)
+                    for (int k = 0; k < 4; k++) {
+                        const int col = 8 * nt + 2 * c + (k & 1);
+                        const float dzv = col < n_out ? gv[nt][k] - expf(lp[nt][k]) * gsum[k >> 1] : 0.f;
+                        S.dz[r0 + g + 8 * (k >> 1)][col] = __float2bfloat16(dzv);
+                    }
+                for (int d = 16; d; d >>= 1) lsum += __shfl_xor_sync(0xffffffffu, lsum, d);
+                if (lane == 0) S.loss[warp] = lsum;
+            }
+        }
+        __syncthreads();
+        if (!a.partial) continue;
+        // ---- training: back through the layers
+        {   // dh3 = (dz W4^T) masked by h3 > 0; dh2 = (dh3 W3^T) masked by h2 > 0
+            float acc[4][4];
+            if (npad == 16) warp_gemm<1, 4, false, true>(&S.dz[r0][0], kLdz, &S.w4[0][c0], kLd, acc);
+            else warp_gemm<2, 4, false, true>(&S.dz[r0][0], kLdz, &S.w4[0][c0], kLd, acc);
+            store_masked<4>(acc, S.h3, S.da, r0, c0);
+            __syncthreads();
+            warp_gemm<8, 4, false, true>(&S.da[r0][0], kLd, &S.w3[0][c0], kLd, acc);
+            store_masked<4>(acc, S.h2, S.db, r0, c0);
+        }
+        __syncthreads();
+        float *P = a.partial + (size_t)tile * partial_stride(a.L);
+        // weight gradients of layers 4 and 3 (need dz, h3, dh3 = da, h2)
+        if (warp < 8) {
+            if (npad == 16) weight_grad<2>(&S.h3[0][0], &S.dz[0][0], kLdz, 16 * warp, 0, n_out, P + a.L.W4);
+            else weight_grad<4>(&S.h3[0][0], &S.dz[0][0], kLdz, 16 * warp, 0, n_out, P + a.L.W4);
+        } else {
+            for (int j = threadIdx.x - 256; j < n_out + kHid; j += 256) {
+                float s = 0.f;
+                if (j < n_out)
+                    for (int r = 0; r < kRows; r++) s += __bfloat162float(S.dz[r][j]);
+                else
+                    for (int r = 0; r < kRows; r++) s += __bfloat162float(S.da[r][j - n_out]);
+                P[j < n_out ? a.L.b4 + j : a.L.b3 + j - n_out] = s;
+            }
+        }
+        for (int q = 0; q < 2; q++)
+            weight_grad<4>(&S.h2[0][0], &S.da[0][0], kLd, 16 * (2 * (warp & 3) + q), c0, kHid, P + a.L.W3);
+        __syncthreads();
+        {   // dh1 = dh2 W2^T, masked by h1 > 0 (into da, which is free now)
+            float acc[4][4];
+            warp_gemm<8, 4, false, true>(&S.db[r0][0], kLd, &S.w2[0][c0], kLd, acc);
+            store_masked<4>(acc, S.h1, S.da, r0, c0);
+        }
+        __syncthreads();
+        for (int q = 0; q < 2; q++)
+            weight_grad<4>(&S.h1[0][0], &S.db[0][0], kLd, 16 * (2 * (warp & 3) + q), c0, kHid, P + a.L.W2);
+        for (int t = threadIdx.x; t < (kIn + 2) * kHid; t += kTileThreads) {
+            const int i = t / kHid, j = t - i * kHid;
             float s = 0.f;
-            for (int r = 0; r < kRows; r++) s += __bfloat162float(S.h3[r][i]) * __bfloat162float(S.dz[r][j]);
-            P[a.L.W4 + t] = s;
+            if (i < kIn) {
+                for (int r = 0; r < kRows; r++) s += S.x[r][i] * __bfloat162float(S.da[r][j]);
+                P[a.L.W1 + t] = s;
+            } else if (i == kIn) {
+                for (int r = 0; r < kRows; r++) s += __bfloat162float(S.db[r][j]);
+                P[a.L.b2 + j] = s;
+            } else {
+                for (int r = 0; r < kRows; r++) s += __bfloat162float(S.da[r][j]);
+                P[a.L.b1 + j] = s;
+            }
         }
-        for (int j = threadIdx.x; j < n_out; j += blockDim.x) {
-            float s = 0.f;
-            for (int r = 0; r < kRows; r++) s += __bfloat162float(S.dz[r][j]);
-            P[a.L.b4 + j] = s;
-        }
-        weight_grad(S.h2, S.da, kRows, kHid, kHid, P + a.L.W3, nullptr);
-        for (int j = threadIdx.x; j < kHid; j += blockDim.x) {
-            float s = 0.f;
-            for (int r = 0; r < kRows; r++) s += __bfloat162float(S.da[r][j]);
-            P[a.L.b3 + j] = s;
-        }
+        if (threadIdx.x == 0) P[a.L.total] = S.loss[0] + S.loss[1] + S.loss[2] + S.loss[3];
+        __syncthreads();
     }
-    __syncthreads();
-    {   // dh1 = dh2 W2^T, masked by h1 > 0 (into da, which is free now)
-        float acc[16][4];
-        warp_gemm<8, 16>(&S.db[r0][0], kHid, a.w.W2, kHid, acc);
-        store_masked<16>(acc, S.h1, S.da, r0);
-    }
-    __syncthreads();
-    weight_grad(S.h1, S.db, kRows, kHid, kHid, P + a.L.W2, nullptr);
-    for (int j = threadIdx.x; j < kHid; j += blockDim.x) {
-        float s = 0.f, s1 = 0.f;
-        for (int r = 0; r < kRows; r++) {
-            s += __bfloat162float(S.db[r][j]);
-            s1 += __bfloat162float(S.da[r][j]);
-        }
-        P[a.L.b2 + j] = s;
-        P[a.L.b1 + j] = s1;
-    }
-    for (int t = threadIdx.x; t < kIn * kHid; t += blockDim.x) {
-        const int i = t / kHid, j = t - i * kHid;
-        float s = 0.f;
-        for (int r = 0; r < kRows; r++) s += S.x[r][i] * __bfloat162float(S.da[r][j]);
-        P[a.L.W1 + t] = s;
-    }
-    if (threadIdx.x == 0) P[a.L.total] = S.loss[0] + S.loss[1] + S.loss[2] + S.loss[3];
 }
 
-__global__ void k_grad_reduce(const float *partial, int nblk, int64_t stride, float *grad, double *loss) {
+// Targets of at least kFracMin among the rows of a batch, into *count (zeroed before).
+__global__ void k_count(int64_t rows, int n_out, const float *Y, const int32_t *index, int *count) {
+    int n = 0;
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < rows * n_out; t += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t r = t / n_out;
+        n += Y[(index ? (int64_t)index[r] : r) * n_out + (t - r * n_out)] >= kFracMin;
+    }
+    n = __reduce_add_sync(0xffffffffu, n);
+    if ((threadIdx.x & 31) == 0 && n) atomicAdd(count, n);
+}
+
+__global__ void __launch_bounds__(64) k_grad_reduce(const float *__restrict__ partial, int nblk, int64_t stride,
+                                                      int64_t total, float *grad, double *loss) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= stride) return;
+    if (t > total) return;
     double s = 0.0;
+#pragma unroll 16
     for (int b = 0; b < nblk; b++) s += (double)partial[(size_t)b * stride + t];
-    if (t == stride - 1) *loss = s;
+    if (t == total) *loss = s;
     else grad[t] = (float)s;
 }
 
@@ -462,6 +539,13 @@ struct mg_mlp {
     float mean[kIn] = {0, 0, 0, 0}, istd[kIn] = {1, 1, 1, 1};
     int64_t step = 0;
     std::string err;
+    // workspace of loss_grad and train, which own the network while they run: inputs, targets,
+    // row indices, per-CTA partials, losses and target counts (kept up to 256 MB each)
+    float *wX = nullptr, *wY = nullptr, *wP = nullptr;
+    int32_t *wI = nullptr;
+    double *wL = nullptr;
+    int *wC = nullptr;
+    size_t cX = 0, cY = 0, cP = 0, cI = 0, cL = 0, cC = 0;
 };
 
 static int mfail(mg_mlp *p, int code, const std::string &msg) {
@@ -525,6 +609,7 @@ extern "C" int mg_mlp_destroy(mg_mlp *p) {
     if (!p) return MG_OK;
     cudaSetDevice(p->device);
     if (p->stream) cudaStreamSynchronize(p->stream);
+    cudaFree(p->wX); cudaFree(p->wY); cudaFree(p->wP); cudaFree(p->wI); cudaFree(p->wL); cudaFree(p->wC);
     cudaFree(p->theta); cudaFree(p->m); cudaFree(p->v); cudaFree(p->grad); cudaFree(p->wbuf);
     if (p->stream) cudaStreamDestroy(p->stream);
     delete p;
@@ -571,19 +656,21 @@ extern "C" int mg_mlp_set_normalisation(mg_mlp *p, const float *mean, const floa
 }
 
 static TileArgs tile_args(mg_mlp *p, int64_t rows, const float *X, const int32_t *index, const float *Y, float *logp,
-                          float *partial, float inv_count) {
+                          float *partial, const int *count) {
     TileArgs a{};
     a.rows = rows; a.X = X; a.index = index; a.Y = Y; a.theta = p->theta; a.w = p->w; a.L = p->L;
     for (int i = 0; i < kIn; i++) { a.mean[i] = p->mean[i]; a.istd[i] = p->istd[i]; }
-    a.inv_count = inv_count; a.logp = logp; a.partial = partial;
+    a.count = count; a.logp = logp; a.partial = partial;
     return a;
 }
 
 static int launch_tile(mg_mlp *p, const TileArgs &a) {
-    const int64_t blocks = (a.rows + kRows - 1) / kRows;
+    int64_t blocks = (a.rows + kRows - 1) / kRows;
+    // without gradients one CTA per SM takes several tiles
+    if (!a.partial) blocks = std::min<int64_t>(blocks, 152);
     const size_t sm = sizeof(TileSmem);
     cudaFuncSetAttribute(k_mlp_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    k_mlp_tile<<<(unsigned)blocks, 128, sm, p->stream>>>(a);
+    k_mlp_tile<<<(unsigned)blocks, kTileThreads, sm, p->stream>>>(a);
     M_CUDA(cudaGetLastError());
     return MG_OK;
 }
@@ -592,19 +679,45 @@ static int launch_tile(mg_mlp *p, const TileArgs &a) {
 int mg_mlp_forward_dev(mg_mlp *p, int64_t rows, const float *d_X, float *d_logp, cudaStream_t s) {
     cudaStream_t keep = p->stream;
     p->stream = s;
-    int rc = launch_tile(p, tile_args(p, rows, d_X, nullptr, nullptr, d_logp, nullptr, 0.f));
+    int rc = launch_tile(p, tile_args(p, rows, d_X, nullptr, nullptr, d_logp, nullptr, nullptr));
     p->stream = keep;
+    return rc;
+}
+
+// Grows a workspace buffer. (Buffers larger than 256 MB are not kept: see release.)
+template <typename T>
+static int reserve(mg_mlp *p, T *&buf, size_t &cap, size_t count) {
+    if (cap >= count) return MG_OK;
+    cudaFree(buf);
+    buf = nullptr;
+    cap = 0;
+    M_CUDA(cudaMalloc(&buf, sizeof(T) * count));
+    cap = count;
+    return MG_OK;
+}
+template <typename T>
+static void release(T *&buf, size_t &cap) {
+    if (sizeof(T) * cap <= (256u << 20)) return;
+    cudaFree(buf);
+    buf = nullptr;
+    cap = 0;
+}
+static int done(mg_mlp *p, int rc) {
+    release(p->wX, p->cX);
+    release(p->wY, p->cY);
+    release(p->wP, p->cP);
+    release(p->wI, p->cI);
     return rc;
 }
 
 extern "C" int mg_mlp_forward(mg_mlp *p, int64_t rows, const float *X, float *logp) {
     if (!p || rows < 1 || !X || !logp) return MG_ERR_ARG;
     cudaSetDevice(p->device);
-    float *dX = nullptr, *dL = nullptr;
+    float *dX = nullptr, *dL = nullptr;   // (not the workspace: threads may share a network's forward pass)
     M_CUDA(cudaMalloc(&dX, 16 * rows));
     M_CUDA(cudaMalloc(&dL, 4 * rows * p->L.n_out));
     M_CUDA(cudaMemcpyAsync(dX, X, 16 * rows, cudaMemcpyHostToDevice, p->stream));
-    int rc = launch_tile(p, tile_args(p, rows, dX, nullptr, nullptr, dL, nullptr, 0.f));
+    int rc = launch_tile(p, tile_args(p, rows, dX, nullptr, nullptr, dL, nullptr, nullptr));
     if (!rc) {
         M_CUDA(cudaMemcpyAsync(logp, dL, 4 * rows * p->L.n_out, cudaMemcpyDeviceToHost, p->stream));
         M_CUDA(cudaStreamSynchronize(p->stream));
@@ -614,51 +727,92 @@ extern "C" int mg_mlp_forward(mg_mlp *p, int64_t rows, const float *X, float *lo
     return rc;
 }
 
-// One gradient evaluation over device rows (index optional); leaves grad in p->grad.
-static int grad_dev(mg_mlp *p, int64_t rows, const float *dX, const int32_t *didx, const float *dY, float inv_count,
-                    float *dpart, double *dloss) {
-    const int64_t blocks = (rows + kRows - 1) / kRows;
-    int rc = launch_tile(p, tile_args(p, rows, dX, didx, dY, nullptr, dpart, inv_count));
+// One gradient evaluation over device rows (index optional); leaves grad in p->grad, the sum
+// of squares in *dloss and the number of targets in *dcount.
+static int grad_dev(mg_mlp *p, int64_t rows, const float *dX, const int32_t *didx, const float *dY, float *dpart,
+                    double *dloss, int *dcount) {
+    const int64_t blocks = (rows + kRows - 1) / kRows, m = rows * p->L.n_out;
+    M_CUDA(cudaMemsetAsync(dcount, 0, sizeof(int), p->stream));
+    k_count<<<(unsigned)std::min<int64_t>(304, (m + 1023) / 1024), 256, 0, p->stream>>>(rows, p->L.n_out, dY, didx, dcount);
+    int rc = launch_tile(p, tile_args(p, rows, dX, didx, dY, nullptr, dpart, dcount));
     if (rc) return rc;
-    const int64_t stride = p->L.total + 1;
-    k_grad_reduce<<<(unsigned)((stride + 255) / 256), 256, 0, p->stream>>>(dpart, (int)blocks, stride, p->grad, dloss);
+    k_grad_reduce<<<(unsigned)(p->L.total / 64 + 1), 64, 0, p->stream>>>(dpart, (int)blocks, partial_stride(p->L),
+                                                                       p->L.total, p->grad, dloss);
     M_CUDA(cudaGetLastError());
     return MG_OK;
 }
 
-static float count_inv(const float *Y, int64_t rows, int n_out, const std::vector<int32_t> *idx, int64_t start) {
-    int64_t cnt = 0;
-    for (int64_t r = 0; r < rows; r++) {
-        const int64_t src = idx ? (*idx)[start + r] : start + r;
-        for (int j = 0; j < n_out; j++) cnt += Y[src * n_out + j] >= kFracMin;
-    }
-    return cnt ? 1.f / (float)cnt : 0.f;
+static int loss_grad_host(mg_mlp *p, int64_t rows, const float *X, const float *Y, double *loss, float *grad) {
+    const int n_out = p->L.n_out;
+    const int64_t blocks = (rows + kRows - 1) / kRows, stride = partial_stride(p->L);
+    int rc;
+    if ((rc = reserve(p, p->wX, p->cX, 4 * rows)) || (rc = reserve(p, p->wY, p->cY, rows * n_out)) ||
+        (rc = reserve(p, p->wP, p->cP, blocks * stride)) || (rc = reserve(p, p->wL, p->cL, 1)) ||
+        (rc = reserve(p, p->wC, p->cC, 1)))
+        return rc;
+    M_CUDA(cudaMemcpyAsync(p->wX, X, 16 * rows, cudaMemcpyHostToDevice, p->stream));
+    M_CUDA(cudaMemcpyAsync(p->wY, Y, 4 * rows * n_out, cudaMemcpyHostToDevice, p->stream));
+    if ((rc = grad_dev(p, rows, p->wX, nullptr, p->wY, p->wP, p->wL, p->wC))) return rc;
+    double lsum = 0.0;
+    int cnt = 0;
+    if (grad) M_CUDA(cudaMemcpyAsync(grad, p->grad, 4 * p->L.total, cudaMemcpyDeviceToHost, p->stream));
+    M_CUDA(cudaMemcpyAsync(&lsum, p->wL, 8, cudaMemcpyDeviceToHost, p->stream));
+    M_CUDA(cudaMemcpyAsync(&cnt, p->wC, 4, cudaMemcpyDeviceToHost, p->stream));
+    M_CUDA(cudaStreamSynchronize(p->stream));
+    if (loss) *loss = lsum * (cnt ? 1.f / (float)cnt : 0.f);
+    return MG_OK;
 }
 
 extern "C" int mg_mlp_loss_grad(mg_mlp *p, int64_t rows, const float *X, const float *Y, double *loss, float *grad) {
     if (!p || rows < 1 || !X || !Y) return MG_ERR_ARG;
     cudaSetDevice(p->device);
+    return done(p, loss_grad_host(p, rows, X, Y, loss, grad));
+}
+
+static int train_host(mg_mlp *p, int64_t rows, const float *X, const float *Y, const mg_train_opts *o,
+                      mg_train_report &r) {
     const int n_out = p->L.n_out;
-    const int64_t blocks = (rows + kRows - 1) / kRows, stride = p->L.total + 1;
-    float *dX = nullptr, *dY = nullptr, *dP = nullptr;
-    double *dl = nullptr;
-    M_CUDA(cudaMalloc(&dX, 16 * rows));
-    M_CUDA(cudaMalloc(&dY, 4 * rows * n_out));
-    M_CUDA(cudaMalloc(&dP, 4 * blocks * stride));
-    M_CUDA(cudaMalloc(&dl, 8));
-    M_CUDA(cudaMemcpyAsync(dX, X, 16 * rows, cudaMemcpyHostToDevice, p->stream));
-    M_CUDA(cudaMemcpyAsync(dY, Y, 4 * rows * n_out, cudaMemcpyHostToDevice, p->stream));
-    const float ic = count_inv(Y, rows, n_out, nullptr, 0);
-    int rc = grad_dev(p, rows, dX, nullptr, dY, ic, dP, dl);
-    double lsum = 0.0;
-    if (!rc) {
-        if (grad) M_CUDA(cudaMemcpyAsync(grad, p->grad, 4 * p->L.total, cudaMemcpyDeviceToHost, p->stream));
-        M_CUDA(cudaMemcpyAsync(&lsum, dl, 8, cudaMemcpyDeviceToHost, p->stream));
+    const int64_t B = o->batch, stride = partial_stride(p->L), blocks = (B + kRows - 1) / kRows;
+    const int64_t steps = std::max<int64_t>(1, rows / B);   // per epoch
+    int rc;
+    if ((rc = reserve(p, p->wX, p->cX, 4 * rows)) || (rc = reserve(p, p->wY, p->cY, rows * n_out)) ||
+        (rc = reserve(p, p->wI, p->cI, rows)) || (rc = reserve(p, p->wP, p->cP, blocks * stride)) ||
+        (rc = reserve(p, p->wL, p->cL, steps)) || (rc = reserve(p, p->wC, p->cC, steps)))
+        return rc;
+    M_CUDA(cudaMemcpyAsync(p->wX, X, 16 * rows, cudaMemcpyHostToDevice, p->stream));
+    M_CUDA(cudaMemcpyAsync(p->wY, Y, 4 * rows * n_out, cudaMemcpyHostToDevice, p->stream));
+    std::vector<int32_t> idx(rows);
+    std::vector<double> lsum(steps);
+    std::vector<int> cnt(steps);
+    std::mt19937_64 rng(o->seed);
+    for (int ep = 0; ep < o->epochs; ep++) {
+        for (int64_t i = 0; i < rows; i++) idx[i] = (int32_t)i;
+        std::shuffle(idx.begin(), idx.end(), rng);
+        M_CUDA(cudaMemcpyAsync(p->wI, idx.data(), 4 * rows, cudaMemcpyHostToDevice, p->stream));
+        int64_t nb = 0;
+        for (int64_t s = 0; s + B <= rows || (s == 0 && rows < B); s += B, nb++) {
+            const int64_t nr = std::min<int64_t>(B, rows - s);
+            if ((rc = grad_dev(p, nr, p->wX, p->wI + s, p->wY, p->wP, p->wL + nb, p->wC + nb))) return rc;
+            p->step++;
+            const float c1 = 1.f - std::pow(0.9f, (float)p->step), c2 = 1.f - std::pow(0.999f, (float)p->step);
+            k_adam<<<(unsigned)((p->L.total + 255) / 256), 256, 0, p->stream>>>(p->theta, p->m, p->v, p->grad,
+                                                                                 p->L.total, o->lr, 0.9f, 0.999f,
+                                                                                 1e-8f, c1, c2);
+            refresh(p);
+            r.steps++;
+        }
+        // the epoch's losses (and the indices' buffer is free for the next shuffle)
+        M_CUDA(cudaMemcpyAsync(lsum.data(), p->wL, 8 * nb, cudaMemcpyDeviceToHost, p->stream));
+        M_CUDA(cudaMemcpyAsync(cnt.data(), p->wC, 4 * nb, cudaMemcpyDeviceToHost, p->stream));
         M_CUDA(cudaStreamSynchronize(p->stream));
-        if (loss) *loss = lsum * ic;
+        double ep_loss = 0.0;
+        for (int64_t k = 0; k < nb; k++) ep_loss += lsum[k] * (cnt[k] ? 1.f / (float)cnt[k] : 0.f);
+        if (nb) {
+            if (r.first_loss < 0) r.first_loss = ep_loss / nb;
+            r.last_loss = ep_loss / nb;
+        }
     }
-    cudaFree(dX); cudaFree(dY); cudaFree(dP); cudaFree(dl);
-    return rc;
+    return MG_OK;
 }
 
 extern "C" int mg_mlp_train(mg_mlp *p, int64_t rows, const float *X, const float *Y, const mg_train_opts *o,
@@ -666,52 +820,9 @@ extern "C" int mg_mlp_train(mg_mlp *p, int64_t rows, const float *X, const float
     if (!p || rows < 1 || !X || !Y || !o || o->epochs < 1 || o->batch < kRows || !(o->lr > 0)) return MG_ERR_ARG;
     cudaSetDevice(p->device);
     auto t0 = std::chrono::steady_clock::now();
-    const int n_out = p->L.n_out;
-    const int64_t B = o->batch, stride = p->L.total + 1, blocks = (B + kRows - 1) / kRows;
-    float *dX = nullptr, *dY = nullptr, *dP = nullptr;
-    int32_t *dI = nullptr;
-    double *dl = nullptr;
-    M_CUDA(cudaMalloc(&dX, 16 * rows));
-    M_CUDA(cudaMalloc(&dY, 4 * rows * n_out));
-    M_CUDA(cudaMalloc(&dI, 4 * rows));
-    M_CUDA(cudaMalloc(&dP, 4 * blocks * stride));
-    M_CUDA(cudaMalloc(&dl, 8));
-    M_CUDA(cudaMemcpyAsync(dX, X, 16 * rows, cudaMemcpyHostToDevice, p->stream));
-    M_CUDA(cudaMemcpyAsync(dY, Y, 4 * rows * n_out, cudaMemcpyHostToDevice, p->stream));
-    std::vector<int32_t> idx(rows);
-    std::mt19937_64 rng(o->seed);
     mg_train_report r{};
     r.first_loss = -1;
-    int rc = MG_OK;
-    for (int ep = 0; ep < o->epochs && !rc; ep++) {
-        for (int64_t i = 0; i < rows; i++) idx[i] = (int32_t)i;
-        std::shuffle(idx.begin(), idx.end(), rng);
-        M_CUDA(cudaMemcpyAsync(dI, idx.data(), 4 * rows, cudaMemcpyHostToDevice, p->stream));
-        double ep_loss = 0.0;
-        int64_t nb = 0;
-        for (int64_t s = 0; s + B <= rows || (s == 0 && rows < B); s += B) {
-            const int64_t nr = std::min<int64_t>(B, rows - s);
-            const float ic = count_inv(Y, nr, n_out, &idx, s);
-            if ((rc = grad_dev(p, nr, dX, dI + s, dY, ic, dP, dl))) break;
-            p->step++;
-            const float c1 = 1.f - std::pow(0.9f, (float)p->step), c2 = 1.f - std::pow(0.999f, (float)p->step);
-            k_adam<<<(unsigned)((p->L.total + 255) / 256), 256, 0, p->stream>>>(p->theta, p->m, p->v, p->grad,
-                                                                                 p->L.total, o->lr, 0.9f, 0.999f,
-                                                                                 1e-8f, c1, c2);
-            refresh(p);
-            double lsum = 0.0;
-            cudaMemcpyAsync(&lsum, dl, 8, cudaMemcpyDeviceToHost, p->stream);
-            cudaStreamSynchronize(p->stream);
-            ep_loss += lsum * ic;
-            nb++;
-            r.steps++;
-        }
-        if (nb) {
-            if (r.first_loss < 0) r.first_loss = ep_loss / nb;
-            r.last_loss = ep_loss / nb;
-        }
-    }
-    cudaFree(dX); cudaFree(dY); cudaFree(dI); cudaFree(dP); cudaFree(dl);
+    const int rc = done(p, train_host(p, rows, X, Y, o, r));
     r.seconds = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
     if (rep) *rep = r;
     return rc;
