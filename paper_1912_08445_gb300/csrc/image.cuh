@@ -56,9 +56,9 @@ struct ImgStage64 {
 constexpr int kImgPairs = 64;
 template <int NOV>
 struct ImgStage32 {
-    float4 g[NOV][kImgPairs];    // (gz, gz, ngy, ngy)
-    float4 x[NOV][kImgPairs];    // (X, X, S, S); NOV > 1: emissivity in place of S
-    float4 y[kImgPairs];         // (emissivity over chi_min, twice; h, h)
+    float4 g[NOV][kImgPairs];    // (gz, gz, ngy, ngy): x' = u gz + ngy
+    float4 x[NOV][kImgPairs];    // (eta, eta, chi, chi)
+    float4 y[kImgPairs];         // (1/b, 1/b, h, h)
 };
 
 // Lists a channel's points of a staged chunk of cnt (from `nearby(j)`, whether point j is near):
@@ -355,7 +355,7 @@ __global__ void __launch_bounds__(256) k_image64_lines(ImageArgs a, int skip, in
 }
 
 // FP32 (mixed-precision contexts), from the FP32 ray store, widths and line data. Here the
-// issue rate bounds it (two ex2 and a rcp per point and channel, ~25 instructions), and walking
+// issue rate bounds it (two ex2 and two rcp per point and channel, ~25 instructions), and walking
 // lists costs more than it saves: every channel goes through every point, two points at a
 // time in packed FP32x2 arithmetic; only the intensity itself is a chain (three FMAs a
 // point). The first point of the pair and one that fills up the last pair have dtau = 0,
@@ -403,14 +403,16 @@ __global__ void __launch_bounds__(256) k_image32_lines(ImageArgs a) {
             __syncthreads();
             for (int t = threadIdx.x; t < 2 * np2; t += blockDim.x) {
                 const int k = k0 + t, pr = t >> 1, odd = t & 1;
-                float h = 0.0f, E0 = 0.0f;
+                float h = 0.0f, ib = 0.0f;
                 if (k < K) {
                     const ImgPoint q = img_point(s, o, ofb, ofl, lb, lf, Kb, k);
                     float wt = 0.0f, w = nvo, b;
                     if (q.x < 0) {
                         b = a.bf[o];
                     } else {
-                        wt = q.j == q.np ? 1.0f : __fdividef((float)q.j, (float)q.np);
+                        // (at the element's own cell, j = np, this can fall one rounding short of 1, so
+                        // that a neighbour 1e7 times denser shows through at that point)
+                        wt = (float)q.j * (1.0f / (float)q.np);
                         const float pv = q.e ? a.vparf[q.off + q.e - 1] : 0.0f;
                         w += q.sgn * ((1.0f - wt) * pv + wt * a.vparf[q.off + q.e]);
                         b = (1.0f - wt) * a.bf[q.p] + wt * a.bf[q.c];
@@ -422,19 +424,17 @@ __global__ void __launch_bounds__(256) k_image32_lines(ImageArgs a) {
                     } else {
                         far_w = w;
                     }
-                    const float ib = 1.0f / b, pz = ks * ib, gy = w * pz, gz = pz - gy * kic;
+                    ib = 1.0f / b;
+                    const float pz = ks * ib, gy = w * pz, gz = pz - gy * kic;
 #pragma unroll
                     for (int i = 0; i < NOV; i++) {
                         const float2 p0 = reinterpret_cast<const float2 *>(a.linef)[(int64_t)q.p * s.L + a.lf[i].l2];
                         const float2 p1 = reinterpret_cast<const float2 *>(a.linef)[(int64_t)q.c * s.L + a.lf[i].l2];
-                        const float et = (1.0f - wt) * p0.x + wt * p1.x, ch = (1.0f - wt) * p0.y + wt * p1.y;
-                        const float nrm = a.lf[i].nrm * ib;
                         float *g = &T.g[i][pr].x + odd, *x = &T.x[i][pr].x + odd;
                         g[0] = a.lf[i].rat * gz;
                         g[2] = a.lf[i].dnl * pz - a.lf[i].rat * gy;
-                        x[0] = fmaxf(ch, 0.0f) * nrm;
-                        x[2] = NOV > 1 ? et * nrm : (ch > 0.0f ? et / ch : 0.0f);
-                        E0 = et * nrm * a.inv_chi_min;
+                        x[0] = (1.0f - wt) * p0.x + wt * p1.x;
+                        x[2] = (1.0f - wt) * p0.y + wt * p1.y;
                     }
                 } else {
 #pragma unroll
@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(256) k_image32_lines(ImageArgs a) {
                     }
                 }
                 float *y = &T.y[pr].x + odd;
-                y[0] = E0;
+                y[0] = ib;
                 y[2] = h;
             }
             __syncthreads();
@@ -459,17 +459,12 @@ __global__ void __launch_bounds__(256) k_image32_lines(ImageArgs a) {
                     const float2 x = __ffma2_rn(u2, make_float2(g.x, g.y), make_float2(g.z, g.w));
                     const float2 xx = __fmul2_rn(x, x);
                     const float2 e = make_float2(ex2(-xx.x), ex2(-xx.y));
-                    if (NOV == 1) {
-                        chi = __fmul2_rn(make_float2(xs.x, xs.y), e);
-                        const float2 fl = __fmul2_rn(make_float2(y.x, y.y), e);
-                        S = make_float2(chi.x < chi_min ? fl.x : xs.z, chi.y < chi_min ? fl.y : xs.w);
-                    } else {
-                        chi = __ffma2_rn(make_float2(xs.x, xs.y), e, chi);
-                        S = __ffma2_rn(make_float2(xs.z, xs.w), e, S);
-                    }
+                    const float2 phi = __fmul2_rn(e, __fmul2_rn(make_float2(y.x, y.y), two(a.lf[i].nrm)));
+                    S = __ffma2_rn(make_float2(xs.x, xs.y), phi, S);         // (the emissivity)
+                    chi = __ffma2_rn(make_float2(xs.z, xs.w), phi, chi);
                 }
                 chi = make_float2(fmaxf(chi.x, chi_min), fmaxf(chi.y, chi_min));
-                if (NOV > 1) S = __fmul2_rn(S, make_float2(rcp(chi.x), rcp(chi.y)));
+                S = __fmul2_rn(S, make_float2(rcp(chi.x), rcp(chi.y)));
                 float2 d = __fmul2_rn(__fadd2_rn(make_float2(chi_prev, chi.x), chi), make_float2(y.z, y.w));
                 // (no floor at the first point of the pair and where a last point is missing)
                 d.x = fmaxf(d.x, k0 + j ? dtau_min : 0.0f);

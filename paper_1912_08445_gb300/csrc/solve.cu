@@ -435,7 +435,7 @@ struct ImageArgs {
     double *I;                // [n][n_ch]
     double *xy;               // [n][2]
     const float *dsf, *vparf, *bf, *linef;   // FP32 copies for the FP32 kernel
-    float nf[3], inv_chi_min;
+    float nf[3];
     struct {                  // the first lines within reach, for the line kernels (image.cuh)
         int32_t l2;
         float rat, dnl, nrm;  // nrm = c/(nu sqrt pi)
@@ -805,7 +805,6 @@ int mg_launch_image(mg_ctx *ctx, int ray, int line, int n_ch, const double *d_u,
     a.dsf = ctx->d_dsf; a.vparf = ctx->d_vparf; a.bf = ctx->d_bf; a.linef = ctx->d_imglf;
     const size_t smem32 = sizeof(float) * (size_t)s.kmax * (3 + 2 * (size_t)n_ov);
     for (int i = 0; i < 3; i++) a.nf[i] = (float)n[i];
-    a.inv_chi_min = (float)(1.0 / s.chi_min);
     for (int i = 0; i < std::min(n_ov, kImgLines); i++) {
         const Overlap &v = h_ov[i];
         const double nu = 1.0 / v.inv_nu2;
