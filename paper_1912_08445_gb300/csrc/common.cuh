@@ -62,6 +62,8 @@ struct mg_ctx {
     int device = 0;
     cudaStream_t own_stream = nullptr;
     cudaStream_t stream = nullptr;
+    bool stream_changed = false;   // since the last trace: work on the rays may run on another stream
+    bool pool_held = false;        // a reference to the device's scratch pool
     mutable std::string err;
 
     // ---- mesh
@@ -123,6 +125,7 @@ struct mg_ctx {
     double *d_ds = nullptr;        // path length from the previous point
     double *d_vpar = nullptr;      // line-of-sight velocity relative to the origin
     float *d_dsf = nullptr, *d_vparf = nullptr;
+    int64_t ray_off_cap = 0, ray_cap[6] = {0, 0, 0, 0, 0, 0};   // elements the buffers hold
     int64_t n_elements = 0, n_expanded = 0, max_pair_len = 0, n_dead = 0;
     int64_t work_solves = 0, work_updates = 0;
 
@@ -232,6 +235,8 @@ struct MgTimed {
 
 // ---------------------------------------------------------------- launchers
 int mg_launch_trace(mg_ctx *ctx);
+void mg_pool_retain(int device);    // the device's scratch pool (trace.cu), one reference per context
+void mg_pool_release(int device);
 int mg_launch_line_data(mg_ctx *ctx);
 int mg_launch_line_data_mixed(mg_ctx *ctx);
 int mg_launch_line_data64(mg_ctx *ctx, float *linef, unsigned long long *neg);

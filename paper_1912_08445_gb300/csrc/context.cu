@@ -87,6 +87,8 @@ extern "C" int mg_create(mg_ctx **out, const mg_options *opt) {
         return MG_ERR_CUDA;
     }
     ctx->stream = ctx->own_stream;
+    mg_pool_retain(ctx->device);
+    ctx->pool_held = true;
     ctx->band_cur = o.alo_band;
     cudaMemset(ctx->d_scal, 0, 8 * sizeof(unsigned long long));
     *out = ctx;
@@ -96,6 +98,8 @@ extern "C" int mg_create(mg_ctx **out, const mg_options *opt) {
 static void free_rays(mg_ctx *ctx) {
     mg_free(ctx->d_ray_off); mg_free(ctx->d_cells); mg_free(ctx->d_xcum); mg_free(ctx->d_ds);
     mg_free(ctx->d_vpar); mg_free(ctx->d_dsf); mg_free(ctx->d_vparf);
+    ctx->ray_off_cap = 0;
+    for (int64_t &c : ctx->ray_cap) c = 0;
     ctx->traced = false;
     ctx->band_geo_ready = false;
 }
@@ -138,6 +142,7 @@ extern "C" int mg_destroy(mg_ctx *ctx) {
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);
     if (ctx->ev1) cudaEventDestroy(ctx->ev1);
     if (ctx->own_stream) cudaStreamDestroy(ctx->own_stream);
+    if (ctx->pool_held) mg_pool_release(ctx->device);
     delete ctx;
     return MG_OK;
 }
@@ -148,7 +153,9 @@ extern "C" const char *mg_last_error(const mg_ctx *ctx) {
 
 extern "C" int mg_set_stream(mg_ctx *ctx, void *stream) {
     if (!ctx) return MG_ERR_ARG;
-    ctx->stream = stream ? (cudaStream_t)stream : ctx->own_stream;
+    const cudaStream_t to = stream ? (cudaStream_t)stream : ctx->own_stream;
+    if (to != ctx->stream) ctx->stream_changed = true;
+    ctx->stream = to;
     return MG_OK;
 }
 

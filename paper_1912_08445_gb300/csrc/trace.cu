@@ -3,6 +3,7 @@
 // the walk (projections, distances, velocity steps) is reproducible bit for bit.
 #include <cmath>
 #include <algorithm>
+#include <mutex>
 #include "common.cuh"
 
 using namespace mg;
@@ -15,6 +16,7 @@ struct TraceArgs {
     int32_t geometry;
     const double *pos, *vel, *b, *dirs;
     const float4 *posf;                // (x, y, z, |x| + |y| + |z|) in FP32, for the filter
+    const float *wmax;                 // largest |x| + |y| + |z|
     const int64_t *nbr_off;
     const int32_t *nbr_idx;
     const uint8_t *bdy;
@@ -26,6 +28,7 @@ struct TraceArgs {
     const int64_t *ray_off;
     int32_t *cells, *xcum;
     double *ds, *vpar;
+    float *dsf, *vparf;                // FP32 copies
     int32_t *err;
     // cells of each half-ray recorded by the count pass: tmp[k * n R + t] for k < cap_tmp
     int32_t *tmp;
@@ -36,9 +39,16 @@ struct TraceArgs {
 // line-of-sight velocity changes by dv > f min(b_a, b_b), ceil(dv/(f min)) - 1 points.
 __device__ __forceinline__ int32_t velocity_inserts(double va, double ba, double vb, double bb, double f) {
     double dv = fabs(vb - va);
-    double wmin = ba < bb ? ba : bb;
+    // (widths are positive: they compare like their bits)
+    double wmin = __double_as_longlong(ba) < __double_as_longlong(bb) ? ba : bb;
     double lim = f * wmin;
-    if (dv > lim) return (int32_t)ceil(dv / lim) - 1;
+    if (dv > lim) {
+        // The FP32 quotient (relative error below 4e-7) decides the ceiling unless it lies that
+        // close to a whole number; an FP64 division costs eight FP64 instructions.
+        const float q = __fdiv_rn((float)dv, (float)lim), near = rintf(q);
+        if (q < 1e6f && fabsf(q - near) > 1e-6f * q) return (int32_t)ceilf(q) - 1;
+        return (int32_t)ceil(dv / lim) - 1;
+    }
     return 0;
 }
 
@@ -57,6 +67,8 @@ __device__ __forceinline__ bool emit(const TraceArgs &a, int64_t base, int32_t &
         a.xcum[base + len] = x;
         a.ds[base + len] = ds;
         a.vpar[base + len] = vp;
+        a.dsf[base + len] = (float)ds;
+        a.vparf[base + len] = (float)vp;
         va = vp;
         ba = bb;
     } else if (a.tmp && len < a.cap_tmp) {
@@ -75,16 +87,31 @@ __device__ __forceinline__ bool emit(const TraceArgs &a, int64_t base, int32_t &
 // is evaluated only where the bound cannot decide:
 // - a candidate is valid when s > s_cur: the FP32 projection decides unless it lies
 //   within its error bound of s_cur, where the FP64 projection decides;
-// - the FP32 squared distance of every valid candidate comes with an interval
-//   [lo, hi] that contains the FP64 value; the FP64 winner's lo is at most the smallest
-//   hi, so every valid candidate with lo <= min hi is evaluated in FP64 and the winner
-//   is chosen among those with the exact tie-breaks. (A non-finite bound leaves the
-//   candidate to FP64.)
+// - the FP32 squared distance d of every valid candidate comes with an error bound Ed(d), so
+//   that the FP64 value lies in [lo, hi] = [d - Ed, d + Ed]. The FP64 winner's lo is at most
+//   the smallest hi, that of the smallest d. The three smallest d are kept: when the
+//   second's lo lies above that hi, the first is the winner; when the third's does, the
+//   first two are evaluated in FP64 and the winner is chosen with the exact tie-breaks;
+//   otherwise every valid candidate with lo <= hi is. (A non-finite d leaves the choice to
+//   the last.)
 // The bounds follow from |fl32(a) - a| <= u|a| (u = 2^-24) for the conversions of the
-// positions and the direction and for each FP32 operation; they are doubled for margin.
-struct Cand32 {
-    bool valid;
-    float lo, hi;   // interval of the FP64 squared distance
+// positions and the direction and for each FP32 operation, with |x|_1 bounded by twice the
+// model's largest (P below); they are doubled for margin. They are the same for every
+// candidate of a walk: bounds per candidate, three times tighter, took more instructions
+// than the distances themselves (20k-point cloud, 960k half-rays: 2.15 ms, now 1.48 ms).
+struct Bounds32 {
+    float margin;          // of |s32 - s_cur|
+    float e1, e0, e2;      // Ed(d) = e1 sqrt(d) + e0 + e2 d
+    __device__ Bounds32(float P) {
+        constexpr float k2u = 1.2e-7f;   // 2u with margin
+        const float Es = k2u * 7.0f * P;                                // |s32 - s64|
+        margin = Es + k2u * 4.0f * P;                                   // and of s_cur and the difference
+        const float Ep = 2.0f * (Es + 0.6e-7f * 8.0f * P);              // |p32 - p64| per component
+        e1 = 1.1f * 2.0f * Ep * 1.7322f;                                // |p|_1 <= sqrt(3 d)
+        e0 = 1.1f * 9.0f * Ep * Ep;
+        e2 = 1.1f * 2.0f * k2u;
+    }
+    __device__ float err(float d) const { return e1 * sqrtf(d) + e0 + e2 * d; }
 };
 
 __device__ __forceinline__ double proj64(const TraceArgs &a, int64_t c, double xo0, double xo1, double xo2,
@@ -95,29 +122,18 @@ __device__ __forceinline__ double proj64(const TraceArgs &a, int64_t c, double x
     return dx * n0 + dy * n1 + dz * n2;
 }
 
-__device__ __forceinline__ Cand32 classify32(const TraceArgs &a, int64_t c, const float4 po, float n0f, float n1f,
-                                             float n2f, float scf, double s_cur, double xo0, double xo1,
-                                             double xo2, double n0, double n1, double n2) {
-    constexpr float k2u = 1.2e-7f;   // 2u with margin
-    const float4 pc = a.posf[c];
+// FP32 squared distance of candidate c from the ray and whether it lies ahead of s_cur.
+__device__ __forceinline__ bool ahead32(const TraceArgs &a, int64_t c, const float4 pc, const float4 po, float n0f,
+                                        float n1f, float n2f, float scf, const Bounds32 &B, double s_cur, double xo0,
+                                        double xo1, double xo2, double n0, double n1, double n2, float &d2) {
     const float dx = pc.x - po.x, dy = pc.y - po.y, dz = pc.z - po.z;
-    const float D = fabsf(dx) + fabsf(dy) + fabsf(dz);
-    const float P = pc.w + po.w;
-    const float sf = dx * n0f + dy * n1f + dz * n2f;
-    const float Es = k2u * (P + 6.0f * D);   // |sf - s64|
+    const float sf = __fmaf_rn(dz, n2f, __fmaf_rn(dy, n1f, dx * n0f));
+    const float px = __fmaf_rn(-sf, n0f, dx), py = __fmaf_rn(-sf, n1f, dy), pz = __fmaf_rn(-sf, n2f, dz);
+    d2 = __fmaf_rn(pz, pz, __fmaf_rn(py, py, px * px));
     const float diff = sf - scf;
-    const float margin = Es + k2u * (fabsf(scf) + fabsf(diff));
-    Cand32 r;
-    if (diff > margin) r.valid = true;
-    else if (diff < -margin) r.valid = false;
-    else r.valid = proj64(a, c, xo0, xo1, xo2, n0, n1, n2) > s_cur;   // inconclusive in FP32
-    const float px = dx - sf * n0f, py = dy - sf * n1f, pz = dz - sf * n2f;
-    const float d2 = px * px + py * py + pz * pz;
-    const float Ep = 2.0f * (Es + 0.6e-7f * (P + 4.0f * D + 3.0f * fabsf(sf)));   // |px - px64| and so on
-    const float Ed = 1.1f * (2.0f * Ep * (fabsf(px) + fabsf(py) + fabsf(pz)) + 9.0f * Ep * Ep + k2u * 2.0f * d2);
-    r.lo = d2 - Ed;
-    r.hi = d2 + Ed;
-    return r;
+    if (diff > B.margin) return true;
+    if (diff < -B.margin) return false;
+    return proj64(a, c, xo0, xo1, xo2, n0, n1, n2) > s_cur;   // inconclusive in FP32
 }
 
 template <bool FILL>
@@ -128,6 +144,7 @@ __device__ void walk_3d(const TraceArgs &a, int64_t o, int r, int64_t base, int3
     const double vo0 = a.vel[3 * o], vo1 = a.vel[3 * o + 1], vo2 = a.vel[3 * o + 2];
     const float n0f = (float)n0, n1f = (float)n1, n2f = (float)n2;
     const float4 po = a.posf[o];
+    const Bounds32 B((*a.wmax + po.w) * 1.0001f);
     int64_t cur = o;
     double s_cur = 0.0;
     double va = 0.0, ba = a.b[o];
@@ -138,47 +155,61 @@ __device__ void walk_3d(const TraceArgs &a, int64_t o, int r, int64_t base, int3
     for (;;) {
         const float scf = (float)s_cur;
         const int64_t e0 = a.nbr_off[cur], e1 = a.nbr_off[cur + 1];
-        // pass 1: validity, the smallest upper bound of a valid candidate's distance, and
-        // the two smallest lower bounds
-        float minhi = INFINITY, lo1 = INFINITY, lo2 = INFINITY;
-        int64_t c1 = -1;
-        bool full = false;   // a bound that is not finite leaves the choice to pass 2
-        for (int64_t e = e0; e < e1; e++) {
-            const int64_t c = a.nbr_idx[e];
-            const Cand32 k = classify32(a, c, po, n0f, n1f, n2f, scf, s_cur, xo0, xo1, xo2, n0, n1, n2);
-            if (!k.valid) continue;
-            if (!(k.lo <= k.hi) || !(fabsf(k.hi) < INFINITY)) full = true;
-            minhi = fminf(minhi, k.hi);
-            if (k.lo < lo1) {
-                lo2 = lo1;
-                lo1 = k.lo;
-                c1 = c;
-            } else if (k.lo < lo2) {
-                lo2 = k.lo;
+        // pass 1: the three smallest FP32 distances among the valid candidates, four
+        // candidates' gathers in flight at a time
+        float d1 = INFINITY, d2 = INFINITY, d3 = INFINITY;
+        int32_t c1 = -1, c2 = -1;
+        bool full = false;   // a distance that is not finite leaves the choice to FP64
+        for (int64_t e = e0; e < e1; e += 4) {
+            int32_t id[4];
+            float4 pc[4];
+#pragma unroll
+            for (int k = 0; k < 4; k++) id[k] = a.nbr_idx[e + k < e1 ? e + k : e0];
+#pragma unroll
+            for (int k = 0; k < 4; k++) pc[k] = a.posf[id[k]];
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                if (e + k >= e1) break;
+                float d;
+                if (!ahead32(a, id[k], pc[k], po, n0f, n1f, n2f, scf, B, s_cur, xo0, xo1, xo2, n0, n1, n2, d)) continue;
+                full = full || !(d < INFINITY);
+                const bool l1 = d < d1, l2 = d < d2;
+                d3 = l2 ? d2 : fminf(d3, d);
+                c2 = l1 ? c1 : (l2 ? id[k] : c2);
+                d2 = l1 ? d1 : (l2 ? d : d2);
+                c1 = l1 ? id[k] : c1;
+                d1 = l1 ? d : d1;
             }
         }
         int64_t best = -1;
         double bs = 0.0, bd2 = 0.0;
-        // Only the candidate with the smallest lower bound reaches min hi: it is the
-        // closest, and only its FP64 projection is needed.
-        const bool unique = c1 >= 0 && !full && lo2 > minhi;
-        if (unique) {
-            best = c1;
-            bs = proj64(a, c1, xo0, xo1, xo2, n0, n1, n2);
-        }
-        // pass 2: FP64 for every valid candidate that may be the closest
-        for (int64_t e = unique ? e1 : e0; e < e1; e++) {
-            const int64_t c = a.nbr_idx[e];
-            const Cand32 k = classify32(a, c, po, n0f, n1f, n2f, scf, s_cur, xo0, xo1, xo2, n0, n1, n2);
-            if (!k.valid || k.lo > minhi) continue;
+        const float hi = d1 + B.err(d1);
+        full = full || !(hi < INFINITY);
+        // FP64 distance of one candidate, with the tie-breaks
+        auto consider = [&](int64_t c) {
             const double dx = a.pos[3 * c] - xo0;
             const double dy = a.pos[3 * c + 1] - xo1;
             const double dz = a.pos[3 * c + 2] - xo2;
             const double s = dx * n0 + dy * n1 + dz * n2;
             const double px = dx - s * n0, py = dy - s * n1, pz = dz - s * n2;
-            const double d2 = px * px + py * py + pz * pz;
-            const bool better = (best < 0) || (d2 < bd2) || (d2 == bd2 && s < bs) || (d2 == bd2 && s == bs && c < best);
-            if (better) { best = c; bs = s; bd2 = d2; }
+            const double dd = px * px + py * py + pz * pz;
+            const bool better = (best < 0) || (dd < bd2) || (dd == bd2 && s < bs) || (dd == bd2 && s == bs && c < best);
+            if (better) { best = c; bs = s; bd2 = dd; }
+        };
+        if (!full && (c2 < 0 || d2 - B.err(d2) > hi)) {
+            best = c1;
+            bs = proj64(a, c1, xo0, xo1, xo2, n0, n1, n2);
+        } else if (!full && (!(d3 < INFINITY) || d3 - B.err(d3) > hi)) {
+            consider(c1);
+            consider(c2);
+        } else if (c1 >= 0 || full) {
+            for (int64_t e = e0; e < e1; e++) {
+                const int64_t c = a.nbr_idx[e];
+                float d;
+                if (!ahead32(a, c, a.posf[c], po, n0f, n1f, n2f, scf, B, s_cur, xo0, xo1, xo2, n0, n1, n2, d)) continue;
+                if (!full && d - B.err(d) > hi) continue;
+                consider(c);
+            }
         }
         if (best < 0) { dead = true; return; }
         const double vp = FILL ? n0 * (a.vel[3 * best] - vo0) + n1 * (a.vel[3 * best + 1] - vo1) +
@@ -194,7 +225,7 @@ __device__ void walk_3d(const TraceArgs &a, int64_t o, int r, int64_t base, int3
 // Fill pass of a half-ray whose cells the count pass recorded: the same projections,
 // path lengths, line-of-sight velocities and velocity steps as the walk, without the
 // neighbour search.
-__device__ void replay_3d(const TraceArgs &a, int64_t o, int r, int64_t t, int64_t base, int32_t n_cells) {
+__device__ int32_t replay_3d(const TraceArgs &a, int64_t o, int r, int64_t t, int64_t base, int32_t n_cells) {
     const double n0 = a.dirs[3 * r], n1 = a.dirs[3 * r + 1], n2 = a.dirs[3 * r + 2];
     const double xo0 = a.pos[3 * o], xo1 = a.pos[3 * o + 1], xo2 = a.pos[3 * o + 2];
     const double vo0 = a.vel[3 * o], vo1 = a.vel[3 * o + 1], vo2 = a.vel[3 * o + 2];
@@ -210,6 +241,7 @@ __device__ void replay_3d(const TraceArgs &a, int64_t o, int r, int64_t t, int64
         emit<true>(a, base, len, x, (int32_t)c, s - s_cur, vp, va, ba);
         s_cur = s;
     }
+    return x;
 }
 
 // Spherically symmetric shells on +z: crossings of the ray with sphere j at
@@ -283,7 +315,8 @@ __global__ void k_trace(TraceArgs a) {
     if (FILL && a.tmp && a.geometry == MG_GEOM_3D) {
         const int32_t n_cells = a.len[ray];
         if (n_cells <= a.cap_tmp) {
-            replay_3d(a, o, r, t, base, n_cells);
+            const int32_t xl = replay_3d(a, o, r, t, base, n_cells);
+            a.xlen[ray] = a.xlen[ray] < 0 ? -xl - 1 : xl;
             return;
         }
     }
@@ -292,7 +325,10 @@ __global__ void k_trace(TraceArgs a) {
     if (overflow) atomicOr(a.err, 1);
     if (!FILL) {
         a.len[ray] = len;
-        a.xlen[ray] = dead ? -1 : 0;   // dead-end flag; the expanded lengths come from the fill pass
+        a.xlen[ray] = dead ? -1 : 0;   // dead-end flag
+    } else {
+        // the expanded length, with the count pass's dead-end flag as the sign (-x - 1)
+        a.xlen[ray] = a.xlen[ray] < 0 ? -x - 1 : x;
     }
 }
 
@@ -358,37 +394,31 @@ __global__ void k_scan_apply(const int32_t *cnt, int64_t m, const int64_t *bsum,
     if (i == m - 1) out[m] = bsum[blockIdx.x] + ex + v;
 }
 
-// Expanded length of every half-ray from the filled store (xcum of its last cell), with
-// the count pass's dead-end flag kept as the sign (-x - 1).
-__global__ void k_xlen(int64_t nr, const int64_t *__restrict__ ray_off, const int32_t *__restrict__ len,
-                       const int32_t *__restrict__ xcum, int32_t *__restrict__ xlen) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= nr) return;
-    const int32_t x = len[t] ? xcum[ray_off[t] + len[t] - 1] : 0;
-    xlen[t] = xlen[t] < 0 ? -x - 1 : x;
-}
-
 // ---------------------------------------------------------------- statistics
-__global__ void k_ray_stats(int64_t n, int R, int P, const int32_t *pf, const int32_t *pb, const int32_t *len,
-                            int32_t *xlen, unsigned long long *st) {
+constexpr int kStatBlocks = 304, kStatThreads = 256;
+
+// Two kernels' worth of blocks per SM, each adding its sums once (a warp each made 81 us of
+// contention on four words of 960k half-rays).
+__global__ void __launch_bounds__(kStatThreads) k_ray_stats(int64_t n, int R, int P, const int32_t *pf, const int32_t *pb,
+                                                            const int32_t *len, const int32_t *xlen,
+                                                            unsigned long long *st) {
     // st: [0] elements, [1] expanded, [2] max pair length, [3] dead ends
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     unsigned long long el = 0, ex = 0, mx = 0, dead = 0;
-    if (t < n * R) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * R; t += (int64_t)gridDim.x * blockDim.x) {
         int32_t xv = xlen[t];
-        if (xv < 0) { dead = 1; xv = -xv - 1; xlen[t] = xv; }
-        el = (unsigned long long)len[t];
-        ex = (unsigned long long)xv;
+        if (xv < 0) { dead++; xv = -xv - 1; }
+        el += (unsigned long long)len[t];
+        ex += (unsigned long long)xv;
     }
-    __syncthreads();
-    if (t < n * P) {
+    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n * P; t += (int64_t)gridDim.x * blockDim.x) {
         const int64_t o = t / P;
         const int p = (int)(t - o * P);
         int32_t a = xlen[o * R + pf[p]], b = xlen[o * R + pb[p]];
         a = a < 0 ? -a - 1 : a;
         b = b < 0 ? -b - 1 : b;
-        mx = (unsigned long long)(a + b + 1);
+        mx = max(mx, (unsigned long long)(a + b + 1));
     }
+    __shared__ unsigned long long sh[4][kStatThreads / 32];
     for (int d = 16; d; d >>= 1) {
         el += __shfl_down_sync(0xffffffffu, el, d);
         ex += __shfl_down_sync(0xffffffffu, ex, d);
@@ -397,61 +427,147 @@ __global__ void k_ray_stats(int64_t n, int R, int P, const int32_t *pf, const in
         mx = m2 > mx ? m2 : mx;
     }
     if ((threadIdx.x & 31) == 0) {
-        atomicAdd(&st[0], el);
-        atomicAdd(&st[1], ex);
-        atomicMax(&st[2], mx);
-        atomicAdd(&st[3], dead);
+        const int w = threadIdx.x >> 5;
+        sh[0][w] = el; sh[1][w] = ex; sh[2][w] = mx; sh[3][w] = dead;
     }
-}
-
-__global__ void k_to_float(const double *a, float *b, int64_t m) {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < m) b[i] = (float)a[i];
+    __syncthreads();
+    if (threadIdx.x < 4) {
+        unsigned long long v = sh[threadIdx.x][0];
+        for (int w = 1; w < kStatThreads / 32; w++)
+            v = threadIdx.x == 2 ? max(v, sh[2][w]) : v + sh[threadIdx.x][w];
+        if (threadIdx.x == 2) atomicMax(&st[2], v);
+        else if (v) atomicAdd(&st[threadIdx.x], v);
+    }
 }
 
 }  // namespace
 
-int mg_scan_counts(mg_ctx *ctx, const int32_t *d_cnt, int64_t m, int64_t *d_out) {
-    int64_t nb = (m + kScanBlock - 1) / kScanBlock;
-    int64_t *bsum = nullptr;
-    int rc;
-    if ((rc = mg_alloc(ctx, &bsum, nb))) return rc;
+// Exclusive prefix sum of m counts into d_out[m + 1]; bsum: scratch of one word per block.
+static int scan_counts(mg_ctx *ctx, const int32_t *d_cnt, int64_t m, int64_t *d_out, int64_t *bsum) {
+    const int64_t nb = (m + kScanBlock - 1) / kScanBlock;
     k_scan_blocks<<<(unsigned)nb, kScanBlock, 0, ctx->stream>>>(d_cnt, m, bsum);
     k_scan_sums<<<1, kScanBlock, 0, ctx->stream>>>(bsum, nb);
     k_scan_apply<<<(unsigned)nb, kScanBlock, 0, ctx->stream>>>(d_cnt, m, bsum, d_out);
-    cudaError_t e = cudaStreamSynchronize(ctx->stream);
-    cudaFree(bsum);
-    if (e != cudaSuccess) return mg_cuda_check(ctx, e, "scan");
+    MG_CUDA(cudaGetLastError());
     return MG_OK;
 }
 
-__global__ void k_posf(int64_t n, const double *__restrict__ pos, float4 *__restrict__ posf) {
+__global__ void k_posf(int64_t n, const double *__restrict__ pos, float4 *__restrict__ posf, unsigned *wmax) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const float x = (float)pos[3 * i], y = (float)pos[3 * i + 1], z = (float)pos[3 * i + 2];
-    posf[i] = make_float4(x, y, z, fabsf(x) + fabsf(y) + fabsf(z));
+    float w = 0.0f;
+    if (i < n) {
+        const float x = (float)pos[3 * i], y = (float)pos[3 * i + 1], z = (float)pos[3 * i + 2];
+        w = fabsf(x) + fabsf(y) + fabsf(z);
+        posf[i] = make_float4(x, y, z, w);
+    }
+    // (non-negative floats order like their bits; a NaN is the largest)
+    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(w) & 0x7fffffffu);
+    if ((threadIdx.x & 31) == 0) atomicMax(wmax, m);
 }
 
-// Temporaries of one trace, freed on every return (cudaFree waits for the kernels that
-// may still use them).
-struct TraceScratch {
-    int32_t *len = nullptr, *xlen = nullptr, *tmp = nullptr;
-    float4 *posf = nullptr;
-    ~TraceScratch() {
-        cudaFree(len);
-        cudaFree(xlen);
-        cudaFree(tmp);
-        cudaFree(posf);
+// Stream-ordered pool for a trace's scratch, one per device: allocating and freeing up to
+// gigabytes at every trace cost 1 ms of a 5.3 ms trace of 20k points. It keeps at most 1 GiB
+// between traces (the release threshold; the rest goes back at the next synchronisation)
+// and is given back with the device's last context. CUDA orders a block's reuse after the
+// work that used it, on whatever streams and threads.
+constexpr int kPoolDevices = 64;
+static std::mutex g_pool_mu;
+static cudaMemPool_t g_pool[kPoolDevices] = {};
+static int g_pool_refs[kPoolDevices] = {};
+
+void mg_pool_retain(int device) {
+    if (device < 0 || device >= kPoolDevices) return;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (g_pool_refs[device]++ > 0) return;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    unsigned long long keep = 1ull << 30;
+    if (cudaMemPoolCreate(&g_pool[device], &props) != cudaSuccess) {
+        g_pool[device] = nullptr;   // plain allocations then
+    } else if (cudaMemPoolSetAttribute(g_pool[device], cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaMemPoolDestroy(g_pool[device]);
+        g_pool[device] = nullptr;
     }
+    cudaGetLastError();
+}
+
+void mg_pool_release(int device) {
+    if (device < 0 || device >= kPoolDevices) return;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    if (--g_pool_refs[device] > 0) return;
+    if (g_pool[device]) cudaMemPoolDestroy(g_pool[device]);
+    g_pool[device] = nullptr;
+}
+
+// Temporaries of one trace, given back on every return (in stream order, or by cudaFree,
+// which waits for the kernels that may still use them).
+struct TraceScratch {
+    mg_ctx *ctx;
+    cudaMemPool_t pool;
+    std::vector<void *> held;
+    explicit TraceScratch(mg_ctx *c) : ctx(c), pool(nullptr) {
+        if (c->device >= 0 && c->device < kPoolDevices) {
+            std::lock_guard<std::mutex> lk(g_pool_mu);
+            pool = g_pool[c->device];
+        }
+    }
+    template <typename T>
+    cudaError_t get(T **p, size_t count) {
+        void *q = nullptr;
+        const size_t bytes = std::max<size_t>(1, count) * sizeof(T);
+        const cudaError_t e = pool ? cudaMallocFromPoolAsync(&q, bytes, pool, ctx->stream) : cudaMalloc(&q, bytes);
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            return e;
+        }
+        held.push_back(q);
+        *p = static_cast<T *>(q);
+        return e;
+    }
+    void give_back() {
+        for (void *q : held) {
+            if (pool) cudaFreeAsync(q, ctx->stream);
+            else cudaFree(q);
+        }
+        held.clear();
+    }
+    ~TraceScratch() { give_back(); }
 };
+
+// A buffer of the ray store for `count` elements: the one at hand when it is large enough and
+// not more than half empty, else a new one with 3 % to spare for the next trace.
+template <typename T>
+static int ray_buffer(mg_ctx *ctx, T **p, int64_t &cap, int64_t count) {
+    if (*p && cap >= count && cap <= 2 * count + 4096) return MG_OK;
+    cap = 0;
+    const int64_t want = count + count / 32;
+    int rc = mg_alloc(ctx, p, want);
+    if (rc && want > count) rc = mg_alloc(ctx, p, count);
+    if (!rc) cap = rc ? 0 : want;
+    return rc;
+}
 
 int mg_launch_trace(mg_ctx *ctx) {
     const int64_t nr = ctx->n * ctx->R;
     int rc;
-    TraceScratch sc;
-    if ((rc = mg_alloc(ctx, &sc.len, nr)) || (rc = mg_alloc(ctx, &sc.xlen, nr))) return rc;
-    int32_t *const d_len = sc.len, *const d_xlen = sc.xlen;
-    if ((rc = mg_alloc(ctx, &ctx->d_ray_off, nr + 1))) return rc;
+    TraceScratch sc(ctx);
+    int32_t *d_len = nullptr, *d_xlen = nullptr, *d_tmp = nullptr;
+    float4 *posf = nullptr;
+    int64_t *bsum = nullptr;
+    unsigned *wmax = nullptr;
+    cudaError_t ce;
+    if ((ce = sc.get(&d_len, nr)) || (ce = sc.get(&d_xlen, nr)) ||
+        (ce = sc.get(&bsum, (nr + kScanBlock - 1) / kScanBlock)) || (ce = sc.get(&wmax, 1)))
+        return mg_fail(ctx, MG_ERR_OOM, std::string("cudaMalloc failed: ") + cudaGetErrorString(ce));
+    // The ray store is written in place: solves and images of the old rays come first. Those
+    // of this stream do; after a change of stream, wait for all (as the frees of a replaced
+    // store do).
+    if (ctx->stream_changed) MG_CUDA(cudaDeviceSynchronize());
+    ctx->stream_changed = false;
+    ctx->traced = false;
+    if ((rc = ray_buffer(ctx, &ctx->d_ray_off, ctx->ray_off_cap, nr + 1))) return rc;
     MG_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int32_t), ctx->stream));
     TraceArgs a{};
     a.n = ctx->n; a.R = ctx->R; a.geometry = ctx->geometry;
@@ -460,14 +576,16 @@ int mg_launch_trace(mg_ctx *ctx) {
     a.dshift_frac = ctx->opt.dshift_frac; a.max_steps = ctx->opt.max_steps;
     a.len = d_len; a.xlen = d_xlen; a.err = ctx->d_err;
     if (ctx->geometry == MG_GEOM_3D) {
-        if ((rc = mg_alloc(ctx, &sc.posf, ctx->n))) return rc;
-        k_posf<<<(unsigned)((ctx->n + 255) / 256), 256, 0, ctx->stream>>>(ctx->n, ctx->d_pos, sc.posf);
+        if ((ce = sc.get(&posf, ctx->n)))
+            return mg_fail(ctx, MG_ERR_OOM, std::string("cudaMalloc failed: ") + cudaGetErrorString(ce));
+        MG_CUDA(cudaMemsetAsync(wmax, 0, sizeof(unsigned), ctx->stream));
+        k_posf<<<(unsigned)((ctx->n + 255) / 256), 256, 0, ctx->stream>>>(ctx->n, ctx->d_pos, posf, wmax);
     }
-    a.posf = sc.posf;
+    a.posf = posf;
+    a.wmax = reinterpret_cast<const float *>(wmax);
     // Record up to cap_tmp cells per half-ray in the count pass, in scratch of at most
-    // 32 GiB and a quarter of the free device memory (freed after tracing; half-rays with
+    // 32 GiB and a quarter of the free device memory (given back after tracing; half-rays with
     // more cells, or all of them without scratch, are walked again by the fill pass).
-    int32_t *&d_tmp = sc.tmp;
     int32_t cap_tmp = 128;
     size_t free_b = 0, total_b = 0;
     if (cudaMemGetInfo(&free_b, &total_b) != cudaSuccess) {
@@ -476,10 +594,7 @@ int mg_launch_trace(mg_ctx *ctx) {
     }
     const double budget = std::min(32.0 * (1 << 30), 0.25 * (double)free_b);
     while (cap_tmp > 0 && (double)nr * cap_tmp * 4.0 > budget) cap_tmp /= 2;
-    if (ctx->geometry == MG_GEOM_3D && cap_tmp > 0 && cudaMalloc(&d_tmp, (size_t)nr * cap_tmp * 4) != cudaSuccess) {
-        cudaGetLastError();
-        d_tmp = nullptr;
-    }
+    if (ctx->geometry == MG_GEOM_3D && cap_tmp > 0) sc.get(&d_tmp, (size_t)nr * cap_tmp);
     a.tmp = d_tmp;
     a.cap_tmp = d_tmp ? cap_tmp : 0;
     const int bs = 128;
@@ -489,36 +604,33 @@ int mg_launch_trace(mg_ctx *ctx) {
         k_trace<false><<<grid, bs, 0, ctx->stream>>>(a);
     }
     MG_CUDA(cudaGetLastError());
-    if ((rc = mg_scan_counts(ctx, d_len, nr, ctx->d_ray_off))) return rc;
+    if ((rc = scan_counts(ctx, d_len, nr, ctx->d_ray_off, bsum))) return rc;
     int64_t total = 0;
     int32_t kerr = 0;
-    MG_CUDA(cudaMemcpy(&total, ctx->d_ray_off + nr, 8, cudaMemcpyDeviceToHost));
-    MG_CUDA(cudaMemcpy(&kerr, ctx->d_err, 4, cudaMemcpyDeviceToHost));
+    MG_CUDA(cudaMemcpyAsync(&total, ctx->d_ray_off + nr, 8, cudaMemcpyDeviceToHost, ctx->stream));
+    MG_CUDA(cudaMemcpyAsync(&kerr, ctx->d_err, 4, cudaMemcpyDeviceToHost, ctx->stream));
+    MG_CUDA(cudaStreamSynchronize(ctx->stream));
     if (kerr) {
         return mg_fail(ctx, MG_ERR_CAPACITY, "ray tracing: a half-ray exceeded max_steps");
     }
-    if ((rc = mg_alloc(ctx, &ctx->d_cells, total)) || (rc = mg_alloc(ctx, &ctx->d_xcum, total)) ||
-        (rc = mg_alloc(ctx, &ctx->d_ds, total)) || (rc = mg_alloc(ctx, &ctx->d_vpar, total)) ||
-        (rc = mg_alloc(ctx, &ctx->d_dsf, total)) || (rc = mg_alloc(ctx, &ctx->d_vparf, total)))
+    if ((rc = ray_buffer(ctx, &ctx->d_cells, ctx->ray_cap[0], total)) || (rc = ray_buffer(ctx, &ctx->d_xcum, ctx->ray_cap[1], total)) ||
+        (rc = ray_buffer(ctx, &ctx->d_ds, ctx->ray_cap[2], total)) || (rc = ray_buffer(ctx, &ctx->d_vpar, ctx->ray_cap[3], total)) ||
+        (rc = ray_buffer(ctx, &ctx->d_dsf, ctx->ray_cap[4], total)) || (rc = ray_buffer(ctx, &ctx->d_vparf, ctx->ray_cap[5], total)))
         return rc;
     a.ray_off = ctx->d_ray_off; a.cells = ctx->d_cells; a.xcum = ctx->d_xcum; a.ds = ctx->d_ds; a.vpar = ctx->d_vpar;
+    a.dsf = ctx->d_dsf; a.vparf = ctx->d_vparf;
     {
         MgTimed t(ctx, "trace_fill");
         k_trace<true><<<grid, bs, 0, ctx->stream>>>(a);
     }
     MG_CUDA(cudaGetLastError());
-    if (total) {
-        k_to_float<<<(unsigned)((total + 255) / 256), 256, 0, ctx->stream>>>(ctx->d_ds, ctx->d_dsf, total);
-        k_to_float<<<(unsigned)((total + 255) / 256), 256, 0, ctx->stream>>>(ctx->d_vpar, ctx->d_vparf, total);
-    }
-    k_xlen<<<(unsigned)((nr + 255) / 256), 256, 0, ctx->stream>>>(nr, ctx->d_ray_off, d_len, ctx->d_xcum, d_xlen);
     MG_CUDA(cudaMemsetAsync(ctx->d_scal, 0, 4 * sizeof(unsigned long long), ctx->stream));
-    const int64_t np = std::max<int64_t>(nr, ctx->n * ctx->P);
-    k_ray_stats<<<(unsigned)((np + 255) / 256), 256, 0, ctx->stream>>>(ctx->n, ctx->R, ctx->P, ctx->d_pf, ctx->d_pb,
-                                                                          d_len, d_xlen, ctx->d_scal);
+    k_ray_stats<<<kStatBlocks, kStatThreads, 0, ctx->stream>>>(ctx->n, ctx->R, ctx->P, ctx->d_pf, ctx->d_pb, d_len, d_xlen,
+                                                              ctx->d_scal);
     MG_CUDA(cudaGetLastError());
     unsigned long long st[4];
     MG_CUDA(cudaMemcpyAsync(st, ctx->d_scal, sizeof(st), cudaMemcpyDeviceToHost, ctx->stream));
+    sc.give_back();   // before the synchronisation, at which the pool lets go of what it does not keep
     MG_CUDA(cudaStreamSynchronize(ctx->stream));
     ctx->n_elements = (int64_t)st[0];
     ctx->n_expanded = (int64_t)st[1];
