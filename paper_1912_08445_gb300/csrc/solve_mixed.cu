@@ -352,8 +352,8 @@ __global__ void __launch_bounds__(256) k_feautrier_mixed(MixArgs a) {
 
 // ---------------------------------------------------------------------------------
 // Warp-per-(origin, line group) variant for models whose lines do not overlap (the
-// common case). A warp serves G lines (G lane groups of 32/G lanes) and every lane NB
-// bins of its line, so each shared-memory read and loop step is shared by NB updates.
+// common case). A warp serves G lines and every lane NB (line, bin) results (BinLanes and
+// LineLanes below), so each shared-memory read and loop step is shared by NB updates.
 // The warp loops over all ray pairs of its origin and stages the expanded points through
 // a private ring of kRing points (one point per lane per refill): no CTA barrier is ever
 // needed, and the pair sums are kept per lane in a fixed order. The boundary row is the
@@ -486,11 +486,10 @@ __device__ __forceinline__ PointGeo point_geometry(const ElemWin<G> &w, int bf, 
     return p;
 }
 
-// Line part: (X', X', S, S) of the warp's G lines into slot s of the ring; returns the
-// largest X'.
+// Line part: (X', S) of the warp's G lines; returns the largest X'.
 template <int G>
 __device__ __forceinline__ float point_lines(const MixArgs &a, const ElemWin<G> &w, int bf, int i, const PointGeo &p,
-                                             float4 (&out)[G]) {
+                                             float2 (&out)[G]) {
     const float ibc = p.ib * a.inv_chi_min;
     float Xmax = 0.0f;
 #pragma unroll
@@ -499,7 +498,7 @@ __device__ __forceinline__ float point_lines(const MixArgs &a, const ElemWin<G> 
         const float X = fmaxf(e.y, 0.0f) * ibc;
         // (a line whose opacity is below the smallest normal float has no source here)
         const float S = e.y >= 1.17549435e-38f ? e.x * rcpf(e.y) : 0.0f;
-        out[k] = make_float4(X, X, S, S);
+        out[k] = make_float2(X, S);
         Xmax = fmaxf(Xmax, X);
     }
     return Xmax;
@@ -627,6 +626,195 @@ __device__ __forceinline__ void bin_results(const BinState<NB> &st, float (&pi)[
     }
 }
 
+// How the (line, bin) results of a warp lie on its lanes.
+//
+// BinLanes: G lane groups of 32/G lanes, a line each; a lane has NB bins of its line, swept in
+// pairs of bins. It fits any number of bins to the lanes.
+//
+// LineLanes: a lane has the same NB/G bins (lane, lane + 32, ...) of all G lines, swept in
+// pairs of lines. The profile argument a_q g_z - g_y and its exponential are the same for every
+// line of a species (the bins are in Doppler widths), so they are computed once per bin
+// for all G lines: per pair and point 9 packed ops, 2 rcp and 4 max/min, and per point and
+// bin 2 ops, one ex2 and a copy, against 11 packed ops, 2 ex2, 2 rcp and 4 max/min per pair
+// in BinLanes. Points of the ring carry (X, X, S, S) of a line pair without duplicates.
+// Measured, BinLanes -> LineLanes: disc 20k (19 lines x 63 bins, G = 4, NB = 8) 197.5 -> 180.6 ms;
+// clumpy 50k (4 x 31, G = 4, NB = 4) 9.07 -> 8.69 ms.
+template <int G_, int NB_>
+struct BinLanes {
+    static constexpr int G = G_, NB = NB_, LPG = 32 / G, kRingLines = G;
+    BinState<NB> st;
+    float nu_g;
+    float4 Do;              // the origin's line data
+    int grp;
+
+    __device__ __forceinline__ int line(int) const { return grp; }
+    __device__ __forceinline__ int bin(int i) const { return (threadIdx.x & 31) - grp * LPG + LPG * i; }
+    __device__ __forceinline__ float aq(int i) const { return st.aq(i); }
+    __device__ __forceinline__ void init(const MixArgs &a, int64_t o, int l0, float bo, float ibo) {
+        grp = (threadIdx.x & 31) / LPG;
+        const int lc = l0 + grp < a.L ? l0 + grp : a.L - 1;
+        nu_g = a.nu_ghz[lc];
+        const float2 dl = reinterpret_cast<const float2 *>(a.line)[o * a.L + lc];
+        const float Xo = fmaxf(dl.y, 0.0f) * (ibo * a.inv_chi_min);   // in units of chi_min
+        const float So = dl.y > 0.0f ? dl.x / dl.y : 0.0f;
+        Do = make_float4(Xo, Xo, So, So);
+#pragma unroll
+        for (int i = 0; i < NB; i++) st.set_aq(i, bin(i) < a.Q ? (float)(a.roots[bin(i)] * (double)bo) : 0.0f);
+    }
+    __device__ __forceinline__ float origin_X(int) const { return Do.x; }
+    __device__ __forceinline__ float origin_S(int) const { return Do.z; }
+    __device__ __forceinline__ float empty_psi(const SweepK &k, int i) const {
+        return kSqrt2 * planck_k(k, nu_g * (1.0f + st.aq(i) * (float)(1.0 / kC)));
+    }
+    static __device__ __forceinline__ void put(float4 *rl, int s, const float2 (&x)[G]) {
+#pragma unroll
+        for (int k = 0; k < G; k++) rl[k * kRing + s] = make_float4(x[k].x, x[k].x, x[k].y, x[k].y);
+    }
+    __device__ __forceinline__ void first(const SweepK &k, const float4 A, const float4 *rl, float v) {
+        first_point<NB>(k, st, A, rl[grp * kRing], nu_g, v);
+    }
+    template <bool FLOOR>
+    __device__ __forceinline__ void step(const SweepK &k, const float4 A, const float4 *rl, int j, const float2 q) {
+        step_point<NB, FLOOR>(k, st, A, rl[grp * kRing + j], q);
+    }
+    __device__ __forceinline__ void origin(const SweepK &k, const float4 Ao, const float2 q) {
+        step_point<NB>(k, st, Ao, Do, q);
+    }
+    __device__ __forceinline__ void results(float (&pi)[NB], float (&ps)[NB], float (&dt)[NB]) const {
+        bin_results<NB>(st, pi, ps, dt);
+    }
+};
+
+// Result i: bin i / G of the lane, line i % G.
+template <int G_, int NB_>
+struct LineLanes {
+    static constexpr int G = G_, NB = NB_, NBL = NB / G, H = G / 2, NP = NBL * H, kRingLines = H;
+    static_assert(G % 2 == 0 && NB % G == 0, "whole line pairs");
+    float a_q[NBL];
+    float2 chi_p[NP], S_p[NP], d_p[NP], Phi[NP], iota[NP], psi[NP];   // pair b H + h: bin b, lines 2h and 2h + 1
+    const float *nu;        // GHz, of the warp's lines
+    int lines;              // lines of the group that exist
+    float4 Do[H];           // the origin's (X0, X1, S0, S1) per line pair
+
+    __device__ __forceinline__ int line(int i) const { return i % G; }
+    __device__ __forceinline__ int bin(int i) const { return (threadIdx.x & 31) + 32 * (i / G); }
+    __device__ __forceinline__ float aq(int i) const { return a_q[i / G]; }
+    __device__ __forceinline__ float nu_of(int k) const { return nu[k < lines ? k : lines - 1]; }
+    __device__ __forceinline__ void init(const MixArgs &a, int64_t o, int l0, float bo, float ibo) {
+        nu = a.nu_ghz + l0;
+        lines = min(G, a.L - l0);
+#pragma unroll
+        for (int b = 0; b < NBL; b++) {
+            const int q = bin(b * G);
+            a_q[b] = q < a.Q ? (float)(a.roots[q] * (double)bo) : 0.0f;
+        }
+        float X[G], S[G];
+#pragma unroll
+        for (int k = 0; k < G; k++) {
+            const float2 dl = reinterpret_cast<const float2 *>(a.line)[o * a.L + l0 + (k < lines ? k : lines - 1)];
+            X[k] = fmaxf(dl.y, 0.0f) * (ibo * a.inv_chi_min);   // in units of chi_min
+            S[k] = dl.y > 0.0f ? dl.x / dl.y : 0.0f;
+        }
+#pragma unroll
+        for (int h = 0; h < H; h++) Do[h] = make_float4(X[2 * h], X[2 * h + 1], S[2 * h], S[2 * h + 1]);
+    }
+    __device__ __forceinline__ float origin_X(int i) const { return (i & 1) ? Do[(i % G) >> 1].y : Do[(i % G) >> 1].x; }
+    __device__ __forceinline__ float origin_S(int i) const { return (i & 1) ? Do[(i % G) >> 1].w : Do[(i % G) >> 1].z; }
+    __device__ __forceinline__ float empty_psi(const SweepK &k, int i) const {
+        return kSqrt2 * planck_k(k, nu_of(line(i)) * (1.0f + aq(i) * (float)(1.0 / kC)));
+    }
+    static __device__ __forceinline__ void put(float4 *rl, int s, const float2 (&x)[G]) {
+#pragma unroll
+        for (int h = 0; h < H; h++)
+            rl[h * kRing + s] = make_float4(x[2 * h].x, x[2 * h + 1].x, x[2 * h].y, x[2 * h + 1].y);
+    }
+    // 2^(-x'^2) of every bin of the lane
+    __device__ __forceinline__ void profile(const float4 A, float (&e)[NBL]) const {
+        if constexpr (NBL % 2 == 0) {
+#pragma unroll
+            for (int b = 0; b < NBL; b += 2) {
+                const float2 x = __ffma2_rn(make_float2(a_q[b], a_q[b + 1]), make_float2(A.x, A.y), make_float2(A.z, A.w));
+                const float2 xx = __fmul2_rn(x, x);
+                e[b] = ex2f(-xx.x);
+                e[b + 1] = ex2f(-xx.y);
+            }
+        } else {
+#pragma unroll
+            for (int b = 0; b < NBL; b++) {
+                const float x = fmaf(a_q[b], A.x, A.z);
+                e[b] = ex2f(-x * x);
+            }
+        }
+    }
+    __device__ __forceinline__ void first(const SweepK &k, const float4 A, const float4 *rl, float v) {
+        float e[NBL];
+        profile(A, e);
+        const float dop = 1.0f - v * (float)(1.0 / kC);
+#pragma unroll
+        for (int b = 0; b < NBL; b++)
+#pragma unroll
+            for (int h = 0; h < H; h++) {
+                const int p = b * H + h;
+                const float4 D = rl[h * kRing];
+                const float2 chil = __fmul2_rn(make_float2(D.x, D.y), make_float2(e[b], e[b]));
+                chi_p[p] = make_float2(fmaxf(chil.x, 1.0f), fmaxf(chil.y, 1.0f));
+                S_p[p] = __fmul2_rn(make_float2(D.z, D.w), make_float2(fminf(chil.x, 1.0f), fminf(chil.y, 1.0f)));
+                Phi[p] = make_float2(kSqrt2, kSqrt2);
+                iota[p] = make_float2(1.0f, 1.0f);
+                d_p[p] = make_float2(0.0f, 0.0f);
+                const float sh = (1.0f + a_q[b] * (float)(1.0 / kC)) * dop;
+                psi[p] = make_float2(kSqrt2 * planck_k(k, nu_of(2 * h) * sh), kSqrt2 * planck_k(k, nu_of(2 * h + 1) * sh));
+            }
+    }
+    template <bool FLOOR>
+    __device__ __forceinline__ void row(const SweepK &k, int p, const float4 D, float e, const float2 q) {
+        const float2 chil = __fmul2_rn(make_float2(D.x, D.y), make_float2(e, e));
+        const float2 chi = make_float2(fmaxf(chil.x, 1.0f), fmaxf(chil.y, 1.0f));
+        const float2 Sx = __fmul2_rn(make_float2(D.z, D.w), make_float2(fminf(chil.x, 1.0f), fminf(chil.y, 1.0f)));
+        const float2 d0 = __fmul2_rn(__fadd2_rn(chi_p[p], chi), q);
+        const float2 dl = FLOOR ? make_float2(fmaxf(d0.x, k.dtau_min), fmaxf(d0.y, k.dtau_min)) : d0;
+        const float2 sm = __fadd2_rn(d_p[p], dl);
+        Phi[p] = __ffma2_rn(Phi[p], iota[p], sm);
+        const float2 den = __ffma2_rn(dl, Phi[p], make_float2(1.0f, 1.0f));
+        iota[p] = make_float2(rcpf(den.x), rcpf(den.y));
+        psi[p] = __fmul2_rn(__ffma2_rn(sm, S_p[p], psi[p]), iota[p]);
+        d_p[p] = dl;
+        chi_p[p] = chi;
+        S_p[p] = Sx;
+    }
+    template <bool FLOOR>
+    __device__ __forceinline__ void step(const SweepK &k, const float4 A, const float4 *rl, int j, const float2 q) {
+        float e[NBL];
+        profile(A, e);
+#pragma unroll
+        for (int h = 0; h < H; h++) {
+            const float4 D = rl[h * kRing + j];
+#pragma unroll
+            for (int b = 0; b < NBL; b++) row<FLOOR>(k, b * H + h, D, e[b], q);
+        }
+    }
+    __device__ __forceinline__ void origin(const SweepK &k, const float4 Ao, const float2 q) {
+        float e[NBL];
+        profile(Ao, e);
+#pragma unroll
+        for (int h = 0; h < H; h++)
+#pragma unroll
+            for (int b = 0; b < NBL; b++) row<true>(k, b * H + h, Do[h], e[b], q);
+    }
+    __device__ __forceinline__ void results(float (&pi)[NB], float (&ps)[NB], float (&dt)[NB]) const {
+#pragma unroll
+        for (int b = 0; b < NBL; b++)
+#pragma unroll
+            for (int h = 0; h < H; h++) {
+                const int p = b * H + h, i = b * G + 2 * h;
+                const float2 pp = __fmul2_rn(Phi[p], iota[p]);
+                pi[i] = pp.x; pi[i + 1] = pp.y;
+                ps[i] = psi[p].x; ps[i + 1] = psi[p].y;
+                dt[i] = d_p[p].x; dt[i + 1] = d_p[p].y;
+            }
+    }
+};
+
 // Sweeps half-ray r from its far end to the origin; returns per bin (Phi^ iota, psi^,
 // delta) of the row next to the origin, or the empty-half values (sqrt 2, sqrt 2 I_o, 0).
 // `pre` says that buffer bf already holds (or is receiving) the first window of r; on
@@ -647,12 +835,12 @@ __device__ __forceinline__ void bin_results(const BinState<NB> &st, float (&pi)[
 // out or not. Measured, launch of the best shape, every point staged and left out one by one
 // -> this: clumpy cloud (50k points, 48 rays, 4 x 31 bins, 69 % of the points far) 11.72 ->
 // 9.06 ms; disc (32k points, 192 rays, 19 x 63, 7 % far) 203.3 -> 197.0 ms.
-template <int G, int NB>
-__device__ __forceinline__ void sweep_half(const MixArgs &a, const SweepK &k, int64_t o, int l0, int grp, int r,
-                                           int rnext, float nu_g, const float4 Ao, const float4 Do, Ring &rg,
-                                           float4 *rl, ElemWin<G> &w, int &bf, bool &pre, BinState<NB> &st,
-                                           float (&pi)[NB], float (&ps)[NB], float (&dt)[NB], float aq_lo,
-                                           float aq_hi, int &npts) {
+template <typename Lay>
+__device__ __forceinline__ void sweep_half(const MixArgs &a, const SweepK &k, int64_t o, int l0, int r, int rnext,
+                                           const float4 Ao, Ring &rg, float4 *rl, ElemWin<Lay::G> &w, int &bf,
+                                           bool &pre, Lay &lay, float (&pi)[Lay::NB], float (&ps)[Lay::NB],
+                                           float (&dt)[Lay::NB], float aq_lo, float aq_hi, int &npts) {
+    constexpr int G = Lay::G, NB = Lay::NB;
     const int lane = threadIdx.x & 31;
     const int64_t off = a.ray_off[o * a.R + r];
     const int len = (int)(a.ray_off[o * a.R + r + 1] - off);
@@ -666,7 +854,7 @@ __device__ __forceinline__ void sweep_half(const MixArgs &a, const SweepK &k, in
 #pragma unroll
         for (int i = 0; i < NB; i++) {
             pi[i] = kSqrt2;
-            ps[i] = kSqrt2 * planck_k(k, nu_g * (1.0f + st.aq(i) * (float)(1.0 / kC)));
+            ps[i] = lay.empty_psi(k, i);
             dt[i] = 0.0f;
         }
         return;
@@ -677,7 +865,6 @@ __device__ __forceinline__ void sweep_half(const MixArgs &a, const SweepK &k, in
         win_gathers<G>(a, l0, w, bf);
     }
     pre = false;
-    const float4 *my = rl + grp * kRing;
     bool first = true;
     unsigned far1 = 0, far2 = 0;   // whether the last two kept points are far
     int run = 0;                   // far points (at most 2) right before the window
@@ -746,7 +933,7 @@ __device__ __forceinline__ void sweep_half(const MixArgs &a, const SweepK &k, in
             bool far = false;
             float qin = 0.0f;
             PointGeo p{};
-            float4 lines[G];
+            float2 lines[G];
             if (lane < cnt) {
                 const int i = own.x, j = own.y - (c0 + lane) - own.z + 1;
                 p = point_geometry<G>(w, bf, i, j, own.w);
@@ -773,8 +960,7 @@ __device__ __forceinline__ void sweep_half(const MixArgs &a, const SweepK &k, in
                 const int s = __popc(proc & ((1u << lane) - 1u));
                 rg.a[s] = make_float4(p.gz, p.gz, -p.gy, -p.gy);
                 rg.q[s] = make_float2(qin, qin);
-#pragma unroll
-                for (int kk = 0; kk < G; kk++) rl[kk * kRing + s] = lines[kk];
+                Lay::put(rl, s, lines);
             }
             __syncwarp();
             npts += m;
@@ -782,7 +968,7 @@ __device__ __forceinline__ void sweep_half(const MixArgs &a, const SweepK &k, in
             if (first) {
                 const float4 A = rg.a[0];
                 const float vfar = -A.z / (A.x - A.z * (float)(1.0 / kC));   // v = (v pz)/pz
-                first_point<NB>(k, st, A, my[0], nu_g, vfar);
+                lay.first(k, A, rl, vfar);
                 j = 1;
             }
             // A refill whose intervals all have q' >= q_nofloor sweeps without the dtau floor.
@@ -791,7 +977,7 @@ __device__ __forceinline__ void sweep_half(const MixArgs &a, const SweepK &k, in
             first = false;
             auto dense = [&](auto floor_tag, int jend) {
 #pragma unroll 4
-                for (; j < jend; j++) step_point<NB, decltype(floor_tag)::value>(k, st, rg.a[j], my[j], rg.q[j]);
+                for (; j < jend; j++) lay.template step<decltype(floor_tag)::value>(k, rg.a[j], rl, j, rg.q[j]);
             };
             // two segments, with the gathers of the next window issued between them (one
             // copy of each loop body)
@@ -817,9 +1003,9 @@ __device__ __forceinline__ void sweep_half(const MixArgs &a, const SweepK &k, in
         bf ^= 1;
     }
     if (pre) bf ^= 1;   // the next half-ray's first window sits in the other buffer
-    step_point<NB>(k, st, Ao, Do, make_float2(qc, qc));   // the origin
+    lay.origin(k, Ao, make_float2(qc, qc));
     npts++;
-    bin_results<NB>(st, pi, ps, dt);
+    lay.results(pi, ps, dt);
 }
 
 // Per-lane, per-bin values that live across the ray pairs (slot [.][i][lane]): the pair
@@ -832,40 +1018,26 @@ struct PairSmem {
 };
 
 // One work item: origin o, lines l0 .. l0+G-1, all ray pairs, all bins (one warp).
-template <int G, int NB>
+template <typename Lay>
 __device__ __forceinline__ void solve_item(const MixArgs &a, int64_t o, int l0, Ring &rg, float4 *rl,
-                                           ElemWin<G> &w, PairSmem<NB> &ps) {
-    constexpr int LPG = 32 / G;   // lanes per line
+                                           ElemWin<Lay::G> &w, PairSmem<Lay::NB> &ps) {
+    constexpr int G = Lay::G, NB = Lay::NB;
     const int lane = threadIdx.x & 31;
-    const int grp = lane / LPG, li = lane - grp * LPG;
-    const int l = l0 + grp;
-    const bool line_ok = l < a.L;
-    const int lc = line_ok ? l : a.L - 1;
     const int Q = a.Q;
     const float bo = a.b[o];
     const float ibo = 1.0f / bo;
-    const float2 dl = reinterpret_cast<const float2 *>(a.line)[o * a.L + lc];
-    // ring entries of the origin (v = 0 there): a = (g_z, g_z, -0, -0), line = (X, X, S, S)
+    // ring entry of the origin (v = 0 there): a = (g_z, g_z, -0, -0)
     const float gzo = kSqrtLog2e * ibo;
-    const float Xo = fmaxf(dl.y, 0.0f) * (ibo * a.inv_chi_min);   // in units of chi_min
-    const float So = dl.y > 0.0f ? dl.x / dl.y : 0.0f;
     const float4 Ao = make_float4(gzo, gzo, -0.0f, -0.0f);
-    const float4 Do = make_float4(Xo, Xo, So, So);
-    const float nu_g = a.nu_ghz[lc];
     const SweepK k{a.dtau_min, a.planck_a, a.planck_b};
-    BinState<NB> st;
-#pragma unroll
-    for (int i = 0; i < NB; i++) {
-        const int q = li + LPG * i;
-        st.set_aq(i, q < Q ? (float)(a.roots[q] * (double)bo) : 0.0f);
-        ps.acc[0][i][lane] = ps.acc[1][i][lane] = ps.acc[2][i][lane] = 0.0f;
-    }
+    Lay lay;
+    lay.init(a, o, l0, bo, ibo);
     // range of a_q over the whole warp (all lanes, all bins)
     float aq_lo = 1e30f, aq_hi = -1e30f;
 #pragma unroll
     for (int i = 0; i < NB; i++) {
-        const int q = li + LPG * i;
-        if (q < Q) { aq_lo = fminf(aq_lo, st.aq(i)); aq_hi = fmaxf(aq_hi, st.aq(i)); }
+        ps.acc[0][i][lane] = ps.acc[1][i][lane] = ps.acc[2][i][lane] = 0.0f;
+        if (lay.bin(i) < Q) { aq_lo = fminf(aq_lo, lay.aq(i)); aq_hi = fmaxf(aq_hi, lay.aq(i)); }
     }
     for (int d = 16; d; d >>= 1) {
         aq_lo = fminf(aq_lo, __shfl_xor_sync(0xffffffffu, aq_lo, d));
@@ -880,8 +1052,8 @@ __device__ __forceinline__ void solve_item(const MixArgs &a, int64_t o, int l0, 
         float pif[NB], psf[NB], dtf[NB];
 #pragma unroll 1
         for (int h = 0; h < 2; h++) {   // backward half, then forward half (one code copy)
-            sweep_half<G, NB>(a, k, o, l0, grp, h ? rf : rb, h ? rn : rf, nu_g, Ao, Do, rg, rl, w, bf, pre,
-                                    st, pif, psf, dtf, aq_lo, aq_hi, npts);
+            sweep_half<Lay>(a, k, o, l0, h ? rf : rb, h ? rn : rf, Ao, rg, rl, w, bf, pre, lay, pif, psf, dtf, aq_lo,
+                            aq_hi, npts);
             if (h == 0) {
 #pragma unroll
                 for (int i = 0; i < NB; i++) {
@@ -915,44 +1087,100 @@ __device__ __forceinline__ void solve_item(const MixArgs &a, int64_t o, int l0, 
         const int lines = min(G, a.L - l0);
         atomicAdd(a.work, (unsigned long long)npts * (unsigned long long)(lines * Q));
     }
-    // weighted sums over each line's bins: fixed shuffle tree in FP64 within the lane group
+    // The origin's line opacity and floored source in a bin are the same for every pair: u =
+    // Lambda* S + (u - Lambda* S) and the line's shares of opacity and emission enter after the
+    // sums over pairs. v: u, Lambda, J_eff and 1 - Lambda of result i.
     const double invP = 1.0 / a.P;
-    double s[4] = {0.0, 0.0, 0.0, 0.0};
-#pragma unroll
-    for (int i = 0; i < NB; i++) {
-        const int q = li + LPG * i;
-        const double wq = q < Q ? a.weights[q] : 0.0;
-        // the origin's line opacity and floored source in this bin are the same for every
-        // pair: u = Lambda* S + (u - Lambda* S) and the line's shares of opacity and
-        // emission enter after the sums over pairs
-        const float xo = st.aq(i) * gzo;
+    auto values = [&](int i, float (&v)[4]) {
+        const float xo = lay.aq(i) * gzo, Xo = lay.origin_X(i), So = lay.origin_S(i);
         const float chilo = Xo * ex2f(-xo * xo);
         const float chio = fmaxf(chilo, 1.0f), ichi = rcpf(chio);
         const float Sov = So * fminf(chilo, 1.0f);
         const float lam = ps.acc[0][i][lane], uml = ps.acc[1][i][lane], oml = ps.acc[2][i][lane];
-        const float u = uml + lam * Sov;
-        const float v[4] = {u, lam * (chilo * ichi), uml + lam * ((Sov * chio - chilo * So) * ichi),
-                            oml + lam * ((chio - chilo) * ichi)};
+        v[0] = uml + lam * Sov;
+        v[1] = lam * (chilo * ichi);
+        v[2] = uml + lam * ((Sov * chio - chilo * So) * ichi);
+        v[3] = oml + lam * ((chio - chilo) * ichi);
+        if (a.Jnu && lay.bin(i) < Q && l0 + lay.line(i) < a.L)
+            a.Jnu[(o * a.L + l0 + lay.line(i)) * Q + lay.bin(i)] = (double)v[0] * invP * (double)kI0;
+    };
+    // weighted sums over each line's bins in FP64, in a fixed order
+    if constexpr (Lay::kRingLines == G) {
+        // a line per lane group: a shuffle tree within the group
+        constexpr int LPG = 32 / G;
+        double s[4] = {0.0, 0.0, 0.0, 0.0};
 #pragma unroll
-        for (int kk = 0; kk < 4; kk++) s[kk] += wq * (double)v[kk];
-        if (a.Jnu && q < Q && line_ok)
-            a.Jnu[(o * a.L + l) * Q + q] = (double)u * invP * (double)kI0;
-    }
+        for (int i = 0; i < NB; i++) {
+            float v[4];
+            values(i, v);
+            const double wq = lay.bin(i) < Q ? a.weights[lay.bin(i)] : 0.0;
 #pragma unroll
-    for (int kk = 0; kk < 4; kk++)
-        for (int d = LPG / 2; d; d >>= 1) s[kk] += __shfl_down_sync(0xffffffffu, s[kk], d);
-    if (li == 0 && line_ok) {
-        a.J[o * a.L + l] = s[0] * invP * (double)kI0;
-        a.Lout[o * a.L + l] = s[1] * invP;
-        a.Jeff[o * a.L + l] = s[2] * invP * (double)kI0;
-        a.Lc[o * a.L + l] = s[3] * invP;
+            for (int kk = 0; kk < 4; kk++) s[kk] += wq * (double)v[kk];
+        }
+#pragma unroll
+        for (int kk = 0; kk < 4; kk++)
+            for (int d = LPG / 2; d; d >>= 1) s[kk] += __shfl_down_sync(0xffffffffu, s[kk], d);
+        const int l = l0 + lay.line(0);
+        if (lane % LPG == 0 && l < a.L) {
+            a.J[o * a.L + l] = s[0] * invP * (double)kI0;
+            a.Lout[o * a.L + l] = s[1] * invP;
+            a.Jeff[o * a.L + l] = s[2] * invP * (double)kI0;
+            a.Lc[o * a.L + l] = s[3] * invP;
+        }
+    } else {
+        // every lane has every line: 4 G sums over the warp, halving the number of sums a lane
+        // carries with each step of the exchange (4 G additions in place of 20 G)
+        constexpr int M = 4 * G;
+        double s[M];
+#pragma unroll
+        for (int t = 0; t < M; t++) s[t] = 0.0;
+#pragma unroll
+        for (int i = 0; i < NB; i++) {
+            float v[4];
+            values(i, v);
+            const double wq = lay.bin(i) < Q ? a.weights[lay.bin(i)] : 0.0;
+#pragma unroll
+            for (int kk = 0; kk < 4; kk++) s[4 * (i % G) + kk] += wq * (double)v[kk];
+        }
+        int m = M;
+#pragma unroll
+        for (int d = 16; d; d >>= 1) {
+            if (m > 1) {
+                m >>= 1;
+                const bool up = lane & d;
+#pragma unroll
+                for (int t = 0; t < M / 2; t++)
+                    if (t < m) {
+                        const double keep = up ? s[t + m] : s[t], give = up ? s[t] : s[t + m];
+                        s[t] = keep + __shfl_xor_sync(0xffffffffu, give, d);
+                    }
+            } else {
+                s[0] += __shfl_xor_sync(0xffffffffu, s[0], d);
+            }
+        }
+        const int t = lane / (32 / M), l = l0 + t / 4, kk = t % 4;   // (M <= 32)
+        if (lane % (32 / M) == 0 && l < a.L) {
+            double *dst = kk == 0 ? a.J : (kk == 1 ? a.Lout : (kk == 2 ? a.Jeff : a.Lc));
+            dst[o * a.L + l] = s[0] * invP * (kk % 2 == 0 ? (double)kI0 : 1.0);
+        }
     }
 }
 
-template <int G, int NB, int MINB, int W>
+// The layout of a shape: lines on every lane where the bins fill whole warps.
+template <int G, int NB, bool LINES>
+struct LayoutOf {
+    using type = BinLanes<G, NB>;
+};
+template <int G, int NB>
+struct LayoutOf<G, NB, true> {
+    using type = LineLanes<G, NB>;
+};
+
+template <int G, int NB, int MINB, int W, bool LINES>
 __global__ void __launch_bounds__(32 * W, MINB) k_feautrier_warp(MixArgs a) {
+    using Lay = typename LayoutOf<G, NB, LINES>::type;
     __shared__ Ring rgs[W];
-    __shared__ float4 rls[W][G * kRing];
+    __shared__ float4 rls[W][Lay::kRingLines * kRing];
     __shared__ ElemWin<G> ews[W];
     __shared__ PairSmem<NB> pss[W];
     const int warp = threadIdx.x >> 5;
@@ -961,7 +1189,7 @@ __global__ void __launch_bounds__(32 * W, MINB) k_feautrier_warp(MixArgs a) {
     if (item >= a.n * ngroups) return;
     const int64_t o = item / ngroups;
     const int l0 = (int)(item - o * ngroups) * G;
-    solve_item<G, NB>(a, o, l0, rgs[warp], rls[warp], ews[warp], pss[warp]);
+    solve_item<Lay>(a, o, l0, rgs[warp], rls[warp], ews[warp], pss[warp]);
 }
 
 // Persistent variant over a batch of models: every warp takes work items (model, origin,
@@ -972,12 +1200,13 @@ struct BatchItem {
     int32_t local;   // origin * L + first line of the warp's line group
 };
 
-template <int G, int NB, int MINB, int W>
+template <int G, int NB, int MINB, int W, bool LINES>
 __global__ void __launch_bounds__(32 * W, MINB)
 k_feautrier_batch(const MixArgs *__restrict__ models, const BatchItem *__restrict__ items, int64_t n_items,
                   unsigned long long *counter, const int32_t *__restrict__ active, int32_t skip) {
+    using Lay = typename LayoutOf<G, NB, LINES>::type;
     __shared__ Ring rgs[W];
-    __shared__ float4 rls[W][G * kRing];
+    __shared__ float4 rls[W][Lay::kRingLines * kRing];
     __shared__ ElemWin<G> ews[W];
     __shared__ PairSmem<NB> pss[W];
     __shared__ MixArgs sa[W];
@@ -998,7 +1227,7 @@ k_feautrier_batch(const MixArgs *__restrict__ models, const BatchItem *__restric
         const MixArgs &a = sa[warp];
         const int64_t o = it.local / a.L;
         const int l0 = (int)(it.local - o * a.L);
-        solve_item<G, NB>(a, o, l0, rgs[warp], rls[warp], ews[warp], pss[warp]);
+        solve_item<Lay>(a, o, l0, rgs[warp], rls[warp], ews[warp], pss[warp]);
     }
 }
 
@@ -1011,8 +1240,10 @@ struct WarpVariant {
     void (*fn)(MixArgs);
     void (*batch)(const MixArgs *, const BatchItem *, int64_t, unsigned long long *, const int32_t *, int32_t);
 };
-#define MG_VARIANT_W(G, NB, M, S, W) \
-    {G, NB, M, S, W, k_feautrier_warp<G, NB, M, W>, k_feautrier_batch<G, NB, M, W>}
+// (the shapes whose NB/G bins per lane and line fill 32-bin rounds take LineLanes)
+#define MG_VARIANT_L(G, NB, M, S, W, L) \
+    {G, NB, M, S, W, k_feautrier_warp<G, NB, M, W, L>, k_feautrier_batch<G, NB, M, W, L>}
+#define MG_VARIANT_W(G, NB, M, S, W) MG_VARIANT_L(G, NB, M, S, W, ((G) % 2 == 0 && (NB) % (G) == 0))
 #define MG_VARIANT(G, NB, M, S) MG_VARIANT_W(G, NB, M, S, kWarps2)
 const WarpVariant kWarpVariants[] = {
     // with far-wing skipping
@@ -1041,6 +1272,7 @@ const WarpVariant kWarpVariants[] = {
 };
 #undef MG_VARIANT
 #undef MG_VARIANT_W
+#undef MG_VARIANT_L
 constexpr int kNumWarpVariants = sizeof(kWarpVariants) / sizeof(kWarpVariants[0]);
 
 // Far-wing skipping leaves out the floored intervals of far points. Each changes the
@@ -1176,9 +1408,9 @@ static int launch_mixed(mg_ctx *ctx, int variant) {
 }
 
 // Default launch variant for a model. A warp's time grows with its bins per lane and has a
-// share that does not (staging, windows, pair ends): measured per line group on a disc of 31
-// bins 1.13 ms at 1 line x 1 bin, 1.06 ms at 2 x 2 and 0.83 ms at 4 x 4 per line, and with 63
-// bins 13.8 ms, 10.6 ms and 9.9 ms per line at 1 x 2, 2 x 4 and 4 x 8: proportional to NB +
+// share that does not (staging, windows, pair ends): measured per line on a disc of 31 bins
+// 1.14 ms at 1 line x 1 bin, 1.03 ms at 2 x 2 and 0.80 ms at 4 x 4, and with 63 bins 13.6 ms,
+// 10.1 ms and 9.0 ms at 1 x 2, 2 x 4 and 4 x 8: within a tenth of proportional to NB +
 // 1.6 per group in all six. The default takes the shape with the smallest ceil(L/G) (NB +
 // 1.6): 4 lines x 4 bins (8 for 33-64 bins) for most numbers of lines, two lines per warp
 // where four would leave half of the last warp idle (5, 6 lines). Among equal shapes the
