@@ -1409,7 +1409,7 @@ static int launch_mixed(mg_ctx *ctx, int variant) {
 
 // Default launch variant for a model. A warp's time grows with its bins per lane and has a
 // share that does not (staging, windows, pair ends): measured per line on a disc of 31 bins
-// 1.14 ms at 1 line x 1 bin, 1.03 ms at 2 x 2 and 0.80 ms at 4 x 4, and with 63 bins 13.6 ms,
+// 1.62 ms at 1 line x 1 bin, 1.03 ms at 2 x 2 and 0.80 ms at 4 x 4, and with 63 bins 13.6 ms,
 // 10.1 ms and 9.0 ms at 1 x 2, 2 x 4 and 4 x 8: within a tenth of proportional to NB +
 // 1.6 per group in all six. The default takes the shape with the smallest ceil(L/G) (NB +
 // 1.6): 4 lines x 4 bins (8 for 33-64 bins) for most numbers of lines, two lines per warp
