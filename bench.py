@@ -782,10 +782,6 @@ def run_image(args):
                "cell_channel_updates_per_s": updates / kernel_s, "max_I": float(I.max()), "min_I": float(I.min())}
         imgs[prec] = I
         if prec == mg.MG_FP64:
-            # FP64 bound per point-channel update at the measured pipe rates of this GPU: three
-            # exponentials (profile, exp(-dtau), expm1), two divisions, ~30 DFMA-pipe operations
-            bound_s = updates * (3 / 31e9 + 2 / 66e9 + 30 / 0.50e12)
-            rec.update(fp64_bound_ms=bound_s * 1e3, fraction_of_fp64_bound=bound_s / kernel_s)
             out["fp64"] = rec
         else:
             out["fp32"] = rec

@@ -323,7 +323,7 @@ typedef struct {
 int mg_iterate(mg_ctx *ctx, mg_ali_report *rep);
 
 /* Autotuner of the mixed-precision formal solve: times every launch variant of the
- * Feautrier kernel that suits the model (lines per warp 1/2/4, bins per lane 1/2/4/8,
+ * Feautrier kernel that suits the model (lines per warp 1/2/4, 1 to 8 results per lane,
  * blocks per SM, warps per block, far-wing skipping on or off; 40 variants, indices 0-39,
  * those valid for the model's lines and bins tried; CUDA events, best of reps launches
  * after one warm-up) on the current populations,

@@ -637,7 +637,7 @@ __device__ __forceinline__ void bin_results(const BinState<NB> &st, float (&pi)[
 // for all G lines: per pair and point 9 packed ops, 2 rcp and 4 max/min, and per point and
 // bin 2 ops, one ex2 and a copy, against 11 packed ops, 2 ex2, 2 rcp and 4 max/min per pair
 // in BinLanes. Points of the ring carry (X, X, S, S) of a line pair without duplicates.
-// Measured, BinLanes -> LineLanes: disc 20k (19 lines x 63 bins, G = 4, NB = 8) 197.5 -> 180.6 ms;
+// Measured, BinLanes -> LineLanes: disc of 32k cells (19 lines x 63 bins, G = 4, NB = 8) 197.5 -> 180.6 ms;
 // clumpy 50k (4 x 31, G = 4, NB = 4) 9.07 -> 8.69 ms.
 template <int G_, int NB_>
 struct BinLanes {
