@@ -233,6 +233,13 @@ struct MgTimed {
     ~MgTimed();
 };
 
+// Largest optical depth that the floors alone give a ray pair: chi_min over the longest path
+// through the model and dtau_min in each of its intervals. Kernels leave out intervals at the
+// floors only where this is below what their precision resolves.
+inline double mg_floor_depth(const mg_ctx *ctx) {
+    return ctx->opt.chi_min * ctx->extent + ctx->opt.dtau_min * (double)ctx->max_pair_len;
+}
+
 // ---------------------------------------------------------------- launchers
 int mg_launch_trace(mg_ctx *ctx);
 void mg_pool_retain(int device);    // the device's scratch pool (trace.cu), one reference per context

@@ -17,8 +17,9 @@
 //   divisions of the staging.
 // - S = eta/chi of a line does not depend on the bin: one division per staged point.
 // - A point whose own and two previous points are far (opacity below chi_min and emission
-//   below chi_min times the boundary intensity) changes the sweep by O(chi_min ds) and is left
-//   out while chi_min times the longest path through the model stays below 1e-14 (`skip`):
+//   below chi_min times the boundary intensity) changes the sweep by O(max(chi_min ds, dtau_min))
+//   and is left out while the optical depth that the two floors give a whole ray pair (chi_min
+//   times the longest path through the model, dtau_min per interval) is below 1e-14 (`skip`):
 //   whole elements before they are staged, points far in every bin of the warp before they
 //   reach the ring, and the rest bin by bin, each lane sweeping its own points.
 //

@@ -12,8 +12,8 @@
 // channel, with the points next to them, and walks through its own list; the warp runs as
 // long as its busiest channel. (Over 32 points at a time that saves nothing: they span ten
 // widths, the reach of a channel, and keep some lane busy at each of them.) An interval between two points below that changes the
-// intensity by O(chi_min ds) of the boundary intensity; the lists are used while chi_min times
-// the longest path through the model stays below 1e-14.
+// intensity by O(max(chi_min ds, dtau_min)) of the boundary intensity; the lists are used while
+// the optical depth of the two floors over a whole pair stays below 1e-14.
 //
 // FP64. The FP64 pipe (64-80 cycles per warp instruction) bounds it: per listed point x',
 // (chi_prev + chi) h (2) and the linear-source step (3) are FP64; the exponentials, the

@@ -661,7 +661,7 @@ static int launch_fp64(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount,
         };
         A.cmin = host_pos(a.chi_min);
         A.half_dmin = host_pos(0.5 * a.dtau_min);
-        A.skip = ctx->opt.chi_min * ctx->extent < 1e-14;
+        A.skip = mg_floor_depth(ctx) < 1e-14;
         // A unit is a warp with a chunk of bins and a share of the ray pairs. A CTA has up to
         // 8 units: every chunk, and several groups of pairs when the chunks are few, balanced
         // over the rounds each unit makes. Fewer origins than four waves of two CTAs per SM
@@ -816,7 +816,7 @@ int mg_launch_image(mg_ctx *ctx, int ray, int line, int n_ch, const double *d_u,
         a.lf[i].ic = std::ilogb(2.0 * kH * nu * nu * nu / (kC * kC) / std::expm1(kH * nu / (kKB * s.T_cmb)));
     }
     const size_t smem = sizeof(double) * (size_t)s.kmax * 4 + sizeof(int32_t) * 2 * (size_t)s.kmax;
-    const int skip = ctx->opt.chi_min * ctx->extent < 1e-14;
+    const int skip = mg_floor_depth(ctx) < 1e-14;
     // points staged at a time: a quarter more than the mean pair (more would cost occupancy)
     const double mean = 2.0 * (double)ctx->n_expanded / ((double)ctx->n * ctx->R) + 1.0;
     const int cap = std::min({kImgCap, ((int)(1.25 * mean) + 63) / 32 * 32, (s.kmax + 31) / 32 * 32});

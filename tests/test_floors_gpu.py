@@ -1,0 +1,75 @@
+"""The floors of the transfer and a dark boundary, against the oracle: an optical-depth floor
+`dtau_min` that counts in every interval, and a boundary intensity that underflows to zero,
+against which any emission counts. FP64 within 1e-10 (the step, both band widths, scattering,
+images), mixed precision within 1e-4."""
+import numpy as np
+import pytest
+
+import synthetic as syn
+from oracle import Oracle
+from helpers import rel_err, gpu_context
+
+pytestmark = pytest.mark.gpu
+TOL = {0: 1e-10, 1: 1e-4}
+KINDS = ["step", "band1", "band2", "scatter", "image"]
+
+
+def _cloud():
+    return syn.model_clumpy_3d(n=150, seed=3, n_lev=3, nside=1)
+
+
+def _invert(p):
+    q = p.copy()
+    q[:, 1] = 40.0 * q[:, 0]
+    return q
+
+
+def _check(m, kind, pops=None, precision=0, **opts):
+    """One result of the kind, from LTE populations or pops(LTE populations)."""
+    tol = TOL[precision]
+    band = int(kind[4:]) if kind.startswith("band") else 0
+    o = Oracle(m, nthreads=16, **{k: v for k, v in opts.items() if k in ("chi_min", "dtau_min", "T_cmb")})
+    p0 = o.lte() if pops is None else pops(o.lte())
+    ctx = gpu_context(m, oracle_dirs=o.dirs, precision=precision, spectrum=1, alo_band=band, **opts)
+    ctx.trace_rays()
+    ctx.set_populations(p0)
+    if kind == "image":
+        u = np.linspace(-1.1e4, 1.1e4, 65)
+        for line in range(m.species.n_lines):
+            I, _ = ctx.image(5, line, u)
+            Io, _ = o.image(p0, 5, line, u)
+            assert np.max(rel_err(I, Io)) < tol
+        return
+    if kind == "scatter":
+        xs = 3e-14 * m.n_coll / m.n_coll.max()
+        ctx.set_scattering(xs, tol=1e-30, max_iter=3)
+        Jo, Lo, Eo, Sp, _ = o.formal_solve_scattering(p0, xs, tol=1e-30, max_iter=3)
+    elif band:
+        Jo, Lo, Eo, Mo = o.formal_solve_band(p0, band)
+    else:
+        Jo, Lo, Eo, Sp = o.formal_solve(p0, None, spectrum=True)
+    ctx.formal_solve()
+    J, L, E = ctx.get_radiation()
+    if band:
+        Jb, M = ctx.get_band_terms()
+        for b in range(band):
+            assert np.max(rel_err(Jb[b], Eo[b + 1], floor=1e-300)) < tol
+        assert np.max(rel_err(M, Mo, floor=1e-300)) < tol
+        Eo = Eo[0]
+    else:
+        assert np.max(rel_err(ctx.get_spectrum(), Sp)) < tol
+    assert np.max(rel_err(J, Jo)) < tol
+    if precision == 0:
+        assert np.max(rel_err(E, Eo, floor=1e-300)) < tol and np.max(rel_err(L, Lo, floor=1e-300)) < tol
+
+
+@pytest.mark.parametrize("dtau_min", [1e-12, 1e-9, 1e-6])
+@pytest.mark.parametrize("kind", KINDS)
+def test_optical_depth_floor(kind, dtau_min):
+    """Every interval has at least the optical depth dtau_min, those of far points too."""
+    _check(_cloud(), kind, dtau_min=dtau_min)
+
+
+def test_optical_depth_floor_of_promoted_cells():
+    """Cells solved again in FP64 in a mixed-precision context: all of them here."""
+    _check(_cloud(), "step", precision=1, dtau_min=1e-3, tau_fp64=1.000001)
