@@ -36,6 +36,11 @@ namespace {
 
 constexpr float kLog2e64 = 1.4426950408889634f;
 
+// Least exponent of a boundary intensity: Planck's function is exactly 0 beyond h nu = 710 k T
+// (ilogb(0) is INT_MIN). Every emissivity lies above chi_min times 2^-2000, so any emission
+// counts against a dark boundary.
+constexpr int kDarkExp = -2000;
+
 // Larger of two non-negative doubles, on their bits.
 __device__ __forceinline__ double pos_max(double a, double b) {
     return __double_as_longlong(a) > __double_as_longlong(b) ? a : b;
@@ -516,7 +521,7 @@ __global__ void __launch_bounds__(512) k_feautrier64w(Sweep64 A) {
         // floor test (see the staging): exponents of chi_min nu / 2^28 and of the boundary
         // intensity, rounded down
         __syncwarp();
-        if (lane < nl) W.ic[lane] = ilogb(planck_d(a.lc[l0 + lane].nu, a.T_cmb));
+        if (lane < nl) W.ic[lane] = max(ilogb(planck_d(a.lc[l0 + lane].nu, a.T_cmb)), kDarkExp);
         const int chi_min_e = ilogb(a.chi_min) + ilogbf(nu_lo) - 28 - 1;
         // the origin's opacity and source in this bin
         const double x0 = aq * ibo;

@@ -813,7 +813,8 @@ int mg_launch_image(mg_ctx *ctx, int ray, int line, int n_ch, const double *d_u,
         a.lf[i].dnl = (float)v.dnl;
         a.lf[i].nrm = (float)v.inv_nu2 * (float)(kC / kSqrtPi);
         a.lf[i].cm = std::ilogb(s.chi_min) + std::ilogb(nu) - 28 - 1;
-        a.lf[i].ic = std::ilogb(2.0 * kH * nu * nu * nu / (kC * kC) / std::expm1(kH * nu / (kKB * s.T_cmb)));
+        a.lf[i].ic = std::max(std::ilogb(2.0 * kH * nu * nu * nu / (kC * kC) / std::expm1(kH * nu / (kKB * s.T_cmb))),
+                              kDarkExp);
     }
     const size_t smem = sizeof(double) * (size_t)s.kmax * 4 + sizeof(int32_t) * 2 * (size_t)s.kmax;
     const int skip = mg_floor_depth(ctx) < 1e-14;
