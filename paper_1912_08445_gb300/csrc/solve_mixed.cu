@@ -105,7 +105,8 @@ struct MixArgs {
     const int32_t *ovl_off;
     const Overlap *ovl;
     float chi_min, dtau_min, inv_chi_min;
-    float q_nofloor;             // q' = chi_min ds/(2 sqrt 2) from which 2 q' >= dtau_min in FP32
+    float delta_min;             // dtau_min / sqrt 2
+    float q_nofloor;             // q' = chi_min ds/(2 sqrt 2) from which 2 q' >= delta_min in FP32
     float qscale;                // chi_min/(2 sqrt 2): q' of an interval per unit length
     float planck_a, planck_b;    // B'(nu) = a nu_G^3 / expm1(b nu_G): a = 2h 1e27/c^2/I0, b = h 1e9/(k T_cmb)
     double *J, *Lout, *Jeff, *Lc, *Jnu;
@@ -438,7 +439,8 @@ __device__ __forceinline__ void win_gathers(const MixArgs &a, int l0, ElemWin<G>
 
 // Scalars of the sweep, held in registers (not re-read from the argument block).
 struct SweepK {
-    float dtau_min, planck_a, planck_b;
+    float dmin;              // floor of delta = dtau/sqrt 2
+    float planck_a, planck_b;
 };
 
 // B_nu / I0 at nu_g GHz; e^x - 1 from one ex2 (x = h nu / k T_cmb is O(1) at line
@@ -578,7 +580,7 @@ __device__ __forceinline__ void step_point(const SweepK &k, BinState<NB> &st, co
         const float2 chi = make_float2(fmaxf(chil.x, 1.0f), fmaxf(chil.y, 1.0f));
         const float2 Sx = __fmul2_rn(S, make_float2(fminf(chil.x, 1.0f), fminf(chil.y, 1.0f)));
         const float2 d0 = __fmul2_rn(__fadd2_rn(st.chi_p2[p], chi), qp);
-        const float2 dl = FLOOR ? make_float2(fmaxf(d0.x, k.dtau_min), fmaxf(d0.y, k.dtau_min)) : d0;
+        const float2 dl = FLOOR ? make_float2(fmaxf(d0.x, k.dmin), fmaxf(d0.y, k.dmin)) : d0;
         const float2 sm = __fadd2_rn(st.d_p2[p], dl);
         st.Phi2[p] = __ffma2_rn(st.Phi2[p], st.iota2[p], sm);
         const float2 den = __ffma2_rn(dl, st.Phi2[p], make_float2(1.0f, 1.0f));
@@ -594,7 +596,7 @@ __device__ __forceinline__ void step_point(const SweepK &k, BinState<NB> &st, co
         const float chi = fmaxf(chil, 1.0f);
         const float Sx = S.x * fminf(chil, 1.0f);
         const float d0 = (st.chi_p1 + chi) * qp.x;
-        const float dl = FLOOR ? fmaxf(d0, k.dtau_min) : d0;
+        const float dl = FLOOR ? fmaxf(d0, k.dmin) : d0;
         const float sm = st.d_p1 + dl;
         st.Phi1 = fmaf(st.Phi1, st.iota1, sm);
         st.iota1 = rcpf(fmaf(dl, st.Phi1, 1.0f));
@@ -772,7 +774,7 @@ struct LineLanes {
         const float2 chi = make_float2(fmaxf(chil.x, 1.0f), fmaxf(chil.y, 1.0f));
         const float2 Sx = __fmul2_rn(make_float2(D.z, D.w), make_float2(fminf(chil.x, 1.0f), fminf(chil.y, 1.0f)));
         const float2 d0 = __fmul2_rn(__fadd2_rn(chi_p[p], chi), q);
-        const float2 dl = FLOOR ? make_float2(fmaxf(d0.x, k.dtau_min), fmaxf(d0.y, k.dtau_min)) : d0;
+        const float2 dl = FLOOR ? make_float2(fmaxf(d0.x, k.dmin), fmaxf(d0.y, k.dmin)) : d0;
         const float2 sm = __fadd2_rn(d_p[p], dl);
         Phi[p] = __ffma2_rn(Phi[p], iota[p], sm);
         const float2 den = __ffma2_rn(dl, Phi[p], make_float2(1.0f, 1.0f));
@@ -1029,7 +1031,7 @@ __device__ __forceinline__ void solve_item(const MixArgs &a, int64_t o, int l0, 
     // ring entry of the origin (v = 0 there): a = (g_z, g_z, -0, -0)
     const float gzo = kSqrtLog2e * ibo;
     const float4 Ao = make_float4(gzo, gzo, -0.0f, -0.0f);
-    const SweepK k{a.dtau_min, a.planck_a, a.planck_b};
+    const SweepK k{a.delta_min, a.planck_a, a.planck_b};
     Lay lay;
     lay.init(a, o, l0, bo, ibo);
     // range of a_q over the whole warp (all lanes, all bins)
@@ -1355,8 +1357,9 @@ static void fill_args(mg_ctx *ctx, MixArgs &a) {
     a.chi_min = (float)ctx->opt.chi_min; a.dtau_min = (float)ctx->opt.dtau_min;
     a.inv_chi_min = (float)(1.0 / ctx->opt.chi_min);
     // Every floored opacity is >= 1 in units of chi_min, so an interval with
-    // q' >= q_nofloor has dtau/sqrt 2 = (chi'_prev + chi') q' >= dtau_min: the floor
+    // q' >= q_nofloor has delta = dtau/sqrt 2 = (chi'_prev + chi') q' >= delta_min: the floor
     // cannot bind there.
+    a.delta_min = (float)(ctx->opt.dtau_min / 1.4142135623730951);
     a.q_nofloor = std::nextafter((float)(ctx->opt.dtau_min / 2.0) * 1.000001f, INFINITY);
     a.qscale = (float)(ctx->opt.chi_min * (double)kInvSqrt8);
     a.planck_a = (float)(2.0 * kH * 1e27 / (kC * kC) / (double)kI0);

@@ -87,3 +87,18 @@ def test_dark_boundary(kind, inverted, T_cmb):
     opacity is at the floor) too. (Inverted lines without scattering: their opacity would
     cancel against it.)"""
     _check(_cloud(), kind, _invert if inverted else None, T_cmb=T_cmb, scattering=0.0 if inverted else 3e-14)
+
+
+@pytest.mark.parametrize("dtau_min", [1e-4, 1e-2])
+@pytest.mark.parametrize("variant", [13, 15])   # one line, and two, per warp; every point swept
+def test_optical_depth_floor_of_every_interval_mixed(variant, dtau_min):
+    m = _cloud()
+    o = Oracle(m, nthreads=16, dtau_min=dtau_min)
+    Jo, Lo, Eo, Sp = o.formal_solve(o.lte(), None, spectrum=True)
+    ctx = gpu_context(m, oracle_dirs=o.dirs, precision=1, spectrum=1, dtau_min=dtau_min)
+    ctx.trace_rays()
+    ctx.init_populations()
+    ctx.set_variant(variant)
+    ctx.formal_solve()
+    assert np.max(rel_err(ctx.get_radiation()[0], Jo)) < TOL[1]
+    assert np.max(rel_err(ctx.get_spectrum(), Sp)) < TOL[1]
