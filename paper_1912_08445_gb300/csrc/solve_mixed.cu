@@ -826,7 +826,7 @@ struct LineLanes {
 // wings of every line of its group that the opacity is floored there: X 2^(-x'^2) <
 // chi_min over the warp's range of a_q (x' is monotonic in a_q, so the smallest |x'| is at
 // an end of the range or zero). A point whose own and two previous points are all far
-// changes the state by O(chi_min ds) only (no-ops in FP32) and is left out; rows that
+// changes the state by O(max(chi_min ds, dtau_min)) only and is left out; rows that
 // involve a non-floored interval are still computed exactly. Most far points are left out
 // before they are staged, a whole element at a time: each lane tests one element of the
 // window (|x'| bounded from below by the ends of its velocity range over the larger width,
@@ -1278,10 +1278,10 @@ const WarpVariant kWarpVariants[] = {
 constexpr int kNumWarpVariants = sizeof(kWarpVariants) / sizeof(kWarpVariants[0]);
 
 // Far-wing skipping leaves out the floored intervals of far points. Each changes the
-// sweep by O(chi_min ds), below FP32 resolution only while the floored optical depth of
-// a whole ray, chi_min times the longest path through the model, is; otherwise (a large
-// opacity floor) the variant's non-skipping twin runs instead.
-bool skip_allowed(const mg_ctx *ctx) { return ctx->opt.chi_min * ctx->extent < 1e-7; }
+// sweep by O(max(chi_min ds, dtau_min)), below FP32 resolution only while the optical depth
+// that the floors give a whole ray pair is; otherwise (a large floor) the variant's
+// non-skipping twin runs instead.
+bool skip_allowed(const mg_ctx *ctx) { return mg_floor_depth(ctx) < 1e-7; }
 
 int no_skip_twin(int v) {
     const WarpVariant &w = kWarpVariants[v];

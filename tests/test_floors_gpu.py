@@ -102,3 +102,19 @@ def test_optical_depth_floor_of_every_interval_mixed(variant, dtau_min):
     ctx.formal_solve()
     assert np.max(rel_err(ctx.get_radiation()[0], Jo)) < TOL[1]
     assert np.max(rel_err(ctx.get_spectrum(), Sp)) < TOL[1]
+
+
+@pytest.mark.parametrize("dtau_min", [1e-4, 1e-2])
+def test_optical_depth_floor_mixed(dtau_min):
+    """The default launch shape, then every shape with and without far-wing skipping."""
+    m = _cloud()
+    _check(m, "step", precision=1, dtau_min=dtau_min)
+    o = Oracle(m, nthreads=16, dtau_min=dtau_min)
+    Jo = o.formal_solve(o.lte())[0]
+    ctx = gpu_context(m, oracle_dirs=o.dirs, precision=1, dtau_min=dtau_min)
+    ctx.trace_rays()
+    ctx.init_populations()
+    for v in range(40):
+        ctx.set_variant(v)
+        ctx.formal_solve()
+        assert np.max(rel_err(ctx.get_radiation()[0], Jo)) < TOL[1], v
