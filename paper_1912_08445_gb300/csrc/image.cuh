@@ -32,7 +32,7 @@ struct ImgStage64 {
     double *h;                   // [cap] half the path length from the point before
     double *gz, *ngy, *S;        // [NOV][cap] x' = u gz + ngy
     uint64_t *Xm, *Ym;           // opacity, and emissivity over chi_min, at line centre
-    int32_t *Xe, *Ye;            // (Ye: 2 e + sign)
+    int32_t *Xe, *Ye;            // exponents (2 e + sign, but for Xe of a single line: e)
     uint32_t *todo;              // [cap/32][threads]
     static __host__ __device__ size_t bytes(int cap, int threads) {
         return (size_t)cap * (8 + NOV * (16 + 24 + 16 + 8)) + (size_t)cap / 32 * threads * 4;
@@ -252,14 +252,16 @@ __global__ void __launch_bounds__(256) k_image64_lines(ImageArgs a, int skip, in
                     const double2 p1 = reinterpret_cast<const double2 *>(s.line)[(int64_t)q.c * s.L + ov.l2];
                     const double et = (1.0 - wt) * p0.x + wt * p1.x, ch = (1.0 - wt) * p0.y + wt * p1.y;
                     const double nrm = ov.inv_nu2 * ib * kCsp;
-                    const PosFp X = ch > 0.0 ? pos_from(ch * nrm) : PosFp{0, -(1 << 20)};
+                    // (a negative opacity alone ends at the floor; several lines add up first)
+                    const PosFp X = NOV > 1 ? pos_from(fabs(ch * nrm))
+                                            : (ch > 0.0 ? pos_from(ch * nrm) : PosFp{0, -(1 << 20)});
                     const PosFp Y = pos_from(et * nrm * inv_chi_min);
                     // x' = (dnl + rat (u (1 - w/c) - w)) / b
                     const double gzl = ov.rat * gz, ngl = ov.dnl * ib - ov.rat * gy;
                     T.gz[i * cap + t] = gzl;
                     T.ngy[i * cap + t] = ngl;
                     T.Xm[i * cap + t] = X.m;
-                    T.Xe[i * cap + t] = X.e;
+                    T.Xe[i * cap + t] = NOV > 1 ? 2 * X.e + (ch < 0.0 ? 1 : 0) : X.e;
                     T.Ym[i * cap + t] = Y.m;
                     T.Ye[i * cap + t] = 2 * Y.e + (et < 0.0 ? 1 : 0);
                     double S = 0.0;
@@ -268,7 +270,8 @@ __global__ void __launch_bounds__(256) k_image64_lines(ImageArgs a, int skip, in
                         if (et < 0.0) S = -S;
                     }
                     T.S[i * cap + t] = S;
-                    const int ech = max(__double2hiint(p0.y), __double2hiint(p1.y)) >> 20;
+                    const int sgn = NOV > 1 ? 0x7fffffff : -1;   // (alone, a negative opacity is below every other)
+                    const int ech = max(__double2hiint(p0.y) & sgn, __double2hiint(p1.y) & sgn) >> 20;
                     const int eet = max(__double2hiint(p0.x) & 0x7fffffff, __double2hiint(p1.x) & 0x7fffffff) >> 20;
                     const float bound = (float)(max(max(ech, eet - a.lf[i].ic) - 1022, -100000) + eb - a.lf[i].cm);
                     T.tt[i * cap + t] = make_float4((float)gzl, (float)ngl,
@@ -313,7 +316,8 @@ __global__ void __launch_bounds__(256) k_image64_lines(ImageArgs a, int skip, in
                         if ((__double2hiint(x) & 0x7fffffff) >= 0x404a0000) x = 52.0;   // exp(-52^2) is zero
                         int n;
                         const uint64_t e = exp_neg_sq(x, tab, n);
-                        const PosFp ci = pos_norm(mulhi_near(T.Xm[i * cap + j], e), T.Xe[i * cap + j] + 1 - n);
+                        const int xe = T.Xe[i * cap + j];
+                        const PosFp ci = pos_norm(mulhi_near(T.Xm[i * cap + j], e), (NOV > 1 ? xe >> 1 : xe) + 1 - n);
                         const int ye = T.Ye[i * cap + j];
                         if (NOV == 1) {
                             chi = ci;
@@ -328,11 +332,13 @@ __global__ void __launch_bounds__(256) k_image64_lines(ImageArgs a, int skip, in
                             double ei = pos_pack(mulhi_near(T.Ym[i * cap + j], e), (ye >> 1) + 1 - n);
                             if (ye & 1) ei = -ei;
                             eta += ei;
-                            chis += pos_pack(ci);
+                            double cd = pos_pack(ci);
+                            if (xe & 1) cd = -cd;
+                            chis += cd;
                         }
                     }
                     if (NOV > 1) {
-                        chis = pos_max(chis, s.chi_min);
+                        chis = pos_max(chis, s.chi_min);   // (a negative sum is below it as bits too)
                         chi = pos_from(chis);
                         Sk = eta * s.chi_min * pos_pack(pos_rcp(chi));
                     }
