@@ -55,7 +55,7 @@ struct Warp64 {
     double2 *ln;                 // [nl][32] (eta, chi)
     double *gz, *ngy, *h;        // ring: x' = a_q gz + ngy; h of the interval from the previous point
     uint64_t *Xm, *Ym;           // [nl][32] line opacity X and floored source Y = eta/chi_min at line centre
-    int32_t *Xe, *Ye;            //   (exponents; Ye holds 2 e + sign)
+    int32_t *Xe, *Ye;            //   (exponents; Ye holds 4 e + flags: 1 for Y < 0, 2 for X < 0)
     double *S;                   // [nl][32]
     float4 *tt;                  // [nl][32]: (g_z, -g_y, |x'| beyond which the line is far, -) in FP32
     double *N;                   // ring: profile normalisation without 1/nu (band terms)
@@ -356,12 +356,13 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
                 const double2 p0 = W.ln[32 * k + i + 1], p1 = W.ln[32 * k + i];
                 const double et = (1.0 - w) * p0.x + w * p1.x, ch = (1.0 - w) * p0.y + w * p1.y;
                 const double nrm = a.lc[l0 + k].pnorm * ibk;      // c/(nu sqrt pi) / b
-                const PosFp X = ch > 0.0 ? pos_from(ch * nrm) : PosFp{0, 0};
+                // (a negative opacity alone ends at the floor; scattering opacity adds to it first)
+                const PosFp X = ch > 0.0 || SCAT ? pos_from(fabs(ch * nrm)) : PosFp{0, 0};
                 const PosFp Y = pos_from(et * nrm * A.inv_chi_min);
                 W.Xm[32 * k + j] = X.m;
                 W.Xe[32 * k + j] = X.e;
                 W.Ym[32 * k + j] = Y.m;
-                W.Ye[32 * k + j] = 2 * Y.e + (et < 0.0 ? 1 : 0);
+                W.Ye[32 * k + j] = 4 * Y.e + (et < 0.0 ? 1 : 0) + (SCAT && ch < 0.0 ? 2 : 0);
                 double S = 0.0;
                 if (ch > 0.0) {
                     S = pos_pack(pos_mul(pos_from(et), pos_rcp(pos_from(ch))));
@@ -427,17 +428,18 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
             const double xs = SCAT ? W.xs[j] : 0.0;
             if (SCAT && xs != 0.0) {
                 oth = scattered64(a, roots, l0 + lw, xr, W.w[j], xs, W.ca[j], W.cb[j]);
-                const double c = pos_max(pos_pack(chi.m, chi.e) + xs, a.chi_min);
-                chi = pos_from(c);
-                // line emissivity: Y chi_min e
                 const int ye = Ye[j];
-                double et = pos_pack(mulhi_near(Ym[j], e), (ye >> 1) + 1 - n) * a.chi_min;
+                double cl = pos_pack(chi.m, chi.e);
+                if (ye & 2) cl = -cl;
+                chi = pos_from(pos_max(cl + xs, a.chi_min));   // (a negative sum is below it as bits too)
+                // line emissivity: Y chi_min e
+                double et = pos_pack(mulhi_near(Ym[j], e), (ye >> 2) + 1 - n) * a.chi_min;
                 if (ye & 1) et = -et;
                 S = (et + oth) * pos_pack(pos_rcp(chi));
-            } else if (chi.m == 0 || chi.e < A.cmin.e || (chi.e == A.cmin.e && chi.m < A.cmin.m)) {
+            } else if (chi.m == 0 || chi.e < A.cmin.e || (chi.e == A.cmin.e && chi.m < A.cmin.m) || (SCAT && (Ye[j] & 2))) {
                 chi = A.cmin;
                 const int ye = Ye[j];
-                S = pos_pack(mulhi_near(Ym[j], e), (ye >> 1) + 1 - n);
+                S = pos_pack(mulhi_near(Ym[j], e), (ye >> 2) + 1 - n);
                 if (ye & 1) S = -S;
             }
             if (first && j == 0) {

@@ -29,3 +29,28 @@ def test_image_of_overlapping_lines(n_lev, level):
             I, _ = ctx.image(ray, 0, u)
             Io, _ = o.image(p, ray, 0, u)
             assert np.max(rel_err(I, Io)) < TOL
+
+
+def test_scattering_with_an_inverted_line():
+    """An inverted line's opacity takes from the scattering opacity, by up to a twentieth (so
+    that no sum is ill-conditioned)."""
+    m = syn.model_clumpy_3d(n=150, seed=3, n_lev=3, nside=1)
+    o = Oracle(m, nthreads=16)
+    p = o.lte()
+    p[:, 1] = 3.0 * p[:, 0] * m.species.g[1] / m.species.g[0]
+    h, c = 6.62607015e-34, 299792458.0
+    sp = m.species
+    nu = (sp.E[1] - sp.E[0]) / h
+    Bul = sp.A[0] * c ** 2 / (2 * h * nu ** 3)
+    chi = h * nu / (4 * np.pi) * (p[:, 0] * sp.g[1] / sp.g[0] - p[:, 1]) * Bul
+    peak = chi * c / (nu * np.sqrt(np.pi) * np.array([o.width(k) for k in range(m.n)]))
+    xs = np.full(m.n, 20.0 * np.abs(peak).max())
+    ctx = gpu_context(m, oracle_dirs=o.dirs, precision=0, spectrum=1)
+    ctx.trace_rays()
+    ctx.set_populations(p)
+    ctx.set_scattering(xs, tol=1e-30, max_iter=3)
+    ctx.formal_solve()
+    J, L, E = ctx.get_radiation()
+    Jo, Lo, Eo, Sp, _ = o.formal_solve_scattering(p, xs, tol=1e-30, max_iter=3)
+    assert np.max(rel_err(J, Jo)) < TOL and np.max(rel_err(ctx.get_spectrum(), Sp)) < TOL
+    assert np.max(np.abs(E - Eo) / Jo) < TOL and np.max(np.abs(L - Lo)) < TOL
