@@ -55,7 +55,8 @@ struct Warp64 {
     double2 *ln;                 // [nl][32] (eta, chi)
     double *gz, *ngy, *h;        // ring: x' = a_q gz + ngy; h of the interval from the previous point
     uint64_t *Xm, *Ym;           // [nl][32] line opacity X and floored source Y = eta/chi_min at line centre
-    int32_t *Xe, *Ye;            //   (exponents; Ye holds 4 e + flags: 1 for Y < 0, 2 for X < 0)
+    int32_t *Xe, *Ye;            //   (exponents; Ye holds 8 e + flags: 1 for Y < 0, 2 for X < 0 or NaN, 4
+                                 //   for an emissivity that is not finite, in place of the source in S)
     double *S;                   // [nl][32]
     float4 *tt;                  // [nl][32]: (g_z, -g_y, |x'| beyond which the line is far, -) in FP32
     double *N;                   // ring: profile normalisation without 1/nu (band terms)
@@ -196,6 +197,7 @@ __device__ __forceinline__ float line_bound64(const Warp64 &W, int k, int i, int
     const double2 p0 = W.ln[32 * k + i + 1], p1 = W.ln[32 * k + i];
     const int ech = max(__double2hiint(p0.y), __double2hiint(p1.y));   // (negative: below every positive)
     const int eet = max(__double2hiint(p0.x) & 0x7fffffff, __double2hiint(p1.x) & 0x7fffffff);
+    if (max(ech, eet) >= 0x7ff00000) return INFINITY;                  // (infinite or NaN: never far)
     return (float)(max(max(ech >> 20, (eet >> 20) - W.ic[k]) - 1022, -100000) + eb - chi_min_e);
 }
 
@@ -268,7 +270,7 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
                 float bound = 0.0f;
                 if (el)
                     for (int k2 = 0; k2 < nl; k2++) bound = fmaxf(bound, line_bound64(W, k2, lane, eb, chi_min_e));
-                near = el && !(0.999f * kLog2e64 * xm * xm > bound);
+                near = el && !(0.999f * kLog2e64 * xm * xm > bound && fabsf(vf) + fabsf(v0) < INFINITY);
                 if (B > 0) near = near || (el && x0 < 3);
                 if constexpr (SCAT) near = near || (el && (a.chi_sca[W.cell[lane]] != 0.0 || a.chi_sca[W.cell[lane + 1]] != 0.0));
             }
@@ -362,12 +364,15 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
                 W.Xm[32 * k + j] = X.m;
                 W.Xe[32 * k + j] = X.e;
                 W.Ym[32 * k + j] = Y.m;
-                W.Ye[32 * k + j] = 4 * Y.e + (et < 0.0 ? 1 : 0) + (SCAT && ch < 0.0 ? 2 : 0);
+                const bool bad = not_finite(et) || not_finite(gy);
+                W.Ye[32 * k + j] = 8 * Y.e + (et < 0.0 ? 1 : 0) + (SCAT && !(ch >= 0.0) ? 2 : 0) + (bad ? 4 : 0);
                 double S = 0.0;
                 if (ch > 0.0) {
                     S = pos_pack(pos_mul(pos_from(et), pos_rcp(pos_from(ch))));
                     if (et < 0.0) S = -S;
+                    if (not_finite(ch)) S = ch - ch;
                 }
+                if (bad) S = et * gy;
                 W.S[32 * k + j] = S;
             }
             if constexpr (B > 0) {
@@ -433,14 +438,14 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
                 if (ye & 2) cl = -cl;
                 chi = pos_from(pos_max(cl + xs, a.chi_min));   // (a negative sum is below it as bits too)
                 // line emissivity: Y chi_min e
-                double et = pos_pack(mulhi_near(Ym[j], e), (ye >> 2) + 1 - n) * a.chi_min;
-                if (ye & 1) et = -et;
+                double et = pos_pack(mulhi_near(Ym[j], e), (ye >> 3) + 1 - n) * a.chi_min;
+                if (ye & 5) et = ye & 4 ? S : -et;
                 S = (et + oth) * pos_pack(pos_rcp(chi));
             } else if (chi.m == 0 || chi.e < A.cmin.e || (chi.e == A.cmin.e && chi.m < A.cmin.m) || (SCAT && (Ye[j] & 2))) {
                 chi = A.cmin;
                 const int ye = Ye[j];
-                S = pos_pack(mulhi_near(Ym[j], e), (ye >> 2) + 1 - n);
-                if (ye & 1) S = -S;
+                S = pos_pack(mulhi_near(Ym[j], e), (ye >> 3) + 1 - n);
+                if (ye & 5) S = ye & 4 ? Sr[j] : -S;
             }
             if (first && j == 0) {
                 // the far end: the boundary row starts from Phi iota = 1, psi = I, delta = 0

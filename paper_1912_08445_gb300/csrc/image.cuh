@@ -32,7 +32,8 @@ struct ImgStage64 {
     double *h;                   // [cap] half the path length from the point before
     double *gz, *ngy, *S;        // [NOV][cap] x' = u gz + ngy
     uint64_t *Xm, *Ym;           // opacity, and emissivity over chi_min, at line centre
-    int32_t *Xe, *Ye;            // exponents (2 e + sign, but for Xe of a single line: e)
+    int32_t *Xe, *Ye;            // exponents (Xe: e for a single line, else 2 e + 1 for X < 0 or NaN; Ye: 4 e + flags:
+                                 //   1 for Y < 0, 2 for an emissivity that is not finite, in place of the source in S)
     uint32_t *todo;              // [cap/32][threads]
     static __host__ __device__ size_t bytes(int cap, int threads) {
         return (size_t)cap * (8 + NOV * (16 + 24 + 16 + 8)) + (size_t)cap / 32 * threads * 4;
@@ -261,19 +262,23 @@ __global__ void __launch_bounds__(256) k_image64_lines(ImageArgs a, int skip, in
                     T.gz[i * cap + t] = gzl;
                     T.ngy[i * cap + t] = ngl;
                     T.Xm[i * cap + t] = X.m;
-                    T.Xe[i * cap + t] = NOV > 1 ? 2 * X.e + (ch < 0.0 ? 1 : 0) : X.e;
+                    T.Xe[i * cap + t] = NOV > 1 ? 2 * X.e + (ch >= 0.0 ? 0 : 1) : X.e;
                     T.Ym[i * cap + t] = Y.m;
-                    T.Ye[i * cap + t] = 2 * Y.e + (et < 0.0 ? 1 : 0);
+                    const bool bad = not_finite(et) || not_finite(gy);
+                    T.Ye[i * cap + t] = 4 * Y.e + (et < 0.0 ? 1 : 0) + (bad ? 2 : 0);
                     double S = 0.0;
                     if (ch > 0.0) {
                         S = pos_pack(pos_mul(pos_from(et), pos_rcp(pos_from(ch))));
                         if (et < 0.0) S = -S;
                     }
+                    if (bad) S = et * gy;
                     T.S[i * cap + t] = S;
                     const int sgn = NOV > 1 ? 0x7fffffff : -1;   // (alone, a negative opacity is below every other)
                     const int ech = max(__double2hiint(p0.y) & sgn, __double2hiint(p1.y) & sgn) >> 20;
                     const int eet = max(__double2hiint(p0.x) & 0x7fffffff, __double2hiint(p1.x) & 0x7fffffff) >> 20;
-                    const float bound = (float)(max(max(ech, eet - a.lf[i].ic) - 1022, -100000) + eb - a.lf[i].cm);
+                    const float bound = max(ech, eet) >= 0x7ff   // (infinite or NaN: never far)
+                                            ? INFINITY
+                                            : (float)(max(max(ech, eet - a.lf[i].ic) - 1022, -100000) + eb - a.lf[i].cm);
                     T.tt[i * cap + t] = make_float4((float)gzl, (float)ngl,
                                              skip ? sqrtf(1.001f / kLog2e64 * fmaxf(bound, 0.0f)) +
                                                         1e-6f * fabsf((float)ngl)
@@ -313,7 +318,9 @@ __global__ void __launch_bounds__(256) k_image64_lines(ImageArgs a, int skip, in
 #pragma unroll
                     for (int i = 0; i < NOV; i++) {
                         double x = fma(u, T.gz[i * cap + j], T.ngy[i * cap + j]);
-                        if ((__double2hiint(x) & 0x7fffffff) >= 0x404a0000) x = 52.0;   // exp(-52^2) is zero
+                        const int xh = __double2hiint(x) & 0x7fffffff;
+                        if (xh >= 0x404a0000) x = 52.0;                       // exp(-52^2) is zero
+                        const bool out = xh > 0x403b5025 && xh <= 0x7ff00000;   // x^2 > 746: outside the profile
                         int n;
                         const uint64_t e = exp_neg_sq(x, tab, n);
                         const int xe = T.Xe[i * cap + j];
@@ -324,15 +331,15 @@ __global__ void __launch_bounds__(256) k_image64_lines(ImageArgs a, int skip, in
                             Sk = T.S[i * cap + j];
                             if (chi.m == 0 || chi.e < cmin.e || (chi.e == cmin.e && chi.m < cmin.m)) {
                                 chi = cmin;
-                                Sk = pos_pack(mulhi_near(T.Ym[i * cap + j], e), (ye >> 1) + 1 - n);
-                                if (ye & 1) Sk = -Sk;
+                                Sk = pos_pack(mulhi_near(T.Ym[i * cap + j], e), (ye >> 2) + 1 - n);
+                                if (ye & 3) Sk = ye & 2 ? (out ? 0.0 : T.S[i * cap + j]) : -Sk;
                             }
                         } else {
                             // (the emissivity in units of chi_min)
-                            double ei = pos_pack(mulhi_near(T.Ym[i * cap + j], e), (ye >> 1) + 1 - n);
-                            if (ye & 1) ei = -ei;
+                            double ei = pos_pack(mulhi_near(T.Ym[i * cap + j], e), (ye >> 2) + 1 - n);
+                            if (ye & 3) ei = ye & 2 ? (out ? 0.0 : T.S[i * cap + j]) : -ei;
                             eta += ei;
-                            double cd = pos_pack(ci);
+                            double cd = out ? 0.0 : pos_pack(ci);
                             if (xe & 1) cd = -cd;
                             chis += cd;
                         }

@@ -30,13 +30,16 @@ struct PosFp {
     int e;
 };
 
-// From a non-negative double (subnormals count as zero, whose exponent is below every other).
+// From the magnitude of a double (subnormals count as zero, whose exponent is below every other;
+// infinities and NaN as numbers of 2^1024 and more: callers that can meet them ask `not_finite`).
 __device__ __forceinline__ PosFp pos_from(double x) {
     const uint64_t b = (uint64_t)__double_as_longlong(x);
     const int ex = (int)(b >> 52) & 0x7ff;
     if (ex == 0) return PosFp{0, -(1 << 20)};
     return PosFp{((b << 11) | 0x8000000000000000ull), ex - 1086};   // 1086 = 1023 + 63
 }
+
+__device__ __forceinline__ bool not_finite(double x) { return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000; }
 
 // m 2^e rounded to a double; m may have up to two leading zero bits. Below the smallest
 // normal double the result is 0, beyond the largest it is infinity.
