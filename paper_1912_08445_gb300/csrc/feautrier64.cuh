@@ -118,8 +118,14 @@ struct Sweep64 {
     double dmin;             // dtau_min
     PosFp half_dmin, cmin;   // dtau_min / 2 and chi_min
     double inv_chi_min;
-    double *Mpart;           // band terms: [kl][n][L][R][B] unsummed over chunks
+    int64_t o0, nb;          // origins of this launch: from o0, at most nb
+    double *Mpart;           // band terms of these origins: [kl][nb][L][R][B] unsummed over chunks
 };
+
+// Doubles of scratch for unsummed band terms (1 GiB). A launch covers the origins whose terms
+// fit: two to five times the terms themselves would be 35 GB for 200k points, 19 lines x 63 bins and
+// 192 rays at B = 2. (Those take 33 launches of 6.1k CTAs, 20 waves each.)
+constexpr int64_t kBandScratch = (1ll << 30) / sizeof(double);
 
 // One bin's sweep state and (band terms) its last two rows.
 struct Bin64 {
@@ -488,8 +494,8 @@ __global__ void __launch_bounds__(512) k_feautrier64w(Sweep64 A) {
     // a unit is a warp, or two warps that sweep one half of each pair each
     const int nu = (blockDim.x >> 5) >> A.duo, warp = threadIdx.x >> 5, unit = warp >> A.duo, lane = threadIdx.x & 31;
     const int half = A.duo ? warp & 1 : 2;
-    int64_t o = blockIdx.x / A.split;
-    const int share = blockIdx.x - (int)o * A.split;
+    const int ob = blockIdx.x / A.split, share = blockIdx.x - ob * A.split;
+    int64_t o = A.o0 + ob;
     if (a.olist) {
         if ((int)blockIdx.x >= *a.ocount) return;
         o = a.olist[blockIdx.x];
@@ -670,7 +676,7 @@ __global__ void __launch_bounds__(512) k_feautrier64w(Sweep64 A) {
                     double s = 0.0;
                     for (int ff = f0; ff < f1; ff++) s += W.mac[(ff - 32 * c) * 2 * B + sj];
                     const int side = sj / B, j = sj - side * B, part = c - ll * Q / 32;
-                    A.Mpart[((((size_t)part * a.n + o) * L + ll) * a.R + (side ? rf : rb)) * B + j] = s;
+                    A.Mpart[((((size_t)part * A.nb + ob) * L + ll) * a.R + (side ? rf : rb)) * B + j] = s;
                 }
                 __syncwarp();
             }
@@ -749,17 +755,17 @@ __global__ void __launch_bounds__(128) k_sums64(SolveArgs a, int split, const do
     }
 }
 
-// Coupling terms: the sum over each line's chunks, times chi_int(o)/P.
-__global__ void k_band_terms64(int64_t n, int L, int R, int B, int Q, double invP, const double *part,
-                               const double *line, double *M) {
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, m = n * L * R * B;
+// Coupling terms of a launch's origins (m of them): the sum over each line's chunks, times
+// chi_int(o)/P.
+__global__ void k_band_terms64(Sweep64 A, int64_t m, int L, int R, int B) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, stride = A.nb * L * R * B;
     if (t >= m) return;
-    const int64_t ol = t / (R * B);
-    const int l = (int)(ol % L);
+    const int64_t ol = A.o0 * L + t / (R * B);
+    const int l = (int)(ol % L), Q = A.s.Q;
     const int np = (l * Q + Q - 1) / 32 - l * Q / 32 + 1;
     double s = 0.0;
-    for (int k = 0; k < np; k++) s += part[k * m + t];
-    M[t] = s * invP * line[2 * ol + 1];
+    for (int k = 0; k < np; k++) s += A.Mpart[k * stride + t];
+    A.s.Mb[A.o0 * L * R * B + t] = s * (1.0 / A.s.P) * A.s.line[2 * ol + 1];
 }
 
 }  // namespace

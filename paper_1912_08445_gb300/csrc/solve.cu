@@ -694,23 +694,29 @@ static int launch_fp64(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount,
         while (a.groups == 1 && units > 1 && bytes() > 227 * 1024) units--;
         const int warps = units << A.duo;
         smem = bytes();
-        if (smem <= 227 * 1024) {
-            if (B > 0) {
-                if (ctx->band_part_cap < (int64_t)A.kl * a.n * a.L * a.R * B) {
-                    const int64_t need = (int64_t)A.kl * a.n * a.L * a.R * B;
-                    int rc = mg_alloc(ctx, &ctx->d_Mpart, need);
-                    ctx->band_part_cap = rc ? 0 : need;
-                    if (rc) return rc;
-                }
-                A.Mpart = ctx->d_Mpart;
+        // Scratch. Without room for it the solve goes on without: one CTA per origin, or, for the
+        // band terms, the general kernel.
+        auto scratch = [&](double **p, int64_t *cap, int64_t need) {
+            if (*cap >= need) return true;
+            *cap = 0;
+            if (mg_alloc(ctx, p, need)) {
+                cudaGetLastError();
+                ctx->err.clear();
+                return false;
             }
+            *cap = need;
+            return true;
+        };
+        bool fits = smem <= 227 * 1024;
+        const int64_t per = (int64_t)A.kl * a.L * a.R * B;   // unsummed band terms of an origin
+        A.nb = B > 0 ? std::max<int64_t>(1, std::min<int64_t>(a.n, kBandScratch / per)) : a.n;
+        if (fits && B > 0) {
+            fits = scratch(&ctx->d_Mpart, &ctx->band_part_cap, A.nb * per);
+            A.Mpart = ctx->d_Mpart;
+        }
+        if (fits) {
             if (A.split > 1) {
-                const int64_t need = a.n * A.split * F * (4 + B);
-                if (ctx->part64_cap < need) {
-                    int rc = mg_alloc(ctx, &ctx->d_part64, need);
-                    ctx->part64_cap = rc ? 0 : need;
-                    if (rc) return rc;
-                }
+                if (!scratch(&ctx->d_part64, &ctx->part64_cap, a.n * A.split * F * (4 + B))) A.split = 1;
                 A.part = ctx->d_part64;
             }
             A.s = a;
@@ -718,15 +724,17 @@ static int launch_fp64(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount,
                                         : (B == 0 ? k_feautrier64w<0, false> : (B == 1 ? k_feautrier64w<1, false> : k_feautrier64w<2, false>));
             MG_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kMaxDynSmem));
             MgTimed t(ctx, name);
-            kern<<<grid * A.split, 32 * warps, smem, ctx->stream>>>(A);
+            for (; A.o0 < (int64_t)grid; A.o0 += A.nb) {
+                const int64_t count = std::min<int64_t>(A.nb, grid - A.o0);
+                kern<<<(unsigned)(count * A.split), 32 * warps, smem, ctx->stream>>>(A);
+                if (B > 0) {
+                    const int64_t m = count * a.L * a.R * B;
+                    k_band_terms64<<<(unsigned)((m + 255) / 256), 256, 0, ctx->stream>>>(A, m, a.L, a.R, B);
+                }
+            }
             if (A.split > 1) {
                 void (*sums)(SolveArgs, int, const double *) = B == 0 ? k_sums64<4> : (B == 1 ? k_sums64<5> : k_sums64<6>);
                 sums<<<(unsigned)((a.n * a.L + 3) / 4), 128, 0, ctx->stream>>>(a, A.split, A.part);
-            }
-            if (B > 0) {
-                const int64_t m = a.n * a.L * a.R * B;
-                k_band_terms64<<<(unsigned)((m + 255) / 256), 256, 0, ctx->stream>>>(a.n, a.L, a.R, B, a.Q, 1.0 / a.P,
-                                                                                   A.Mpart, a.line, a.Mb);
             }
             MG_CUDA(cudaGetLastError());
             return MG_OK;
