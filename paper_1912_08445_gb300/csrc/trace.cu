@@ -5,6 +5,7 @@
 #include <algorithm>
 #include <mutex>
 #include "common.cuh"
+#include "kept.h"
 
 using namespace mg;
 
@@ -536,17 +537,13 @@ struct TraceScratch {
     ~TraceScratch() { give_back(); }
 };
 
-// A buffer of the ray store for `count` elements: the one at hand when it is large enough and
-// not more than half empty, else a new one with 3 % to spare for the next trace.
 template <typename T>
 static int ray_buffer(mg_ctx *ctx, T **p, int64_t &cap, int64_t count) {
-    if (*p && cap >= count && cap <= 2 * count + 4096) return MG_OK;
-    cap = 0;
-    const int64_t want = count + count / 32;
-    int rc = mg_alloc(ctx, p, want);
-    if (rc && want > count) rc = mg_alloc(ctx, p, count);
-    if (!rc) cap = rc ? 0 : want;
-    return rc;
+    return kept_buffer(cap, count, [&](int64_t n) {
+        const int rc = mg_alloc(ctx, p, n);
+        if (rc) cudaGetLastError();   // (not the error of a later launch)
+        return rc;
+    });
 }
 
 int mg_launch_trace(mg_ctx *ctx) {
