@@ -36,3 +36,33 @@ def compare_rays(ctx, tr, origins, R):
             if not ok:
                 bad.append((int(o), r))
     return bad
+
+
+class FullDevice:
+    """Holds all device memory but `leave` bytes (to 32 MB; what allocation pools hold unused is
+    taken too) while the block runs."""
+
+    def __init__(self, leave):
+        self.leave = leave
+
+    def __enter__(self):
+        import torch
+        torch.cuda.synchronize()
+        torch.cuda.empty_cache()
+        step = 32 << 20
+        rest = torch.cuda.mem_get_info()[0] - self.leave - (2 << 30)
+        self.held = [torch.empty(rest, dtype=torch.uint8, device="cuda")] if rest > 0 else []
+        try:
+            while True:
+                self.held.append(torch.empty(step, dtype=torch.uint8, device="cuda"))
+        except torch.OutOfMemoryError:
+            pass
+        for _ in range((self.leave + step - 1) // step):
+            self.held.pop()
+        torch.cuda.empty_cache()
+        return self
+
+    def __exit__(self, *exc):
+        import torch
+        self.held.clear()
+        torch.cuda.empty_cache()

@@ -5,7 +5,7 @@ import pytest
 
 import synthetic as syn
 from oracle import Oracle
-from helpers import rel_err, gpu_context
+from helpers import FullDevice, rel_err, gpu_context
 
 pytestmark = pytest.mark.gpu
 TOL = 1e-10
@@ -46,16 +46,9 @@ def test_origins_in_parts(model):
 def test_no_room_for_the_scratch(model):
     """With the memory for the coupling terms themselves and half of the scratch left, the
     solve still succeeds."""
-    import torch
     m, o, origins, want = model
     ctx = _context(m, o)
     terms = m.n * 3072 * 2 * (8 * 4 + 16)      # coupling terms and geometry of the band points
-    torch.cuda.synchronize()
-    free, _ = torch.cuda.mem_get_info()
-    fill = torch.empty(free - terms - (1 << 29), dtype=torch.uint8, device="cuda")
-    try:
+    with FullDevice(terms + (1 << 29)):
         ctx.formal_solve()
         _compare(ctx, origins, want)
-    finally:
-        del fill
-        torch.cuda.empty_cache()
