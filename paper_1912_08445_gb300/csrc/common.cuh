@@ -125,6 +125,7 @@ struct mg_ctx {
     double *d_ds = nullptr;        // path length from the previous point
     double *d_vpar = nullptr;      // line-of-sight velocity relative to the origin
     float *d_dsf = nullptr, *d_vparf = nullptr;
+    bool rays_idle = true;         // no valid rays: their buffers only wait for the next trace
     int64_t ray_off_cap = 0, ray_cap[6] = {0, 0, 0, 0, 0, 0};   // elements the buffers hold
     int64_t n_elements = 0, n_expanded = 0, max_pair_len = 0, n_dead = 0;
     int64_t work_solves = 0, work_updates = 0;
@@ -208,11 +209,14 @@ int mg_cuda_check(const mg_ctx *ctx, cudaError_t e, const char *what);
         if (e_ != cudaSuccess) return mg_cuda_check(ctx, e_, #call);      \
     } while (0)
 
+bool mg_release_idle_rays(mg_ctx *ctx);   // (context.cu) gives back a ray store without valid rays
+
 template <typename T>
 int mg_alloc(mg_ctx *ctx, T **p, size_t count) {
     if (*p) { cudaFree(*p); *p = nullptr; }
     if (count == 0) count = 1;
     cudaError_t e = cudaMalloc((void **)p, count * sizeof(T));
+    if (e != cudaSuccess && mg_release_idle_rays(ctx)) e = cudaMalloc((void **)p, count * sizeof(T));
     if (e != cudaSuccess) {
         *p = nullptr;
         return mg_fail(ctx, MG_ERR_OOM, std::string("cudaMalloc failed: ") + cudaGetErrorString(e));

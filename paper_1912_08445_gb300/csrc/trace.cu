@@ -514,11 +514,15 @@ struct TraceScratch {
             pool = g_pool[c->device];
         }
     }
+    cudaError_t take(void **q, size_t bytes) {
+        return pool ? cudaMallocFromPoolAsync(q, bytes, pool, ctx->stream) : cudaMalloc(q, bytes);
+    }
     template <typename T>
     cudaError_t get(T **p, size_t count) {
         void *q = nullptr;
         const size_t bytes = std::max<size_t>(1, count) * sizeof(T);
-        const cudaError_t e = pool ? cudaMallocFromPoolAsync(&q, bytes, pool, ctx->stream) : cudaMalloc(&q, bytes);
+        cudaError_t e = take(&q, bytes);
+        if (e != cudaSuccess && mg_release_idle_rays(ctx)) e = take(&q, bytes);
         if (e != cudaSuccess) {
             cudaGetLastError();
             return e;
@@ -556,7 +560,8 @@ int mg_launch_trace(mg_ctx *ctx) {
     unsigned *wmax = nullptr;
     cudaError_t ce;
     if ((ce = sc.get(&d_len, nr)) || (ce = sc.get(&d_xlen, nr)) ||
-        (ce = sc.get(&bsum, (nr + kScanBlock - 1) / kScanBlock)) || (ce = sc.get(&wmax, 1)))
+        (ce = sc.get(&bsum, (nr + kScanBlock - 1) / kScanBlock)) || (ce = sc.get(&wmax, 1)) ||
+        (ctx->geometry == MG_GEOM_3D && (ce = sc.get(&posf, ctx->n))))
         return mg_fail(ctx, MG_ERR_OOM, std::string("cudaMalloc failed: ") + cudaGetErrorString(ce));
     // The ray store is written in place: solves and images of the old rays come first. Those
     // of this stream do; after a change of stream, wait for all (as the frees of a replaced
@@ -564,6 +569,11 @@ int mg_launch_trace(mg_ctx *ctx) {
     if (ctx->stream_changed) MG_CUDA(cudaDeviceSynchronize());
     ctx->stream_changed = false;
     ctx->traced = false;
+    struct InUse {           // the store is this trace's until it returns, and then the rays' if it succeeded
+        mg_ctx *c;
+        explicit InUse(mg_ctx *ctx) : c(ctx) { c->rays_idle = false; }
+        ~InUse() { c->rays_idle = !c->traced; }
+    } in_use(ctx);
     if ((rc = ray_buffer(ctx, &ctx->d_ray_off, ctx->ray_off_cap, nr + 1))) return rc;
     MG_CUDA(cudaMemsetAsync(ctx->d_err, 0, sizeof(int32_t), ctx->stream));
     TraceArgs a{};
@@ -573,8 +583,6 @@ int mg_launch_trace(mg_ctx *ctx) {
     a.dshift_frac = ctx->opt.dshift_frac; a.max_steps = ctx->opt.max_steps;
     a.len = d_len; a.xlen = d_xlen; a.err = ctx->d_err;
     if (ctx->geometry == MG_GEOM_3D) {
-        if ((ce = sc.get(&posf, ctx->n)))
-            return mg_fail(ctx, MG_ERR_OOM, std::string("cudaMalloc failed: ") + cudaGetErrorString(ce));
         MG_CUDA(cudaMemsetAsync(wmax, 0, sizeof(unsigned), ctx->stream));
         k_posf<<<(unsigned)((ctx->n + 255) / 256), 256, 0, ctx->stream>>>(ctx->n, ctx->d_pos, posf, wmax);
     }
@@ -610,10 +618,18 @@ int mg_launch_trace(mg_ctx *ctx) {
     if (kerr) {
         return mg_fail(ctx, MG_ERR_CAPACITY, "ray tracing: a half-ray exceeded max_steps");
     }
-    if ((rc = ray_buffer(ctx, &ctx->d_cells, ctx->ray_cap[0], total)) || (rc = ray_buffer(ctx, &ctx->d_xcum, ctx->ray_cap[1], total)) ||
-        (rc = ray_buffer(ctx, &ctx->d_ds, ctx->ray_cap[2], total)) || (rc = ray_buffer(ctx, &ctx->d_vpar, ctx->ray_cap[3], total)) ||
-        (rc = ray_buffer(ctx, &ctx->d_dsf, ctx->ray_cap[4], total)) || (rc = ray_buffer(ctx, &ctx->d_vparf, ctx->ray_cap[5], total)))
-        return rc;
+    auto store = [&]() {
+        int64_t *c = ctx->ray_cap;
+        return ray_buffer(ctx, &ctx->d_cells, c[0], total) || ray_buffer(ctx, &ctx->d_xcum, c[1], total) ||
+               ray_buffer(ctx, &ctx->d_ds, c[2], total) || ray_buffer(ctx, &ctx->d_vpar, c[3], total) ||
+               ray_buffer(ctx, &ctx->d_dsf, c[4], total) || ray_buffer(ctx, &ctx->d_vparf, c[5], total);
+    };
+    if (store()) {           // once more without what the buffers held before
+        mg_free(ctx->d_cells); mg_free(ctx->d_xcum); mg_free(ctx->d_ds);
+        mg_free(ctx->d_vpar); mg_free(ctx->d_dsf); mg_free(ctx->d_vparf);
+        for (int64_t &c : ctx->ray_cap) c = 0;
+        if (store()) return MG_ERR_OOM;
+    }
     a.ray_off = ctx->d_ray_off; a.cells = ctx->d_cells; a.xcum = ctx->d_xcum; a.ds = ctx->d_ds; a.vpar = ctx->d_vpar;
     a.dsf = ctx->d_dsf; a.vparf = ctx->d_vparf;
     {
