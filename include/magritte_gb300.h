@@ -403,7 +403,9 @@ int mg_mlp_set_normalisation(mg_mlp *mlp, const float *mean, const float *std);
 /* Host rows: X [rows][4] raw features -> logp [rows][n_out] log fractions. */
 int mg_mlp_forward(mg_mlp *mlp, int64_t rows, const float *X, float *logp);
 /* Loss (mean squared error of log fractions over targets Y >= 1e-12, Y [rows][n_out]
- * fractions) and its gradient [param_count] (either may be NULL). */
+ * fractions) and its gradient [param_count] (either may be NULL). Its workspace, and that of
+ * mg_mlp_train, is allocated by the first call that needs it and kept with the network (up to
+ * 256 MB a buffer). Threads may call both on one network: one runs, the others wait. */
 int mg_mlp_loss_grad(mg_mlp *mlp, int64_t rows, const float *X, const float *Y, double *loss, float *grad);
 /* Adam training on host rows (copied to the device once). */
 int mg_mlp_train(mg_mlp *mlp, int64_t rows, const float *X, const float *Y, const mg_train_opts *opts,

@@ -17,9 +17,9 @@
 #include <cmath>
 #include <cstring>
 #include <algorithm>
+#include <mutex>
 #include <random>
 #include <cstdio>
-#include <cstring>
 #include "common.cuh"
 
 using namespace mg;
@@ -539,8 +539,9 @@ struct mg_mlp {
     float mean[kIn] = {0, 0, 0, 0}, istd[kIn] = {1, 1, 1, 1};
     int64_t step = 0;
     std::string err;
-    // workspace of loss_grad and train, which own the network while they run: inputs, targets,
-    // row indices, per-CTA partials, losses and target counts (kept up to 256 MB each)
+    // workspace of loss_grad and train, one at a time (`busy`), other threads wait: inputs,
+    // targets, row indices, per-CTA partials, losses and target counts (kept up to 256 MB each)
+    std::mutex busy;
     float *wX = nullptr, *wY = nullptr, *wP = nullptr;
     int32_t *wI = nullptr;
     double *wL = nullptr;
@@ -765,6 +766,7 @@ static int loss_grad_host(mg_mlp *p, int64_t rows, const float *X, const float *
 
 extern "C" int mg_mlp_loss_grad(mg_mlp *p, int64_t rows, const float *X, const float *Y, double *loss, float *grad) {
     if (!p || rows < 1 || !X || !Y) return MG_ERR_ARG;
+    std::lock_guard<std::mutex> own(p->busy);
     cudaSetDevice(p->device);
     return done(p, loss_grad_host(p, rows, X, Y, loss, grad));
 }
@@ -818,6 +820,7 @@ static int train_host(mg_mlp *p, int64_t rows, const float *X, const float *Y, c
 extern "C" int mg_mlp_train(mg_mlp *p, int64_t rows, const float *X, const float *Y, const mg_train_opts *o,
                             mg_train_report *rep) {
     if (!p || rows < 1 || !X || !Y || !o || o->epochs < 1 || o->batch < kRows || !(o->lr > 0)) return MG_ERR_ARG;
+    std::lock_guard<std::mutex> own(p->busy);
     cudaSetDevice(p->device);
     auto t0 = std::chrono::steady_clock::now();
     mg_train_report r{};
