@@ -335,10 +335,10 @@ extern "C" int mg_batch_iterate(mg_batch *b, mg_ali_report *reps) {
         }
         // Ng acceleration, as in mg_iterate (outside the graph: the history rings rotate and
         // a step's acceptance is read on the host), all models in one launch per kernel
-        if (!push.empty() && mg_launch_push_history_batch(push.data(), (int)push.size(), b->stream))
-            return bfail(b, MG_ERR_CUDA, "batch: Ng history");
+        int rc = push.empty() ? MG_OK : mg_launch_push_history_batch(push.data(), (int)push.size(), b->stream);
+        if (rc) return bfail(b, rc, "batch: Ng history");
         if (!step.empty()) {
-            if (mg_launch_ng_batch(step.data(), (int)step.size(), b->stream)) return bfail(b, MG_ERR_CUDA, "batch: Ng step");
+            if ((rc = mg_launch_ng_batch(step.data(), (int)step.size(), b->stream))) return bfail(b, rc, "batch: Ng step");
             for (size_t i = 0; i < step.size(); i++)
                 B_CUDA(cudaMemcpyAsync(b->h_scal_all + i, step[i]->d_scal + 3, 8, cudaMemcpyDeviceToHost, b->stream));
             B_CUDA(cudaStreamSynchronize(b->stream));

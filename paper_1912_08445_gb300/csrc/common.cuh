@@ -218,6 +218,7 @@ int mg_alloc(mg_ctx *ctx, T **p, size_t count) {
     cudaError_t e = cudaMalloc((void **)p, count * sizeof(T));
     if (e != cudaSuccess && mg_release_idle_rays(ctx)) e = cudaMalloc((void **)p, count * sizeof(T));
     if (e != cudaSuccess) {
+        cudaGetLastError();   // (reported here, not by the next launch)
         *p = nullptr;
         return mg_fail(ctx, MG_ERR_OOM, std::string("cudaMalloc failed: ") + cudaGetErrorString(e));
     }

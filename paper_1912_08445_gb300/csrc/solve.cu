@@ -700,7 +700,6 @@ static int launch_fp64(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount,
             if (*cap >= need) return true;
             *cap = 0;
             if (mg_alloc(ctx, p, need)) {
-                cudaGetLastError();
                 ctx->err.clear();
                 return false;
             }

@@ -543,11 +543,7 @@ struct TraceScratch {
 
 template <typename T>
 static int ray_buffer(mg_ctx *ctx, T **p, int64_t &cap, int64_t count) {
-    return kept_buffer(cap, count, [&](int64_t n) {
-        const int rc = mg_alloc(ctx, p, n);
-        if (rc) cudaGetLastError();   // (not the error of a later launch)
-        return rc;
-    });
+    return kept_buffer(cap, count, [&](int64_t n) { return mg_alloc(ctx, p, n); });
 }
 
 int mg_launch_trace(mg_ctx *ctx) {
