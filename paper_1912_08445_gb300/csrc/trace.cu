@@ -16,8 +16,8 @@ struct TraceArgs {
     int32_t R;
     int32_t geometry;
     const double *pos, *vel, *b, *dirs;
-    const float4 *posf;                // (x, y, z, |x| + |y| + |z|) in FP32, for the filter
-    const float *wmax;                 // largest |x| + |y| + |z|
+    const float4 *posf;                // (x, y, z, reach) in FP32, for the filter: the reach of a cell is
+                                       // the largest |x| + |y| + |z| of it and its neighbours
     const int64_t *nbr_off;
     const int32_t *nbr_idx;
     const uint8_t *bdy;
@@ -96,10 +96,12 @@ __device__ __forceinline__ bool emit(const TraceArgs &a, int64_t base, int32_t &
 //   otherwise every valid candidate with lo <= hi is. (A non-finite d leaves the choice to
 //   the last.)
 // The bounds follow from |fl32(a) - a| <= u|a| (u = 2^-24) for the conversions of the
-// positions and the direction and for each FP32 operation, with |x|_1 bounded by twice the
-// model's largest (P below); they are doubled for margin. They are the same for every
-// candidate of a walk: bounds per candidate, three times tighter, took more instructions
-// than the distances themselves (20k-point cloud, 960k half-rays: 2.15 ms, now 1.48 ms).
+// positions and the direction and for each FP32 operation, with |x|_1 bounded by the reaches
+// of the current cell and of the origin (P below); they are doubled for margin. They are the
+// same for every candidate of a step: bounds per candidate took more instructions than the
+// distances themselves (20k-point cloud, 960k half-rays: 2.02 ms, per step 1.41 ms). Bounds for
+// the whole model (1.42 ms) decide nothing near the centre of a model with many scales: 20k
+// points over five decades of radius took 36.0 ms, bounds per candidate 5.7 ms, per step 4.1 ms.
 struct Bounds32 {
     float margin;          // of |s32 - s_cur|
     float e1, e0, e2;      // Ed(d) = e1 sqrt(d) + e0 + e2 d
@@ -145,7 +147,6 @@ __device__ void walk_3d(const TraceArgs &a, int64_t o, int r, int64_t base, int3
     const double vo0 = a.vel[3 * o], vo1 = a.vel[3 * o + 1], vo2 = a.vel[3 * o + 2];
     const float n0f = (float)n0, n1f = (float)n1, n2f = (float)n2;
     const float4 po = a.posf[o];
-    const Bounds32 B((*a.wmax + po.w) * 1.0001f);
     int64_t cur = o;
     double s_cur = 0.0;
     double va = 0.0, ba = a.b[o];
@@ -155,6 +156,7 @@ __device__ void walk_3d(const TraceArgs &a, int64_t o, int r, int64_t base, int3
     overflow = false;
     for (;;) {
         const float scf = (float)s_cur;
+        const Bounds32 B((a.posf[cur].w + po.w) * 1.0001f);
         const int64_t e0 = a.nbr_off[cur], e1 = a.nbr_off[cur + 1];
         // pass 1: the three smallest FP32 distances among the valid candidates, four
         // candidates' gathers in flight at a time
@@ -453,17 +455,17 @@ static int scan_counts(mg_ctx *ctx, const int32_t *d_cnt, int64_t m, int64_t *d_
     return MG_OK;
 }
 
-__global__ void k_posf(int64_t n, const double *__restrict__ pos, float4 *__restrict__ posf, unsigned *wmax) {
+__global__ void k_posf(int64_t n, const double *__restrict__ pos, const int64_t *__restrict__ nbr_off,
+                       const int32_t *__restrict__ nbr_idx, float4 *__restrict__ posf) {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    float w = 0.0f;
-    if (i < n) {
-        const float x = (float)pos[3 * i], y = (float)pos[3 * i + 1], z = (float)pos[3 * i + 2];
-        w = fabsf(x) + fabsf(y) + fabsf(z);
-        posf[i] = make_float4(x, y, z, w);
-    }
-    // (non-negative floats order like their bits; a NaN is the largest)
-    const unsigned m = __reduce_max_sync(0xffffffffu, __float_as_uint(w) & 0x7fffffffu);
-    if ((threadIdx.x & 31) == 0) atomicMax(wmax, m);
+    if (i >= n) return;
+    auto at = [&](int64_t c) { return make_float3((float)pos[3 * c], (float)pos[3 * c + 1], (float)pos[3 * c + 2]); };
+    auto size = [](const float3 p) { return fabsf(p.x) + fabsf(p.y) + fabsf(p.z); };
+    const float3 p = at(i);
+    // (as bits: non-negative floats order like them, and a NaN is the largest)
+    unsigned m = __float_as_uint(size(p)) & 0x7fffffffu;
+    for (int64_t e = nbr_off[i]; e < nbr_off[i + 1]; e++) m = max(m, __float_as_uint(size(at(nbr_idx[e]))) & 0x7fffffffu);
+    posf[i] = make_float4(p.x, p.y, p.z, __uint_as_float(m));
 }
 
 // Stream-ordered pool for a trace's scratch, one per device: allocating and freeing up to
@@ -553,10 +555,9 @@ int mg_launch_trace(mg_ctx *ctx) {
     int32_t *d_len = nullptr, *d_xlen = nullptr, *d_tmp = nullptr;
     float4 *posf = nullptr;
     int64_t *bsum = nullptr;
-    unsigned *wmax = nullptr;
     cudaError_t ce;
     if ((ce = sc.get(&d_len, nr)) || (ce = sc.get(&d_xlen, nr)) ||
-        (ce = sc.get(&bsum, (nr + kScanBlock - 1) / kScanBlock)) || (ce = sc.get(&wmax, 1)) ||
+        (ce = sc.get(&bsum, (nr + kScanBlock - 1) / kScanBlock)) ||
         (ctx->geometry == MG_GEOM_3D && (ce = sc.get(&posf, ctx->n))))
         return mg_fail(ctx, MG_ERR_OOM, std::string("cudaMalloc failed: ") + cudaGetErrorString(ce));
     // The ray store is written in place: solves and images of the old rays come first. Those
@@ -578,12 +579,10 @@ int mg_launch_trace(mg_ctx *ctx) {
     a.nbr_off = ctx->d_nbr_off; a.nbr_idx = ctx->d_nbr_idx; a.bdy = ctx->d_bdy;
     a.dshift_frac = ctx->opt.dshift_frac; a.max_steps = ctx->opt.max_steps;
     a.len = d_len; a.xlen = d_xlen; a.err = ctx->d_err;
-    if (ctx->geometry == MG_GEOM_3D) {
-        MG_CUDA(cudaMemsetAsync(wmax, 0, sizeof(unsigned), ctx->stream));
-        k_posf<<<(unsigned)((ctx->n + 255) / 256), 256, 0, ctx->stream>>>(ctx->n, ctx->d_pos, posf, wmax);
-    }
+    if (ctx->geometry == MG_GEOM_3D)
+        k_posf<<<(unsigned)((ctx->n + 127) / 128), 128, 0, ctx->stream>>>(ctx->n, ctx->d_pos, ctx->d_nbr_off,
+                                                                         ctx->d_nbr_idx, posf);
     a.posf = posf;
-    a.wmax = reinterpret_cast<const float *>(wmax);
     // Record up to cap_tmp cells per half-ray in the count pass, in scratch of at most
     // 32 GiB and a quarter of the free device memory (given back after tracing; half-rays with
     // more cells, or all of them without scratch, are walked again by the fill pass).
