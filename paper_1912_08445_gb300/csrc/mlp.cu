@@ -59,11 +59,10 @@ Layout make_layout(int n_out) {
 // CTA's share starts on a 16-byte boundary.
 __host__ __device__ inline int64_t partial_stride(const Layout &L) { return (L.total + 4) & ~(int64_t)3; }
 
-// BF16 weight copies: forward operands stored [out][in] (WT), backward operands stored
-// [in][out] (W), W4 padded to npad outputs with zeros.
+// BF16 weight copies stored [out][in], W4 padded to npad outputs with zeros (the backward
+// products read them transposed).
 struct BfWeights {
     __nv_bfloat16 *W2T, *W3T, *W4T;   // [128][128], [128][128], [npad][128]
-    __nv_bfloat16 *W2, *W3, *W4;      // [128][128], [128][128], [128][npad]
 };
 
 __device__ __forceinline__ void mma_bf16(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
@@ -423,15 +422,12 @@ __global__ void k_refresh_bf16(const float *theta, Layout L, BfWeights w) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t < kHid * kHid) {
         const int i = t / kHid, j = t - (t / kHid) * kHid;   // W[i][j], i = in, j = out
-        w.W2[t] = __float2bfloat16(theta[L.W2 + t]);
-        w.W3[t] = __float2bfloat16(theta[L.W3 + t]);
         w.W2T[j * kHid + i] = __float2bfloat16(theta[L.W2 + t]);
         w.W3T[j * kHid + i] = __float2bfloat16(theta[L.W3 + t]);
     }
     if (t < kHid * L.npad) {
         const int i = t / L.npad, j = t - (t / L.npad) * L.npad;
         const float v = j < L.n_out ? theta[L.W4 + i * L.n_out + j] : 0.f;
-        w.W4[i * L.npad + j] = __float2bfloat16(v);
         w.W4T[j * kHid + i] = __float2bfloat16(v);
     }
 }
@@ -574,7 +570,7 @@ extern "C" int mg_mlp_create(mg_mlp **out, int32_t n_out, uint64_t seed, int32_t
         return MG_ERR_CUDA;
     }
     const int64_t T = p->L.total;
-    const size_t nbf = 4 * (size_t)kHid * kHid + 2 * (size_t)kHid * kMaxOut;
+    const size_t nbf = 2 * (size_t)kHid * kHid + (size_t)kHid * kMaxOut;
     if (cudaMalloc(&p->theta, 4 * T) || cudaMalloc(&p->m, 4 * T) || cudaMalloc(&p->v, 4 * T) ||
         cudaMalloc(&p->grad, 4 * T) || cudaMalloc(&p->wbuf, 2 * nbf)) {
         mg_mlp_destroy(p);
@@ -582,10 +578,7 @@ extern "C" int mg_mlp_create(mg_mlp **out, int32_t n_out, uint64_t seed, int32_t
     }
     p->w.W2T = p->wbuf;
     p->w.W3T = p->w.W2T + kHid * kHid;
-    p->w.W2 = p->w.W3T + kHid * kHid;
-    p->w.W3 = p->w.W2 + kHid * kHid;
-    p->w.W4T = p->w.W3 + kHid * kHid;
-    p->w.W4 = p->w.W4T + kHid * kMaxOut;
+    p->w.W4T = p->w.W3T + kHid * kHid;
     // He-uniform initial weights from a seeded generator, zero biases
     std::mt19937_64 rng(seed);
     std::vector<float> th(T, 0.f);
