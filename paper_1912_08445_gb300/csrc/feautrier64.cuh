@@ -56,7 +56,7 @@ struct Warp64 {
     double *gz, *ngy, *h;        // ring: x' = a_q gz + ngy; h of the interval from the previous point
     uint64_t *Xm, *Ym;           // [nl][32] line opacity X and floored source Y = eta/chi_min at line centre
     int32_t *Xe, *Ye;            //   (exponents; Ye holds 8 e + flags: 1 for Y < 0, 2 for X < 0 or NaN, 4
-                                 //   for an emissivity that is not finite, in place of the source in S)
+                                 //   for an emissivity that is not finite; S is NaN then)
     double *S;                   // [nl][32]
     float4 *tt;                  // [nl][32]: (g_z, -g_y, |x'| beyond which the line is far, -) in FP32
     double *N;                   // ring: profile normalisation without 1/nu (band terms)
@@ -161,6 +161,11 @@ __device__ __forceinline__ void row64(Bin64 &z, double h, double dmin, const Pos
         z.P *= 0x1p-256; z.Q *= 0x1p-256; z.R *= 0x1p-256;
         if constexpr (B > 0) { z.q1 *= 0x1p-256; z.r1 *= 0x1p-256; z.q2 *= 0x1p-256; z.r2 *= 0x1p-256; }
     }
+}
+
+// A magnitude with the flags of its Ye: negative (1), NaN in place of what is not finite (4).
+__device__ __forceinline__ double flagged64(double v, int ye) {
+    return __hiloint2double((__double2hiint(v) | ((ye & 4) ? 0x7ff80000 : 0)) ^ (ye << 31), __double2loint(v));
 }
 
 // Position of a comoving offset between the roots: segment and fraction.
@@ -357,6 +362,16 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
             W.gz[j] = gz;
             W.ngy[j] = -gy;
             W.h[j] = hin;
+            bool scatters = false;
+            if constexpr (SCAT) {
+                const int32_t ca = W.cell[i + 1], cb = W.cell[i];
+                const double xs = (1.0 - w) * a.chi_sca[ca] + w * a.chi_sca[cb];
+                W.w[j] = w;
+                W.xs[j] = xs;
+                W.ca[j] = ca;
+                W.cb[j] = cb;
+                scatters = xs != 0.0;
+            }
             for (int k = 0; k < nl; k++) {
                 W.tt[32 * k + j] = make_float4(
                     (float)gz, -(float)gy, A.skip ? sqrtf(1.001f / kLog2e64 * fmaxf(line_bound64(W, k, i, eb, chi_min_e), 0.0f)) / shrink + xerr : INFINITY,
@@ -365,7 +380,7 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
                 const double et = (1.0 - w) * p0.x + w * p1.x, ch = (1.0 - w) * p0.y + w * p1.y;
                 const double nrm = a.lc[l0 + k].pnorm * ibk;      // c/(nu sqrt pi) / b
                 // (a negative opacity alone ends at the floor; scattering opacity adds to it first)
-                const PosFp X = ch > 0.0 || SCAT ? pos_from(fabs(ch * nrm)) : PosFp{0, 0};
+                const PosFp X = ch > 0.0 || scatters ? pos_from(ch * nrm) : PosFp{0, 0};
                 const PosFp Y = pos_from(et * nrm * A.inv_chi_min);
                 W.Xm[32 * k + j] = X.m;
                 W.Xe[32 * k + j] = X.e;
@@ -376,21 +391,14 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
                 if (ch > 0.0) {
                     S = pos_pack(pos_mul(pos_from(et), pos_rcp(pos_from(ch))));
                     if (et < 0.0) S = -S;
-                    if (not_finite(ch)) S = ch - ch;
+                    if (not_finite(ch)) S = nan64();
                 }
-                if (bad) S = et * gy;
+                if (bad) S = nan64();
                 W.S[32 * k + j] = S;
             }
             if constexpr (B > 0) {
                 W.N[j] = ibk * (kC / kSqrtPi);
                 W.rx[j] = x;
-            }
-            if constexpr (SCAT) {
-                const int32_t ca = W.cell[i + 1], cb = W.cell[i];
-                W.w[j] = w;
-                W.xs[j] = (1.0 - w) * a.chi_sca[ca] + w * a.chi_sca[cb];
-                W.ca[j] = ca;
-                W.cb[j] = cb;
             }
         }
         __syncwarp();
@@ -440,18 +448,18 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
             if (SCAT && xs != 0.0) {
                 oth = scattered64(a, roots, l0 + lw, xr, W.w[j], xs, W.ca[j], W.cb[j]);
                 const int ye = Ye[j];
-                double cl = pos_pack(chi.m, chi.e);
-                if (ye & 2) cl = -cl;
-                chi = pos_from(pos_max(cl + xs, a.chi_min));   // (a negative sum is below it as bits too)
+                const double cl = pos_pack(chi.m, chi.e);
+                const double c = __hiloint2double(__double2hiint(cl) ^ ((ye & 2) << 30), __double2loint(cl)) + xs;
+                chi = pos_from(pos_max(c, a.chi_min));   // (a negative sum is below it as bits too)
                 // line emissivity: Y chi_min e
                 double et = pos_pack(mulhi_near(Ym[j], e), (ye >> 3) + 1 - n) * a.chi_min;
-                if (ye & 5) et = ye & 4 ? S : -et;
+                et = flagged64(et, ye);
                 S = (et + oth) * pos_pack(pos_rcp(chi));
-            } else if (chi.m == 0 || chi.e < A.cmin.e || (chi.e == A.cmin.e && chi.m < A.cmin.m) || (SCAT && (Ye[j] & 2))) {
+            } else if (chi.m == 0 || chi.e < A.cmin.e || (chi.e == A.cmin.e && chi.m < A.cmin.m)) {
                 chi = A.cmin;
                 const int ye = Ye[j];
                 S = pos_pack(mulhi_near(Ym[j], e), (ye >> 3) + 1 - n);
-                if (ye & 5) S = ye & 4 ? Sr[j] : -S;
+                S = flagged64(S, ye);
             }
             if (first && j == 0) {
                 // the far end: the boundary row starts from Phi iota = 1, psi = I, delta = 0
@@ -495,7 +503,7 @@ __global__ void __launch_bounds__(512) k_feautrier64w(Sweep64 A) {
     const int nu = (blockDim.x >> 5) >> A.duo, warp = threadIdx.x >> 5, unit = warp >> A.duo, lane = threadIdx.x & 31;
     const int half = A.duo ? warp & 1 : 2;
     const int ob = blockIdx.x / A.split, share = blockIdx.x - ob * A.split;
-    int64_t o = A.o0 + ob;
+    int64_t o = B > 0 ? A.o0 + ob : ob;   // (only band terms need several launches)
     if (a.olist) {
         if ((int)blockIdx.x >= *a.ocount) return;
         o = a.olist[blockIdx.x];

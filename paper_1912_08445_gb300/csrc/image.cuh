@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(256) k_image64_lines(ImageArgs a, int skip, in
                         S = pos_pack(pos_mul(pos_from(et), pos_rcp(pos_from(ch))));
                         if (et < 0.0) S = -S;
                     }
-                    if (bad) S = et * gy;
+                    if (bad) S = nan64();
                     T.S[i * cap + t] = S;
                     const int sgn = NOV > 1 ? 0x7fffffff : -1;   // (alone, a negative opacity is below every other)
                     const int ech = max(__double2hiint(p0.y) & sgn, __double2hiint(p1.y) & sgn) >> 20;

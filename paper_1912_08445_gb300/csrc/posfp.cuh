@@ -39,6 +39,8 @@ __device__ __forceinline__ PosFp pos_from(double x) {
     return PosFp{((b << 11) | 0x8000000000000000ull), ex - 1086};   // 1086 = 1023 + 63
 }
 
+// (a constant: FP64 instructions under a predicate cost as much as executed ones)
+__device__ __forceinline__ double nan64() { return __longlong_as_double(0x7ff8000000000000ll); }
 __device__ __forceinline__ bool not_finite(double x) { return (__double2hiint(x) & 0x7ff00000) == 0x7ff00000; }
 
 // m 2^e rounded to a double; m may have up to two leading zero bits. Below the smallest
