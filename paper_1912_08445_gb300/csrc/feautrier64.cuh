@@ -362,19 +362,20 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
             W.gz[j] = gz;
             W.ngy[j] = -gy;
             W.h[j] = hin;
-            bool scatters = false;
+            bool scatters = false, beside = false;   // (beside: this point or the next may scatter)
             if constexpr (SCAT) {
                 const int32_t ca = W.cell[i + 1], cb = W.cell[i];
-                const double xs = (1.0 - w) * a.chi_sca[ca] + w * a.chi_sca[cb];
+                const double xa = a.chi_sca[ca], xb = a.chi_sca[cb], xs = (1.0 - w) * xa + w * xb;
                 W.w[j] = w;
                 W.xs[j] = xs;
                 W.ca[j] = ca;
                 W.cb[j] = cb;
                 scatters = xs != 0.0;
+                beside = xa != 0.0 || xb != 0.0;
             }
             for (int k = 0; k < nl; k++) {
                 W.tt[32 * k + j] = make_float4(
-                    (float)gz, -(float)gy, A.skip ? sqrtf(1.001f / kLog2e64 * fmaxf(line_bound64(W, k, i, eb, chi_min_e), 0.0f)) / shrink + xerr : INFINITY,
+                    (float)gz, -(float)gy, A.skip && !beside ? sqrtf(1.001f / kLog2e64 * fmaxf(line_bound64(W, k, i, eb, chi_min_e), 0.0f)) / shrink + xerr : INFINITY,
                     0.0f);
                 const double2 p0 = W.ln[32 * k + i + 1], p1 = W.ln[32 * k + i];
                 const double et = (1.0 - w) * p0.x + w * p1.x, ch = (1.0 - w) * p0.y + w * p1.y;
@@ -415,9 +416,6 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
                 const float4 t4 = W.tt[32 * lw + j];
                 if (fabsf(fmaf(aqf, t4.x, t4.y)) > t4.z) fb |= 1u << j;
             }
-            if constexpr (SCAT)
-                for (int j = 0; j < nr; j++)
-                    if (W.xs[j] != 0.0) fb &= ~(1u << j);
             todo = ~(fb & ((fb << 1) | bin_far1) & ((fb << 2) | (bin_far1 << 1) | bin_far2)) & ring;
             if (first) todo |= 1u;
             if constexpr (B > 0)
