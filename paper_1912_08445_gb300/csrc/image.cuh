@@ -383,7 +383,8 @@ __global__ void __launch_bounds__(256) k_image32_lines(ImageArgs a) {
     const SolveArgs &s = a.s;
     const int64_t o = blockIdx.x;
     const double *vo = a.vel + 3 * o;
-    const float chi_min = (float)s.chi_min, dtau_min = (float)s.dtau_min;
+    // (a normal number: its reciprocal is finite; below it a floor changes no FP32 intensity)
+    const float chi_min = fmaxf((float)s.chi_min, 1.17549435e-38f), dtau_min = (float)s.dtau_min;
     const float nvo = a.nf[0] * (float)vo[0] + a.nf[1] * (float)vo[1] + a.nf[2] * (float)vo[2];
     const int64_t ofb = s.ray_off[o * s.R + a.rb], ofl = s.ray_off[o * s.R + a.rf];
     const int lb = (int)(s.ray_off[o * s.R + a.rb + 1] - ofb);

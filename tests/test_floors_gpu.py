@@ -37,6 +37,7 @@ def _check(m, kind, pops=None, precision=0, scattering=3e-14, **opts):
         u = np.linspace(-1.1e4, 1.1e4, 65)
         for line in range(m.species.n_lines):
             I, _ = ctx.image(5, line, u)
+            assert np.isfinite(I).all()
             Io, _ = o.image(p0, 5, line, u)
             # (the oracle's emissivity times profile is a subnormal number, good to 2^-1075, where
             # the intensity it gives over up to 1e15 m is below 1e-298)
@@ -52,6 +53,7 @@ def _check(m, kind, pops=None, precision=0, scattering=3e-14, **opts):
         Jo, Lo, Eo, Sp = o.formal_solve(p0, None, spectrum=True)
     ctx.formal_solve()
     J, L, E = ctx.get_radiation()
+    assert np.isfinite(J).all() and np.isfinite(L).all() and np.isfinite(E).all()
     if band:
         Jb, M = ctx.get_band_terms()
         for b in range(band):
@@ -118,3 +120,9 @@ def test_optical_depth_floor_mixed(dtau_min):
         ctx.set_variant(v)
         ctx.formal_solve()
         assert np.max(rel_err(ctx.get_radiation()[0], Jo)) < TOL[1], v
+
+
+@pytest.mark.parametrize("chi_min", [1e-36, 1e-40, 1e-60])
+def test_tiny_opacity_floor_of_an_fp32_image(chi_min):
+    """Floors that are not normal FP32 numbers."""
+    _check(_cloud(), "image", precision=1, chi_min=chi_min)
