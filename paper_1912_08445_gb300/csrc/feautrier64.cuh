@@ -112,6 +112,7 @@ struct Sweep64 {
     int32_t nl;              // lines a chunk can touch
     int32_t kl;              // chunks a line can touch (band terms)
     int32_t skip;
+    int32_t wide;            // neighbouring points may differ by more than a third of a width in velocity
     int32_t duo;             // the two halves of a pair go to two warps
     int32_t split;           // CTAs per origin, each with its share of the ray pairs
     double *part;            // split > 1: [n][split][F][4 + B] sums of each CTA
@@ -317,7 +318,7 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
         const int i = own.x, x = own.y - (c0 + lane);
         bool far = false;
         double hin = 0.0, gz = 0.0, gy = 0.0, ibk = 0.0, w = 0.0;
-        float xerr = 0.0f, shrink = 1.0f;
+        float xerr = 0.0f, shrink = 1.0f, step = 0.0f;
         int eb = 0;
         if (lane < cnt) {
             const int j = x - own.z + 1;
@@ -339,8 +340,12 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
                 const float xlo = ylo - gyf, xhi = yhi - gyf;
                 // (with the larger width of the element's ends, so that the next point, up to the
                 // inner cell itself, is at the floor too: its opacity is in the line's bound)
-                shrink = 0.999999f * (float)bp / fmaxf((float)W.b[i], (float)W.b[i + 1]);
-                const float xm = fmaxf((xlo > 0.0f ? xlo : (xhi < 0.0f ? -xhi : 0.0f)) - xerr, 0.0f) * shrink;
+                const float bmax = fmaxf((float)W.b[i], (float)W.b[i + 1]);
+                shrink = 0.999999f * (float)bp / bmax;
+                // the next point's velocity differs by `step` widths: within a third, the default, it
+                // stays below 200 chi_min there (exp(2 x' / 3) at x' = 7.6)
+                if (A.wide) step = 1.000001f * fabsf((float)(W.v[i] - W.v[i + 1])) * (float)W.rn[i] / bmax;
+                const float xm = fmaxf(fmaxf((xlo > 0.0f ? xlo : (xhi < 0.0f ? -xhi : 0.0f)) - xerr, 0.0f) * shrink - step, 0.0f);
                 far = 0.999f * kLog2e64 * xm * xm > bound;
                 if (B > 0) far = far && x >= 3;
                 if constexpr (SCAT) far = far && a.chi_sca[W.cell[i]] == 0.0 && a.chi_sca[W.cell[i + 1]] == 0.0;
@@ -375,7 +380,7 @@ __device__ __forceinline__ bool sweep_half64(const Sweep64 &A, const Warp64 &W, 
             }
             for (int k = 0; k < nl; k++) {
                 W.tt[32 * k + j] = make_float4(
-                    (float)gz, -(float)gy, A.skip && !beside ? sqrtf(1.001f / kLog2e64 * fmaxf(line_bound64(W, k, i, eb, chi_min_e), 0.0f)) / shrink + xerr : INFINITY,
+                    (float)gz, -(float)gy, A.skip && !beside ? (sqrtf(1.001f / kLog2e64 * fmaxf(line_bound64(W, k, i, eb, chi_min_e), 0.0f)) + step) / shrink + xerr : INFINITY,
                     0.0f);
                 const double2 p0 = W.ln[32 * k + i + 1], p1 = W.ln[32 * k + i];
                 const double et = (1.0 - w) * p0.x + w * p1.x, ch = (1.0 - w) * p0.y + w * p1.y;

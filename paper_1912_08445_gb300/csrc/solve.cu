@@ -662,6 +662,7 @@ static int launch_fp64(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount,
         A.cmin = host_pos(a.chi_min);
         A.half_dmin = host_pos(0.5 * a.dtau_min);
         A.skip = mg_floor_depth(ctx) < 1e-14;
+        A.wide = ctx->opt.dshift_frac > 0.34;
         // A unit is a warp with a chunk of bins and a share of the ray pairs. A CTA has up to
         // 8 units: every chunk, and several groups of pairs when the chunks are few, balanced
         // over the rounds each unit makes. Fewer origins than four waves of two CTAs per SM
