@@ -1280,8 +1280,11 @@ constexpr int kNumWarpVariants = sizeof(kWarpVariants) / sizeof(kWarpVariants[0]
 // Far-wing skipping leaves out the floored intervals of far points. Each changes the
 // sweep by O(max(chi_min ds, dtau_min)), below FP32 resolution only while the optical depth
 // that the floors give a whole ray pair is; otherwise (a large floor) the variant's
-// non-skipping twin runs instead.
-bool skip_allowed(const mg_ctx *ctx) { return mg_floor_depth(ctx) < 1e-7; }
+// non-skipping twin runs instead. The point after a left-out one must be near the floor as well,
+// which the velocity-step rule sees to: with steps of up to two widths its opacity is below
+// chi_min exp(4 x' - 4) = 3e11 chi_min at x' = 7.6 (a line 1e25 times the floor), 3e-6 over 1e13 m.
+// Where dshift_frac allows larger steps every point is swept (J per bin was off by 3e-3 at 30).
+bool skip_allowed(const mg_ctx *ctx) { return mg_floor_depth(ctx) < 1e-7 && ctx->opt.dshift_frac <= 2.0; }
 
 int no_skip_twin(int v) {
     const WarpVariant &w = kWarpVariants[v];

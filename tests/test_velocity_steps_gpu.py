@@ -54,3 +54,16 @@ def test_large_steps(kind, dshift_frac):
             assert np.max(rel_err(ctx.get_spectrum(), Sp)) < tol
         if kind != "mixed":
             assert np.max(rel_err(L, Lo, floor=1e-300)) < tol and np.max(np.abs(E - Eo) / Jo) < tol
+
+
+@pytest.mark.parametrize("dshift_frac", [2.0, 5.0, 30.0])
+def test_large_steps_mixed(dshift_frac):
+    for m in _models():
+        o = Oracle(m, nthreads=16, dshift_frac=dshift_frac)
+        Jo, Lo, Eo, Sp = o.formal_solve(o.lte(), None, spectrum=True)
+        ctx = gpu_context(m, oracle_dirs=o.dirs, precision=1, spectrum=1, dshift_frac=dshift_frac)
+        ctx.trace_rays()
+        ctx.init_populations()
+        ctx.formal_solve()
+        assert np.max(rel_err(ctx.get_radiation()[0], Jo)) < 1e-4
+        assert np.max(rel_err(ctx.get_spectrum(), Sp)) < 1e-4
