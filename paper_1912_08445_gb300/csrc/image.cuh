@@ -383,8 +383,11 @@ __global__ void __launch_bounds__(256) k_image32_lines(ImageArgs a) {
     const SolveArgs &s = a.s;
     const int64_t o = blockIdx.x;
     const double *vo = a.vel + 3 * o;
-    // (a normal number: its reciprocal is finite; below it a floor changes no FP32 intensity)
-    const float chi_min = fmaxf((float)s.chi_min, 1.17549435e-38f), dtau_min = (float)s.dtau_min;
+    // Opacities and emissivities in units of 2^-40, lengths of 2^40 (powers of two: the same bits), so
+    // that floors down to 1e-50 are normal FP32 numbers, whose reciprocals are finite. Below
+    // that the floor is the smallest such number.
+    constexpr float kUnit = 0x1p40f;
+    const float chi_min = fmaxf((float)(s.chi_min * (double)kUnit), 1.17549435e-38f), dtau_min = (float)s.dtau_min;
     const float nvo = a.nf[0] * (float)vo[0] + a.nf[1] * (float)vo[1] + a.nf[2] * (float)vo[2];
     const int64_t ofb = s.ray_off[o * s.R + a.rb], ofl = s.ray_off[o * s.R + a.rf];
     const int lb = (int)(s.ray_off[o * s.R + a.rb + 1] - ofb);
@@ -434,7 +437,7 @@ __global__ void __launch_bounds__(256) k_image32_lines(ImageArgs a) {
                     if (k) {
                         int np;
                         const int64_t at = img_interval(s, q, ofb, k, Kb, np);
-                        h = __fdividef(0.5f * a.dsf[at], (float)np);
+                        h = __fdividef((0.5f / kUnit) * a.dsf[at], (float)np);
                     } else {
                         far_w = w;
                     }
@@ -447,8 +450,8 @@ __global__ void __launch_bounds__(256) k_image32_lines(ImageArgs a) {
                         float *g = &T.g[i][pr].x + odd, *x = &T.x[i][pr].x + odd;
                         g[0] = a.lf[i].rat * gz;
                         g[2] = a.lf[i].dnl * pz - a.lf[i].rat * gy;
-                        x[0] = (1.0f - wt) * p0.x + wt * p1.x;
-                        x[2] = (1.0f - wt) * p0.y + wt * p1.y;
+                        x[0] = ((1.0f - wt) * p0.x + wt * p1.x) * kUnit;
+                        x[2] = ((1.0f - wt) * p0.y + wt * p1.y) * kUnit;
                     }
                 } else {
 #pragma unroll

@@ -126,3 +126,9 @@ def test_optical_depth_floor_mixed(dtau_min):
 def test_tiny_opacity_floor_of_an_fp32_image(chi_min):
     """Floors that are not normal FP32 numbers."""
     _check(_cloud(), "image", precision=1, chi_min=chi_min)
+
+
+@pytest.mark.parametrize("chi_min", [1e-36, 1e-40, 1e-48])
+def test_tiny_opacity_floor_of_inverted_lines_in_an_fp32_image(chi_min):
+    """An inverted line has its emissivity over the floor as its source function."""
+    _check(_cloud(), "image", _invert, precision=1, chi_min=chi_min)
