@@ -185,6 +185,7 @@ struct mg_ctx {
     bool sca_on = false;
     double *d_chisca = nullptr, *d_Jsca = nullptr, *d_Jsca_new = nullptr;
     unsigned long long *d_scaw = nullptr;
+    int32_t *d_least = nullptr;    // [L] least source function of a line over the model (solve.cu)
     double *d_part64 = nullptr;    // FP64 solve: sums of the CTAs that share an origin (grow-only)
     int64_t part64_cap = 0;
     double sca_tol = 1e-8, sca_change = 0.0;

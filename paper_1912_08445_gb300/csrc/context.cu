@@ -135,7 +135,7 @@ static void drop_state(mg_ctx *ctx) {
     mg_band_free(ctx);
     ctx->band_solved = 0;
     // scattering buffers are sized by the point, line and bin counts: set them again
-    mg_free(ctx->d_chisca); mg_free(ctx->d_Jsca); mg_free(ctx->d_part64); ctx->part64_cap = 0; mg_free(ctx->d_Jsca_new); mg_free(ctx->d_scaw);
+    mg_free(ctx->d_chisca); mg_free(ctx->d_Jsca); mg_free(ctx->d_part64); mg_free(ctx->d_least); ctx->part64_cap = 0; mg_free(ctx->d_Jsca_new); mg_free(ctx->d_scaw);
     ctx->sca_on = false;
 }
 
@@ -157,7 +157,7 @@ extern "C" int mg_destroy(mg_ctx *ctx) {
     mg_free(ctx->d_err);
     mg_free(ctx->d_uch); mg_free(ctx->d_img); mg_free(ctx->d_imgxy); mg_free(ctx->d_imgov); mg_free(ctx->d_imglf);
     mg_band_free(ctx);
-    mg_free(ctx->d_chisca); mg_free(ctx->d_Jsca); mg_free(ctx->d_part64); mg_free(ctx->d_Jsca_new); mg_free(ctx->d_scaw);
+    mg_free(ctx->d_chisca); mg_free(ctx->d_Jsca); mg_free(ctx->d_part64); mg_free(ctx->d_least); mg_free(ctx->d_Jsca_new); mg_free(ctx->d_scaw);
     if (ctx->h_scal) cudaFreeHost(ctx->h_scal);
     if (ctx->ev0) cudaEventDestroy(ctx->ev0);
     if (ctx->ev1) cudaEventDestroy(ctx->ev1);
@@ -642,7 +642,8 @@ static int ensure_state(mg_ctx *ctx) {
         if ((rc = mg_alloc(ctx, &ctx->d_pops, n * lev)) || (rc = mg_alloc(ctx, &ctx->d_pops_new, n * lev)) ||
             (rc = mg_alloc(ctx, &ctx->d_line, n * L * 2)) || (rc = mg_alloc(ctx, &ctx->d_linef, n * L * 2)) ||
             (rc = mg_alloc(ctx, &ctx->d_J, n * L)) || (rc = mg_alloc(ctx, &ctx->d_L, n * L)) ||
-            (rc = mg_alloc(ctx, &ctx->d_Jeff, n * L)) || (rc = mg_alloc(ctx, &ctx->d_Lc, n * L)))
+            (rc = mg_alloc(ctx, &ctx->d_Jeff, n * L)) || (rc = mg_alloc(ctx, &ctx->d_Lc, n * L)) ||
+            (rc = mg_alloc(ctx, &ctx->d_least, L)))
             return rc;
     }
     if (ctx->opt.spectrum && !ctx->d_Jnu && ctx->have_quad)

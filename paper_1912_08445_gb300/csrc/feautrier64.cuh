@@ -17,7 +17,7 @@
 //   divisions of the staging.
 // - S = eta/chi of a line does not depend on the bin: one division per staged point.
 // - A point whose own and two previous points are far (opacity below chi_min and emission
-//   below chi_min times the boundary intensity) changes the sweep by O(max(chi_min ds, dtau_min))
+//   below chi_min times the least intensity, note_source) changes the sweep by O(max(chi_min ds, dtau_min))
 //   and is left out while the optical depth that the two floors give a whole ray pair (chi_min
 //   times the longest path through the model, dtau_min per interval) is below 1e-14 (`skip`):
 //   whole elements before they are staged, points far in every bin of the warp before they
@@ -35,11 +35,6 @@
 namespace {
 
 constexpr float kLog2e64 = 1.4426950408889634f;
-
-// Least exponent of a boundary intensity: Planck's function is exactly 0 beyond h nu = 710 k T
-// (ilogb(0) is INT_MIN). Every emissivity lies above chi_min times 2^-2000, so any emission
-// counts against a dark boundary.
-constexpr int kDarkExp = -2000;
 
 // Larger of two non-negative doubles, on their bits.
 __device__ __forceinline__ double pos_max(double a, double b) {
@@ -64,7 +59,7 @@ struct Warp64 {
     double *w, *xs;              // ring: weight, scattering opacity
     int32_t *ca, *cb;            // ring: cells (scattering)
     double *mac;                 // [32][2 B]
-    int32_t *ic;                 // [nl] exponent of the boundary intensity at the line, rounded down
+    int32_t *ic;                 // [nl] exponent of the least intensity at the line, rounded down (note_source)
 };
 
 __host__ __device__ inline size_t warp64_bytes(int nl, int B, bool sca) {
@@ -203,7 +198,7 @@ __device__ __forceinline__ double scattered64(const SolveArgs &a, const double *
 
 // Bound of log2(e) x'^2 beyond which line k of the warp is far between slots i and i + 1 of the
 // window, for widths with 1/b < 2^eb: its opacity X exp(-x'^2) is below chi_min and its
-// emissivity below chi_min times the boundary intensity (binary exponents, rounded to the safe
+// emissivity below chi_min times the least intensity (binary exponents, rounded to the safe
 // side): X = c ib (c/sqrt pi)/nu < 2^ec 2^eb 2^28/nu.
 __device__ __forceinline__ float line_bound64(const Warp64 &W, int k, int i, int eb, int chi_min_e) {
     const double2 p0 = W.ln[32 * k + i + 1], p1 = W.ln[32 * k + i];
@@ -542,10 +537,10 @@ __global__ void __launch_bounds__(512) k_feautrier64w(Sweep64 A) {
             aq_hi = fmaxf(aq_hi, __shfl_xor_sync(0xffffffffu, aq_hi, d));
             nu_lo = fminf(nu_lo, __shfl_xor_sync(0xffffffffu, nu_lo, d));
         }
-        // floor test (see the staging): exponents of chi_min nu / 2^28 and of the boundary
-        // intensity, rounded down
+        // floor test (see the staging): exponents of chi_min nu / 2^28 and of the least intensity,
+        // rounded down
         __syncwarp();
-        if (lane < nl) W.ic[lane] = max(ilogb(planck_d(a.lc[l0 + lane].nu, a.T_cmb)), kDarkExp);
+        if (lane < nl) W.ic[lane] = least_exponent(ilogb(planck_d(a.lc[l0 + lane].nu, a.T_cmb)), a.least[l0 + lane]);
         const int chi_min_e = ilogb(a.chi_min) + ilogbf(nu_lo) - 28 - 1;
         // the origin's opacity and source in this bin
         const double x0 = aq * ibo;

@@ -8,11 +8,11 @@
 // A point matters to the channels within a few widths of its velocity only: channels that
 // span tens of widths leave each of them a small share of the points (a fifth on the discs).
 // Each thread therefore lists, as bits over the staged points, those whose opacity is above
-// the floor (or whose emission is above the floor's times the boundary intensity) in its
+// the floor (or whose emission is above the floor's times the least intensity, note_source) in its
 // channel, with the points next to them, and walks through its own list; the warp runs as
 // long as its busiest channel. (Over 32 points at a time that saves nothing: they span ten
 // widths, the reach of a channel, and keep some lane busy at each of them.) An interval between two points below that changes the
-// intensity by O(max(chi_min ds, dtau_min)) of the boundary intensity; the lists are used while
+// intensity by O(max(chi_min ds, dtau_min)) of itself; the lists are used while
 // the optical depth of the two floors over a whole pair stays below 1e-14.
 //
 // FP64. The FP64 pipe (64-80 cycles per warp instruction) bounds it: per listed point x',
@@ -216,6 +216,9 @@ __global__ void __launch_bounds__(256) k_image64_lines(ImageArgs a, int skip, in
     }
     const double inv_chi_min = 1.0 / s.chi_min;
     const PosFp cmin = pos_from(s.chi_min);
+    int ic = 2048;                       // exponent of the least intensity over the lines in reach
+#pragma unroll
+    for (int i = 0; i < NOV; i++) ic = min(ic, least_exponent(a.lf[i].ic, s.least[a.lf[i].l2]));
     constexpr double kCsp = kC / kSqrtPi;
     for (int c0 = 0; c0 < a.n_ch; c0 += blockDim.x) {
         const int c = c0 + threadIdx.x;
@@ -278,7 +281,7 @@ __global__ void __launch_bounds__(256) k_image64_lines(ImageArgs a, int skip, in
                     const int eet = max(__double2hiint(p0.x) & 0x7fffffff, __double2hiint(p1.x) & 0x7fffffff) >> 20;
                     const float bound = max(ech, eet) >= 0x7ff   // (infinite or NaN: never far)
                                             ? INFINITY
-                                            : (float)(max(max(ech, eet - a.lf[i].ic) - 1022, -100000) + eb - a.lf[i].cm);
+                                            : (float)(max(max(ech, eet - ic) - 1022, -100000) + eb - a.lf[i].cm);
                     T.tt[i * cap + t] = make_float4((float)gzl, (float)ngl,
                                              skip ? sqrtf(1.001f / kLog2e64 * fmaxf(bound, 0.0f)) +
                                                         1e-6f * fabsf((float)ngl)

@@ -8,11 +8,44 @@ using namespace mg;
 
 namespace {
 
+// ---------------------------------------------------------------- least source function
+// Emission counts as nothing at a far point where it is below chi_min times the least
+// intensity that can occur: intensities are averages of the boundary's and of the source
+// functions along the ray, S = eta/chi of every line where its opacity is positive. (Behind a
+// cold cloud a bright background can be 20 decades dimmer.) The binary exponent of the least S
+// of each line, rounded down, is kept as kLeastBias less it, so that words start from zero and
+// grow.
+constexpr int kLeastBias = 3000;
+
+// Least exponent that is told apart: Planck's function is exactly 0 beyond h nu = 710 k T
+// (ilogb(0) is INT_MIN), a line without upper populations has no source. Every emissivity lies
+// above chi_min times 2^-2000, so any emission counts against a dark boundary.
+constexpr int kDarkExp = -2000;
+
+__device__ __forceinline__ void note_source(int32_t *least, int l, double eta, double chi) {
+    if (!(chi > 0.0)) return;   // (an inverted line ends at the floor, where its source is large)
+    const int e = eta > 0.0 ? (__double2hiint(eta) >> 20) - (__double2hiint(chi) >> 20) - 1 : kDarkExp;
+    const int v = kLeastBias - max(e, kDarkExp);
+    if (v > *(volatile int32_t *)(least + l)) atomicMax(least + l, v);   // (the first few only)
+}
+
+// The exponent to compare with: the boundary's ic, or that of the least source below it.
+__host__ __device__ __forceinline__ int least_exponent(int ic, int word) {
+    const int e = word > 0 && kLeastBias - word < ic ? kLeastBias - word : ic;
+    return e > kDarkExp ? e : kDarkExp;
+}
+
+__global__ void k_least_source(int64_t n, int L, const double *__restrict__ line, int32_t *least) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < n * L) note_source(least, (int)(t % L), line[2 * t], line[2 * t + 1]);
+}
+
 // ---------------------------------------------------------------- K2 line data
 // eta_int = h nu/4pi n_u A_ul, chi_int = h nu/4pi (n_l B_lu - n_u B_ul) (eq. 'lines'),
 // stored per point as [L][2] so that one gather brings all lines of a point.
 __global__ void k_line_data(int64_t n, int L, int nlev, const double *__restrict__ pops,
-                            const LineConst *__restrict__ lc, double *__restrict__ line, float *__restrict__ linef, unsigned long long *neg) {
+                            const LineConst *__restrict__ lc, double *__restrict__ line, float *__restrict__ linef, unsigned long long *neg,
+                            int32_t *least) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= n * L) return;
     const int64_t c = t / L;
@@ -24,6 +57,7 @@ __global__ void k_line_data(int64_t n, int L, int nlev, const double *__restrict
     line[2 * t] = eta;
     line[2 * t + 1] = chi;
     if (chi < 0.0) atomicAdd(neg, 1ull);
+    note_source(least, l, eta, chi);
     if (linef) {
         linef[2 * t] = (float)eta;
         linef[2 * t + 1] = (float)chi;
@@ -52,6 +86,7 @@ struct SolveArgs {
     int32_t groups;          // FP64 kernel: warps that solve different ray pairs of a point (1: the whole CTA per pair)
     double *Jeffb;           // band ALO: [B][n][L] J_eff of bandwidths 1..B
     double *Mb;              // band ALO: [n][L][R][B] coupling coefficients of the band points
+    const int32_t *least;    // [L] see note_source
     const double *chi_sca;   // scattering: [n] opacity, m^-1
     const double *Jsca;      // scattering: [n][L][Q] previous mean intensity per bin
 };
@@ -572,12 +607,8 @@ int mg_launch_max_rel_change(mg_ctx *ctx, int64_t m, const double *a_new, const 
 
 int mg_launch_line_data(mg_ctx *ctx) {
     if (ctx->opt.precision == MG_MIXED) return mg_launch_line_data_mixed(ctx);
-    const int64_t m = ctx->n * ctx->n_lines;
     MgTimed t(ctx, "line_data");
-    k_line_data<<<(unsigned)((m + 255) / 256), 256, 0, ctx->stream>>>(
-        ctx->n, ctx->n_lines, ctx->n_lev, ctx->d_pops, ctx->d_lines, ctx->d_line, nullptr, ctx->d_scal + 4);
-    MG_CUDA(cudaGetLastError());
-    return MG_OK;
+    return mg_launch_line_data64(ctx, nullptr, ctx->d_scal + 4);
 }
 
 int mg_launch_feautrier_mixed(mg_ctx *ctx);
@@ -606,6 +637,9 @@ int mg_launch_feautrier(mg_ctx *ctx) {
         MG_CUDA(cudaMemsetAsync(ctx->d_promo + ctx->n, 0, sizeof(int32_t), ctx->stream));
         k_mark_thick<<<(unsigned)((ctx->n + 255) / 256), 256, 0, ctx->stream>>>(
             ctx->n, ctx->n_lines, ctx->d_L, 1.0 - 1.0 / ctx->opt.tau_fp64, ctx->d_promo, ctx->d_promo + ctx->n);
+        const int64_t m = ctx->n * ctx->n_lines;
+        MG_CUDA(cudaMemsetAsync(ctx->d_least, 0, sizeof(int32_t) * ctx->n_lines, ctx->stream));
+        k_least_source<<<(unsigned)((m + 255) / 256), 256, 0, ctx->stream>>>(ctx->n, ctx->n_lines, ctx->d_line, ctx->d_least);
         MG_CUDA(cudaGetLastError());
         return launch_fp64(ctx, ctx->d_promo, ctx->d_promo + ctx->n, (unsigned)ctx->n);
     }
@@ -623,6 +657,7 @@ static int launch_fp64(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount,
     a.Jnu = ctx->opt.spectrum ? ctx->d_Jnu : nullptr;
     a.kmax = (int32_t)ctx->max_pair_len;
     a.err = ctx->d_err;
+    a.least = ctx->d_least;
     a.olist = olist;
     a.ocount = ocount;
     const int B = olist ? 0 : ctx->band_cur;   // the band ALO is built for FP64 contexts
@@ -767,8 +802,9 @@ static int launch_fp64(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount,
 // populations, for the images in either precision.
 int mg_launch_line_data64(mg_ctx *ctx, float *linef, unsigned long long *neg) {
     const int64_t m = ctx->n * ctx->n_lines;
+    MG_CUDA(cudaMemsetAsync(ctx->d_least, 0, sizeof(int32_t) * ctx->n_lines, ctx->stream));
     k_line_data<<<(unsigned)((m + 255) / 256), 256, 0, ctx->stream>>>(
-        ctx->n, ctx->n_lines, ctx->n_lev, ctx->d_pops, ctx->d_lines, ctx->d_line, linef, neg);
+        ctx->n, ctx->n_lines, ctx->n_lev, ctx->d_pops, ctx->d_lines, ctx->d_line, linef, neg, ctx->d_least);
     MG_CUDA(cudaGetLastError());
     return MG_OK;
 }
@@ -782,6 +818,7 @@ int mg_launch_image(mg_ctx *ctx, int ray, int line, int n_ch, const double *d_u,
     s.ds = ctx->d_ds; s.vpar = ctx->d_vpar; s.b = ctx->d_b; s.line = ctx->d_line; s.lc = ctx->d_lines;
     s.chi_min = ctx->opt.chi_min; s.dtau_min = ctx->opt.dtau_min; s.T_cmb = ctx->opt.T_cmb;
     s.kmax = (int32_t)ctx->max_pair_len;
+    s.least = ctx->d_least;
     s.err = ctx->d_err;
     a.rf = ray;
     a.rb = ctx->h_anti[ray];

@@ -132,3 +132,21 @@ def test_tiny_opacity_floor_of_an_fp32_image(chi_min):
 def test_tiny_opacity_floor_of_inverted_lines_in_an_fp32_image(chi_min):
     """An inverted line has its emissivity over the floor as its source function."""
     _check(_cloud(), "image", _invert, precision=1, chi_min=chi_min)
+
+
+def _no_emission(p):
+    """Upper levels empty in two cells of three: those only absorb."""
+    q = p.copy()
+    q[np.random.default_rng(1).random(p.shape[0]) < 0.67, 1:] = 0.0
+    return q
+
+
+@pytest.mark.parametrize("overlap", [False, True])
+@pytest.mark.parametrize("kind", KINDS)
+def test_bright_background_behind_cold_cells(kind, overlap):
+    """Intensities far below the boundary's, to which points at the floor still add."""
+    m = _cloud()
+    if overlap:
+        m.species = syn.species_ladder(4)
+    m.n_spec = 1e3 * m.n_spec
+    _check(m, kind, _no_emission, T_cmb=1500.0)
