@@ -180,7 +180,10 @@ int mg_get_populations_dev(const mg_ctx *ctx, double *d_pops);
  *   J    = (1/P) sum_pairs sum_q w_q u,                       (mean intensity)
  *   L    = (1/P) sum sum w_q Lambda*_oo chi_l/chi,            (diagonal ALO weight)
  *   Jeff = (1/P) sum sum w_q (u - Lambda*_oo eta_l/chi).      (effective intensity)
- * Requires traced rays, quadrature, species and populations. Asynchronous. */
+ * Requires traced rays, quadrature, species and populations. Asynchronous, but for the first
+ * solve of a model, which may allocate scratch that the context keeps (band terms: at most
+ * 1 GiB; without room for them the solve takes a kernel that needs none). Populations that
+ * are not finite make J and Jeff so at the points whose rays meet their cell. */
 int mg_formal_solve(mg_ctx *ctx);
 /* Copies J, L, Jeff, each [n][n_lines], to host buffers (any may be NULL). */
 int mg_get_radiation(const mg_ctx *ctx, double *J, double *L, double *Jeff);
@@ -373,7 +376,7 @@ int mg_batch_work_counts(const mg_batch *batch, int64_t *solves, int64_t *cell_f
  * depth of line 0 at LTE -- to its log fractional level populations: 4 -> 128 -> 128 ->
  * 128 -> n_out, ReLU, log-softmax. Inference and training run in hand-written kernels:
  * BF16 tensor-core products (FP32 accumulation) for the 128-wide layers and the
- * back-propagated deltas, FP32 weight gradients, Adam on FP32 master weights. The ALI
+ * back-propagated deltas, weight gradients with FP32 accumulation, Adam on FP32 master weights. The ALI
  * from such a start converges to the same fixed point as from LTE. */
 typedef struct mg_mlp mg_mlp;
 typedef struct {

@@ -26,12 +26,10 @@
 // The general kernel k_feautrier64 (a bin sums several lines) takes, per point and bin, an
 // exponential (16 DFMA), two divisions (8 each), four interpolations and ~15 further
 // operations, and sweeps every point. Measured, one ALI step, general kernel -> this one:
-// clumpy cloud of 1500 points, 48 rays, 4 x 31 bins 174.9 -> 8.2 ms (11.1 ms with 8 FP64
-// operations per point and bin, warp-wide far points and every point staged; FP64 pipe 78 %
-// busy); with the band ALO (600 points) 124.8 -> 5.7 ms; spherical cloud of 200 shells 1.64 ->
-// 0.35 ms; one scattering pass of a 200-point cloud 7.1 -> 1.5 ms.
-// Error against an 80-bit solve (2-norm of J; 200 shells, two models, and a cloud of 150 points):
-// general kernel 4.1e-16, 4.0e-16, 3.0e-16; this one 3.8e-16, 3.5e-16, 2.6e-16.
+// clumpy cloud of 1500 points, 48 rays, 4 x 31 bins 174.9 -> 8.3 ms (11.1 ms with 8 FP64
+// operations per point and bin, warp-wide far points and every point staged), FP64 pipe active
+// in 74 % of the cycles; with the band ALO (600 points) 124.8 -> 5.8 ms; spherical cloud of 200
+// shells 1.64 -> 0.35 ms; scattering on a 200-point cloud, to a change of 1e-10, 7.1 -> 1.5 ms.
 namespace {
 
 constexpr float kLog2e64 = 1.4426950408889634f;
