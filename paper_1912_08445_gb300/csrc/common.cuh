@@ -258,7 +258,6 @@ int mg_launch_image(mg_ctx *ctx, int ray, int line, int n_ch, const double *d_u,
 int mg_launch_feautrier(mg_ctx *ctx);
 int mg_launch_max_rel_change(mg_ctx *ctx, int64_t m, const double *a_new, const double *a_old,
                              unsigned long long *word);
-int mg_launch_feautrier_fp64_list(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount);
 int mg_autotune_mixed(mg_ctx *ctx, int reps, int *best, double *best_ms, int *n_tried);
 int mg_launch_lte(mg_ctx *ctx);
 int mg_launch_collision_rates(mg_ctx *ctx);

@@ -25,6 +25,11 @@ namespace {
 
 constexpr int kImgCap = 512;   // points staged at a time, at most
 
+// The FP32 kernel has opacities and emissivities in units of 1/kImgUnit and lengths in units of
+// kImgUnit (a power of two: the same bits), so that floors down to 1e-50 are normal FP32 numbers,
+// whose reciprocals are finite. Below that the floor is the smallest such number.
+constexpr float kImgUnit = 0x1p40f;
+
 // Shared memory: per staged point and line, then the channels' lists.
 template <int NOV>
 struct ImgStage64 {
@@ -386,11 +391,7 @@ __global__ void __launch_bounds__(256) k_image32_lines(ImageArgs a) {
     const SolveArgs &s = a.s;
     const int64_t o = blockIdx.x;
     const double *vo = a.vel + 3 * o;
-    // Opacities and emissivities in units of 2^-40, lengths of 2^40 (powers of two: the same bits), so
-    // that floors down to 1e-50 are normal FP32 numbers, whose reciprocals are finite. Below
-    // that the floor is the smallest such number.
-    constexpr float kUnit = 0x1p40f;
-    const float chi_min = fmaxf((float)(s.chi_min * (double)kUnit), 1.17549435e-38f), dtau_min = (float)s.dtau_min;
+    const float chi_min = a.chi_min32, dtau_min = a.dtau_min32;
     const float nvo = a.nf[0] * (float)vo[0] + a.nf[1] * (float)vo[1] + a.nf[2] * (float)vo[2];
     const int64_t ofb = s.ray_off[o * s.R + a.rb], ofl = s.ray_off[o * s.R + a.rf];
     const int lb = (int)(s.ray_off[o * s.R + a.rb + 1] - ofb);
@@ -440,7 +441,7 @@ __global__ void __launch_bounds__(256) k_image32_lines(ImageArgs a) {
                     if (k) {
                         int np;
                         const int64_t at = img_interval(s, q, ofb, k, Kb, np);
-                        h = __fdividef((0.5f / kUnit) * a.dsf[at], (float)np);
+                        h = __fdividef((0.5f / kImgUnit) * a.dsf[at], (float)np);
                     } else {
                         far_w = w;
                     }
@@ -453,8 +454,8 @@ __global__ void __launch_bounds__(256) k_image32_lines(ImageArgs a) {
                         float *g = &T.g[i][pr].x + odd, *x = &T.x[i][pr].x + odd;
                         g[0] = a.lf[i].rat * gz;
                         g[2] = a.lf[i].dnl * pz - a.lf[i].rat * gy;
-                        x[0] = ((1.0f - wt) * p0.x + wt * p1.x) * kUnit;
-                        x[2] = ((1.0f - wt) * p0.y + wt * p1.y) * kUnit;
+                        x[0] = (1.0f - wt) * p0.x + wt * p1.x;
+                        x[2] = (1.0f - wt) * p0.y + wt * p1.y;
                     }
                 } else {
 #pragma unroll

@@ -57,7 +57,7 @@ __global__ void k_line_data(int64_t n, int L, int nlev, const double *__restrict
     line[2 * t] = eta;
     line[2 * t + 1] = chi;
     if (chi < 0.0) atomicAdd(neg, 1ull);
-    note_source(least, l, eta, chi);
+    if (least) note_source(least, l, eta, chi);
     if (linef) {
         linef[2 * t] = (float)eta;
         linef[2 * t + 1] = (float)chi;
@@ -471,9 +471,10 @@ struct ImageArgs {
     double *xy;               // [n][2]
     const float *dsf, *vparf, *bf, *linef;   // FP32 copies for the FP32 kernel
     float nf[3];
+    float chi_min32, dtau_min32;   // floors of the FP32 kernel, the opacity's in its units
     struct {                  // the first lines within reach, for the line kernels (image.cuh)
         int32_t l2;
-        float rat, dnl, nrm;  // nrm = c/(nu sqrt pi)
+        float rat, dnl, nrm;  // nrm = c/(nu sqrt pi) in the FP32 kernel's units
         int32_t cm, ic;       // exponents of chi_min nu/2^28 and of the boundary intensity, rounded down
     } lf[4];
 };
@@ -605,6 +606,16 @@ int mg_launch_max_rel_change(mg_ctx *ctx, int64_t m, const double *a_new, const 
     return MG_OK;
 }
 
+// The least sources of line data that were computed without them (mixed contexts, whose FP32
+// kernels need none).
+static int launch_least(mg_ctx *ctx) {
+    const int64_t m = ctx->n * ctx->n_lines;
+    MG_CUDA(cudaMemsetAsync(ctx->d_least, 0, sizeof(int32_t) * ctx->n_lines, ctx->stream));
+    k_least_source<<<(unsigned)((m + 255) / 256), 256, 0, ctx->stream>>>(ctx->n, ctx->n_lines, ctx->d_line, ctx->d_least);
+    MG_CUDA(cudaGetLastError());
+    return MG_OK;
+}
+
 int mg_launch_line_data(mg_ctx *ctx) {
     if (ctx->opt.precision == MG_MIXED) return mg_launch_line_data_mixed(ctx);
     MgTimed t(ctx, "line_data");
@@ -624,10 +635,6 @@ __global__ void k_mark_thick(int64_t n, int L, const double *Lw, double lmin, in
 
 static int launch_fp64(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount, unsigned grid);
 
-int mg_launch_feautrier_fp64_list(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount) {
-    return launch_fp64(ctx, olist, ocount, (unsigned)ctx->n);
-}
-
 int mg_launch_feautrier(mg_ctx *ctx) {
     if (ctx->opt.precision == MG_MIXED) {
         int rc = mg_launch_feautrier_mixed(ctx);
@@ -637,10 +644,8 @@ int mg_launch_feautrier(mg_ctx *ctx) {
         MG_CUDA(cudaMemsetAsync(ctx->d_promo + ctx->n, 0, sizeof(int32_t), ctx->stream));
         k_mark_thick<<<(unsigned)((ctx->n + 255) / 256), 256, 0, ctx->stream>>>(
             ctx->n, ctx->n_lines, ctx->d_L, 1.0 - 1.0 / ctx->opt.tau_fp64, ctx->d_promo, ctx->d_promo + ctx->n);
-        const int64_t m = ctx->n * ctx->n_lines;
-        MG_CUDA(cudaMemsetAsync(ctx->d_least, 0, sizeof(int32_t) * ctx->n_lines, ctx->stream));
-        k_least_source<<<(unsigned)((m + 255) / 256), 256, 0, ctx->stream>>>(ctx->n, ctx->n_lines, ctx->d_line, ctx->d_least);
         MG_CUDA(cudaGetLastError());
+        if ((rc = launch_least(ctx))) return rc;
         return launch_fp64(ctx, ctx->d_promo, ctx->d_promo + ctx->n, (unsigned)ctx->n);
     }
     return launch_fp64(ctx, nullptr, nullptr, (unsigned)ctx->n);
@@ -802,9 +807,10 @@ static int launch_fp64(mg_ctx *ctx, const int32_t *olist, const int32_t *ocount,
 // populations, for the images in either precision.
 int mg_launch_line_data64(mg_ctx *ctx, float *linef, unsigned long long *neg) {
     const int64_t m = ctx->n * ctx->n_lines;
-    MG_CUDA(cudaMemsetAsync(ctx->d_least, 0, sizeof(int32_t) * ctx->n_lines, ctx->stream));
+    int32_t *least = ctx->opt.precision == MG_FP64 ? ctx->d_least : nullptr;
+    if (least) MG_CUDA(cudaMemsetAsync(least, 0, sizeof(int32_t) * ctx->n_lines, ctx->stream));
     k_line_data<<<(unsigned)((m + 255) / 256), 256, 0, ctx->stream>>>(
-        ctx->n, ctx->n_lines, ctx->n_lev, ctx->d_pops, ctx->d_lines, ctx->d_line, linef, neg, ctx->d_least);
+        ctx->n, ctx->n_lines, ctx->n_lev, ctx->d_pops, ctx->d_lines, ctx->d_line, linef, neg, least);
     MG_CUDA(cudaGetLastError());
     return MG_OK;
 }
@@ -850,13 +856,15 @@ int mg_launch_image(mg_ctx *ctx, int ray, int line, int n_ch, const double *d_u,
     a.dsf = ctx->d_dsf; a.vparf = ctx->d_vparf; a.bf = ctx->d_bf; a.linef = ctx->d_imglf;
     const size_t smem32 = sizeof(float) * (size_t)s.kmax * (3 + 2 * (size_t)n_ov);
     for (int i = 0; i < 3; i++) a.nf[i] = (float)n[i];
+    a.chi_min32 = std::max((float)(s.chi_min * kImgUnit), 1.17549435e-38f);
+    a.dtau_min32 = (float)s.dtau_min;
     for (int i = 0; i < std::min(n_ov, kImgLines); i++) {
         const Overlap &v = h_ov[i];
         const double nu = 1.0 / v.inv_nu2;
         a.lf[i].l2 = v.l2;
         a.lf[i].rat = (float)v.rat;
         a.lf[i].dnl = (float)v.dnl;
-        a.lf[i].nrm = (float)v.inv_nu2 * (float)(kC / kSqrtPi);
+        a.lf[i].nrm = (float)v.inv_nu2 * (float)(kC / kSqrtPi) * kImgUnit;
         a.lf[i].cm = std::ilogb(s.chi_min) + std::ilogb(nu) - 28 - 1;
         a.lf[i].ic = std::max(std::ilogb(2.0 * kH * nu * nu * nu / (kC * kC) / std::expm1(kH * nu / (kKB * s.T_cmb))),
                               kDarkExp);
@@ -876,6 +884,10 @@ int mg_launch_image(mg_ctx *ctx, int ray, int line, int n_ch, const double *d_u,
     } else if (smem > 227 * 1024) {
         return mg_fail(ctx, MG_ERR_CAPACITY, "mg_image: longest ray pair does not fit in shared memory");
     } else if (n_ov <= kImgLines) {
+        if (ctx->opt.precision == MG_MIXED) {
+            int rc = launch_least(ctx);
+            if (rc) return rc;
+        }
         void (*kern)(ImageArgs, int, int) = n_ov == 1 ? k_image64_lines<1> : n_ov == 2 ? k_image64_lines<2>
                                           : n_ov == 3 ? k_image64_lines<3> : k_image64_lines<4>;
         auto bytes = [&](int cap) {
