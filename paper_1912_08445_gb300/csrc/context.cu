@@ -643,8 +643,10 @@ static int ensure_state(mg_ctx *ctx) {
             (rc = mg_alloc(ctx, &ctx->d_line, n * L * 2)) || (rc = mg_alloc(ctx, &ctx->d_linef, n * L * 2)) ||
             (rc = mg_alloc(ctx, &ctx->d_J, n * L)) || (rc = mg_alloc(ctx, &ctx->d_L, n * L)) ||
             (rc = mg_alloc(ctx, &ctx->d_Jeff, n * L)) || (rc = mg_alloc(ctx, &ctx->d_Lc, n * L)) ||
-            (rc = mg_alloc(ctx, &ctx->d_least, L)))
+            (rc = mg_alloc(ctx, &ctx->d_least, L))) {
+            mg_free(ctx->d_pops);   // (says that the others are there)
             return rc;
+        }
     }
     if (ctx->opt.spectrum && !ctx->d_Jnu && ctx->have_quad)
         if ((rc = mg_alloc(ctx, &ctx->d_Jnu, n * L * ctx->Q))) return rc;
